@@ -154,23 +154,34 @@ __global__ void mip_kernel(const long long *psums, const uint2 *prec, int Np, in
 }
 
 // Occupancy bits of one level: a texel is occupied when its colour is not
-// zero.  The renderer walks only the occupied texels of a footprint row.
-__global__ void occupancy_kernel(const uint2 *rec, int NL, unsigned *mask) {
-  long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  int wpr = (NL + 31) / 32;
-  long long nw = 6LL * NL * wpr;
-  if (t >= nw) return;
-  long long row = t / wpr;  // face * NL + j
-  int w = (int)(t % wpr);
-  const uint2 *r = rec + row * NL;
-  unsigned bits = 0;
-  for (int b = 0; b < 32; ++b) {
-    int i = 32 * w + b;
-    if (i >= NL) break;
-    uint2 v = r[i];
-    if ((v.x | (v.y & 0xffffu)) != 0u) bits |= 1u << b;
+// zero.  The renderer takes only the occupied texels of a footprint.  One warp
+// per block; a ballot gives the bits of 8 columns x 4 rows (lane = 8 row +
+// column, reversed into bit 31 - lane), two of them side by side a block.
+__global__ void occupancy_kernel(const uint2 *rec, int NL, uint2 *mask) {
+  const long long blk = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5;
+  const int lane = threadIdx.x & 31, nbx = max(NL >> 3, 1), nby = max(NL >> 2, 1);
+  if (blk >= 6LL * nbx * nby) return;  // whole warps leave together
+  const int bx = (int)(blk % nbx), by = (int)((blk / nbx) % nby), face = (int)(blk / ((long long)nbx * nby));
+  const int j = by * 4 + (lane >> 3), i = bx * 8 + (lane & 7);
+  auto occupied = [&](const int ii) {
+    if (ii >= NL || j >= NL) return false;
+    const uint2 v = rec[((long long)face * NL + j) * NL + ii];
+    return (v.x | (v.y & 0xffffu)) != 0u;
+  };
+  const unsigned a = __brev(__ballot_sync(0xffffffffu, occupied(i)));
+  const unsigned b = __brev(__ballot_sync(0xffffffffu, occupied(i + 8)));
+  // bytes of a and b are rows (row 0 on top): interleave them
+  if (lane == 0) mask[blk] = make_uint2(__byte_perm(a, b, 0x3726u), __byte_perm(a, b, 0x1504u));
+}
+
+// The occupancy mask of every level from the records.
+void occupancy_launch(bh_ctx *ctx, const bh_cubemap *c, cudaStream_t s) {
+  for (int L = 0; L < c->levels; ++L) {
+    const long long blocks = mask_level_offset(c->n, L + 1) - mask_level_offset(c->n, L);
+    occupancy_kernel<<<(unsigned)((blocks + 7) / 8), 256, 0, s>>>(c->rec + cube_level_offset(c->n, L), c->n >> L,
+                                                                 c->mask + mask_level_offset(c->n, L));
+    count_launch(ctx);
   }
-  mask[t] = bits;
 }
 
 }  // namespace bh
@@ -210,9 +221,9 @@ extern "C" bh_status bh_build_star_cubemap(bh_ctx *ctx, const bh_star *stars, lo
   long long *sums0 = nullptr, *sums1 = nullptr;
   double *cmf = nullptr;
   bh_star *dstars = nullptr;
-  c->mask_words = mask_level_offset(N, c->levels);
+  const size_t mask_bytes = sizeof(uint2) * mask_level_offset(N, c->levels);
   cudaError_t e = cudaMalloc((void **)&c->rec, sizeof(uint2) * c->records);
-  if (e == cudaSuccess) e = cudaMalloc((void **)&c->mask, sizeof(unsigned) * c->mask_words);
+  if (e == cudaSuccess) e = cudaMalloc((void **)&c->mask, mask_bytes);
   if (e == cudaSuccess) e = cudaMallocAsync((void **)&acc, sizeof(unsigned long long) * 5 * nt0, s);
   if (e == cudaSuccess) e = cudaMallocAsync((void **)&sums0, sizeof(long long) * 3 * nt0, s);
   if (e == cudaSuccess) e = cudaMallocAsync((void **)&sums1, sizeof(long long) * 3 * nt1, s);
@@ -241,13 +252,7 @@ extern "C" bh_status bh_build_star_cubemap(bh_ctx *ctx, const bh_star *stars, lo
       ps = cs;
       cs = tmp;
     }
-    for (int L = 0; L < c->levels; ++L) {
-      int NL = N >> L;
-      long long nw = 6LL * NL * ((NL + 31) / 32);
-      occupancy_kernel<<<(unsigned)((nw + 255) / 256), 256, 0, s>>>(c->rec + cube_level_offset(N, L), NL,
-                                                                   c->mask + mask_level_offset(N, L));
-      count_launch(ctx);
-    }
+    occupancy_launch(ctx, c, s);
     e = cudaGetLastError();
   }
   cudaFreeAsync(acc, s);
@@ -285,9 +290,9 @@ bh_status cubemap_alloc_public(bh_ctx *ctx, int N, bh_dtype storage, bh_cubemap 
   c->levels = cube_levels(N);
   c->storage = storage;
   c->records = bh_cubemap_records(N);
-  c->mask_words = mask_level_offset(N, c->levels);
+  const size_t mask_bytes = sizeof(uint2) * mask_level_offset(N, c->levels);
   cudaError_t e = cudaMalloc((void **)&c->rec, sizeof(uint2) * c->records);
-  if (e == cudaSuccess) e = cudaMalloc((void **)&c->mask, sizeof(unsigned) * c->mask_words);
+  if (e == cudaSuccess) e = cudaMalloc((void **)&c->mask, mask_bytes);
   if (e != cudaSuccess) {
     cudaFree(c->rec);
     cudaFree(c->mask);

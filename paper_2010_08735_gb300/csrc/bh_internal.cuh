@@ -160,8 +160,7 @@ struct bh_cubemap {
   bh_dtype storage = BH_F16;
   uint2 *rec = nullptr;  // all levels
   long long records = 0;
-  unsigned *mask = nullptr;  // occupancy bits: one per texel, rows padded to 32-bit words
-  long long mask_words = 0;
+  uint2 *mask = nullptr;     // occupancy bits by blocks of texels (mask_level_offset)
 };
 
 namespace bh {
@@ -170,13 +169,18 @@ inline long long cube_level_offset(int N, int L) {
   for (int l = 0; l < L; ++l) off += 6LL * (N >> l) * (N >> l);
   return off;
 }
-// Occupancy mask layout: level-major, face, row; a row of n texels takes
-// (n + 31) / 32 words, bit (i & 31) of word i / 32 is texel i.
+// Occupancy mask layout: level-major, face, then blocks of 16 columns x 4
+// rows in row-major order, one every 8 columns and 4 rows (each texel is in
+// two blocks; at least one block; texels past the face are 0).  Row r of a
+// block is 16 bits, the first column in the top bit: rows 0 and 1 in x (row 0
+// on top), rows 2 and 3 in y.  Any 8 columns x 8 rows of a face lie in one
+// block column and at most three of its blocks, so a footprint's occupancy is
+// one to three loads instead of one or two per texel row.
 inline long long mask_level_offset(int N, int L) {
   long long off = 0;
   for (int l = 0; l < L; ++l) {
-    long long n = N >> l;
-    off += 6LL * n * ((n + 31) / 32);
+    const long long n = N >> l;
+    off += 6 * (n >= 8 ? n / 8 : 1) * (n >= 4 ? n / 4 : 1);
   }
   return off;
 }
@@ -188,4 +192,5 @@ inline int cube_levels(int N) {
 void count_launch(bh_ctx *ctx, int n = 1);
 bh_status check_status(bh_ctx *ctx, cudaStream_t s);
 bh_status colour_tables_launch(bh_ctx *ctx, bh_tables *t, cudaStream_t s);
+void occupancy_launch(bh_ctx *ctx, const bh_cubemap *c, cudaStream_t s);
 }  // namespace bh

@@ -102,6 +102,35 @@ struct Reader {
   }
 };
 
+// Occupancy in a cube-map file: level-major, face, row; a row of n texels
+// takes (n + 31) / 32 words, bit (i & 31) of word i / 32 is texel i.
+long long file_mask_words(int N) {
+  long long words = 0;
+  for (int l = 0; l < cube_levels(N); ++l) {
+    const long long n = N >> l;
+    words += 6LL * n * ((n + 31) / 32);
+  }
+  return words;
+}
+
+// The file's occupancy words of a map's records (colour not zero).
+std::vector<unsigned> file_mask(const std::vector<uint2> &rec, int N) {
+  std::vector<unsigned> mask;
+  mask.reserve((size_t)file_mask_words(N));
+  const uint2 *r = rec.data();
+  for (int l = 0; l < cube_levels(N); ++l) {
+    const int n = N >> l;
+    for (long long row = 0; row < 6LL * n; ++row, r += n)
+      for (int i = 0; i < n; i += 32) {
+        unsigned bits = 0;
+        for (int b = 0; b < 32 && i + b < n; ++b)
+          if (r[i + b].x | (r[i + b].y & 0xffffu)) bits |= 1u << b;
+        mask.push_back(bits);
+      }
+  }
+  return mask;
+}
+
 template <typename T>
 bh_status copy_out(std::vector<T> &v, const void *dev, size_t n) {
   v.resize(n);
@@ -210,14 +239,13 @@ extern "C" bh_status bh_cubemap_save(const bh_cubemap *c, const char *path) {
   BH_CUDA(cudaSetDevice(c->ctx->device));
   BH_CUDA(cudaDeviceSynchronize());
   std::vector<uint2> rec;
-  std::vector<unsigned> mask;
   bh_status st;
-  if ((st = copy_out(rec, c->rec, (size_t)c->records)) || (st = copy_out(mask, c->mask, (size_t)c->mask_words)))
-    return st;
+  if ((st = copy_out(rec, c->rec, (size_t)c->records))) return st;
+  const std::vector<unsigned> mask = file_mask(rec, c->n);
   Writer w(path);
   const uint32_t hdr[8] = {kFormatVersion, (uint32_t)c->n, (uint32_t)c->levels, (uint32_t)c->storage,
                            (uint32_t)(c->records & 0xffffffffu), (uint32_t)(c->records >> 32),
-                           (uint32_t)(c->mask_words & 0xffffffffu), (uint32_t)(c->mask_words >> 32)};
+                           (uint32_t)(mask.size() & 0xffffffffu), (uint32_t)((unsigned long long)mask.size() >> 32)};
   w.put(kCubeMagic, 8);
   w.put(hdr, sizeof hdr);
   w.put(rec.data(), rec.size() * sizeof(uint2));
@@ -245,7 +273,7 @@ extern "C" bh_status bh_cubemap_load(bh_ctx *ctx, const char *path, void *stream
   const long long words = (long long)hdr[6] | ((long long)hdr[7] << 32);
   if (hdr[0] != kFormatVersion || N < 1 || N > 8192 || (N & (N - 1)) || (int)hdr[2] != cube_levels(N) ||
       (storage != BH_F16 && storage != BH_BF16) || records != cube_level_offset(N, cube_levels(N)) ||
-      words != mask_level_offset(N, cube_levels(N))) {
+      words != file_mask_words(N)) {
     set_error("bh_cubemap_load: %s has an unknown format or inconsistent sizes", path);
     return BH_ERR_INVALID_ARG;
   }
@@ -261,7 +289,10 @@ extern "C" bh_status bh_cubemap_load(bh_ctx *ctx, const char *path, void *stream
   bh_status st = cubemap_alloc_public(ctx, N, storage, &c);
   if (st) return st;
   cudaError_t e = cudaMemcpyAsync(c->rec, rec, (size_t)records * sizeof(uint2), cudaMemcpyHostToDevice, s);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(c->mask, mask, (size_t)words * sizeof(unsigned), cudaMemcpyHostToDevice, s);
+  if (e == cudaSuccess) {
+    occupancy_launch(ctx, c, s);  // the renderer's layout, from the records
+    e = cudaGetLastError();
+  }
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) {
     bh_cubemap_free(c);

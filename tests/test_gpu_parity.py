@@ -402,6 +402,54 @@ def test_render_configs_small(ctx, orc, gpu_tables, static_scene, cam):
     check_rgb(og, oo, od, mask, cam, "small")
 
 
+@pytest.mark.parametrize("face,n,dtype", [(1, 50, 1), (2, 50, 2), (4, 200, 1), (8, 300, 2), (16, 40, 1),
+                                          (32, 60_000, 1), (64, 3_000, 2), (256, 400_000, 1), (512, 20_000, 2)])
+def test_render_star_windows(ctx, orc, orc_tables, orc_colour, gpu_tables, face, n, dtype):
+    """Star gathers over occupancy windows: faces smaller than a block, window
+    edges, sparse fields and dense ones (whose windows are culled to the
+    footprint), seen at footprints from under one texel to the coarsest level."""
+    st = synth.stars(n, 11)
+    cube = bh.bh_build_star_cubemap(ctx, st, face, dtype)
+    try:
+        scene = orc_scene(orc, orc_tables, orc_colour, orc.build_cubemap(st, face, dtype), face, dtype)
+        for cam in (synth.camera(6.0, 85.0, v=(0.0, 0.0, 0.5), width=72, height=48),
+                    synth.camera(20.0, 50.0, phi_deg=200.0, v=(0.3, 0.2, 0.0), width=45, height=61, fov_deg=100.0),
+                    synth.camera(9.0, 75.0, phi_deg=70.0, width=64, height=64, fov_deg=3.0)):
+            og, gd, oo, od, mask = compare_render(orc, ctx, gpu_tables, cube, scene, cam, synth.disc(),
+                                                  name=f"windows_{face}")
+            has = ~mask & (od[..., 6] >= 0)
+            assert (gd[..., 6][has] != od[..., 6][has]).mean() <= 1e-3 if has.any() else True
+            ill = star_ill_conditioned(od, oo, cam)
+            mean, mx, rel = image_error(og, oo, mask | ill)
+            assert mean <= RGB_MEAN_REL and mx <= RGB_MAX_REL, (face, cam["r"], mean, mx)
+            assert ill_conditioned_ok(rel, od, oo, cam, mask)
+            timed, _ = gpu_render(ctx, gpu_tables, cube, cam, synth.disc(), debug=False)
+            assert np.array_equal(timed, og)
+    finally:
+        bh.bh_cubemap_free(cube)
+
+
+@pytest.mark.parametrize("face", [1, 4, 64, 256])
+def test_cubemap_file_keeps_its_layout(ctx, tmp_path, face):
+    """A saved map holds its records and, per level, face and row, the bits of
+    its occupied texels in words of 32, whatever layout the renderer reads."""
+    cube = bh.bh_build_star_cubemap(ctx, synth.stars(500, 3), face, 1)
+    path = tmp_path / "cube.bhc"
+    try:
+        bh.bh_cubemap_save(cube, path)
+        rec = bh.bh_cubemap_copy_out(cube, face)
+    finally:
+        bh.bh_cubemap_free(cube)
+    words, at, n = [], 0, face
+    while n:
+        on = (rec[at:at + 6 * n * n, :3] != 0).any(1).reshape(6 * n, n)
+        on = np.pad(on, ((0, 0), (0, -n % 32))).reshape(6 * n, -1, 32)
+        words.append((on.astype(np.uint64) << np.arange(32, dtype=np.uint64)).sum(2).astype(np.uint32).reshape(-1))
+        at, n = at + 6 * n * n, n // 2
+    body = path.read_bytes()[40:-8]
+    assert body == rec.tobytes() + np.concatenate(words).tobytes()
+
+
 def test_empty_star_field_equals_no_cube_map(ctx, gpu_tables):
     """A cube map built from no stars adds no light: the frame equals the one
     rendered without a cube map, bit for bit, in the timed and debug forms."""
