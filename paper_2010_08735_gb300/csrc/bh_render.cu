@@ -340,7 +340,7 @@ __global__ void __launch_bounds__(256, BH_RENDER_MIN_BLOCKS) render_kernel(const
     const float x0 = C.x[0], x1 = C.x[1], x2 = C.x[2];
     float c0 = fmaf(x1, d2, -x2 * d1), c1 = fmaf(x2, d0, -x0 * d2), c2 = fmaf(x0, d1, -x1 * d0);
     const float cn2 = fmaf(c0, c0, fmaf(c1, c1, c2 * c2));
-    const float icn = rsqrtf(fmaxf(cn2, 1e-38f));  // 1/|e_x' ^ d| (guarded for radial beams)
+    const float icn = rsqrtf(fmaxf(cn2, 1.2e-38f));  // 1/|e_x' ^ d| (guarded for radial beams)
     float cosd = fmaf(x0, d0, fmaf(x1, d1, x2 * d2));
     const float dd2 = fmaf(d0, d0, fmaf(d1, d1, d2 * d2));
     // delta itself is needed only for the debug channels: the disc hits use
