@@ -77,7 +77,7 @@ struct BatchGraph {
 
 struct RenderTuning {
   int warps_per_block = 8;   // block = warps * 32 threads
-  int fetch = 2;             // 8 x 4 pixel warp tiles a warp takes per fetch
+  int fetch = 4;             // 8 x 4 pixel warp tiles a warp takes per fetch (before the launch's tail)
   int blocks_per_sm = 4;     // persistent grid = SMs * blocks_per_sm
 };
 

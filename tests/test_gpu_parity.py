@@ -514,6 +514,20 @@ def test_batch_equals_single(ctx, gpu_tables, static_scene):
         assert torch.equal(single, o)
 
 
+@pytest.mark.parametrize("n", [1, 37, 300])
+def test_batch_of_small_cameras_equals_single(ctx, gpu_tables, static_scene, n):
+    """Launches in which a warp's next tile lies several cameras further on."""
+    cube, _ = static_scene
+    cams = synth.batch_cameras(n, seed=9, resolutions=((1, 1), (9, 5), (8, 4), (33, 17), (120, 90)))
+    sh = bh.make_shading(1.0, EXPOSURE_STARS)
+    outs = [torch.zeros((c["height"], c["width"], 4), device="cuda") for c in cams]
+    bh.bh_render_batch(ctx, gpu_tables, cube, cams, synth.disc(), sh, outs)
+    for c, o in zip(cams, outs):
+        one = torch.zeros_like(o)
+        bh.bh_render(ctx, gpu_tables, cube, c, synth.disc(), sh, one)
+        assert torch.equal(o, one)
+
+
 def test_autotune_every_candidate_same_image(gpu_tables, static_scene):
     """The autotuner launches every candidate launch shape; the image does not
     depend on the shape, and batched renders stay equal to single ones."""
