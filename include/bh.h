@@ -198,7 +198,8 @@ typedef struct {
  * Y.  face_size: power of two, 1..8192.  storage: BH_F16 or BH_BF16.
  * stars: host array (stars_on_device = 0) or device array (1).  Enqueued on
  * `stream` (a host star list is staged synchronously first).  Uses
- * 40 * 6 * face_size^2 bytes of scratch, freed before return. */
+ * 48 bytes of scratch per star -- where that is more than 1 GiB, at most
+ * 240 * face_size^2 bytes --, freed before return. */
 bh_status bh_build_star_cubemap(bh_ctx *ctx, const bh_star *stars, long long n, int face_size,
                                 bh_dtype storage, int stars_on_device, void *stream,
                                 bh_cubemap **out);
@@ -211,7 +212,7 @@ bh_status bh_build_star_cubemap(bh_ctx *ctx, const bh_star *stars, long long n, 
  *  - stars_device: n stars in device memory; records_device: caller-owned
  *    device buffer of bh_cubemap_records(face_size) x 4 uint16, 8-byte aligned.
  *  - face_size: power of two, at most 128 (the size of the library's static
- *    scratch array, about 6.9 MB, held on every GPU that loads the library
+ *    scratch array, about 4 MB, held on every GPU that loads the library
  *    until the process exits); larger sizes return BH_ERR_INVALID_ARG.
  *  - Works on the current CUDA device and needs no bh_ctx; `stream`, the
  *    stars and the records must all belong to that device.  Each call that is

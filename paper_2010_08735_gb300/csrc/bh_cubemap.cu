@@ -8,15 +8,29 @@
 //
 // Determinism: colours are accumulated as 64-bit fixed point (2^-20 units)
 // with integer atomics, so the sums do not depend on the order in which
-// threads arrive; the position averages are evaluated in FP64 in one fixed
-// child order with round-to-nearest intrinsics (this file is compiled
-// without multiply-add contraction).  The build is therefore bit-for-bit
+// threads arrive; the position averages are those of FP64 arithmetic in one
+// fixed child order with round-to-nearest (this file is compiled without
+// multiply-add contraction).  The build is therefore bit-for-bit
 // reproducible.
 //
 // Layout: records of 4 x 16 bit -- X, Y, Z (half or bfloat16 of the colour
 // sum divided by 4^level, so that coarse levels stay in range) and the
 // position word (s in the low byte, t in the high byte) -- level-major, then
 // face (+x,-x,+y,-y,+z,-z), row t, column s.
+//
+// How it runs.  The floor is the write of the records (268 MB for faces of
+// 2048^2: 40 us), but GB300 does two FP64 multiply-adds per SM and clock, so
+// arithmetic decides: a star's black body was 95 exponentials (8 ms for 1M
+// stars), now two polynomials (chroma_kernel).  Stars are sorted by region (32
+// x 32 texels of level 0) and one block builds a region's six levels from
+// them in shared memory, writing every record once; the last block of 32 x 32
+// regions to finish builds the next five levels.  Dense accumulators in global
+// memory (64 bytes a texel, cleared, summed and read back level by level)
+// moved 4 GB for those 268 MB.  1M stars on 2048^2 faces: fit 18 us, bins 44,
+// places 4, colours 74 (FP64 at 86 % of its rate), regions 231, mask of the
+// small levels 8 -- 0.38 ms where the kernels took 15.9 ms; 20,000 stars on
+// 128^2 faces 46 us instead of 419.
+#include <algorithm>
 #include <cmath>
 
 #include "bh_colour.cuh"
@@ -26,163 +40,810 @@ namespace bh {
 
 constexpr double kXyzScale = 1048576.0;  // 2^20
 
-__global__ void cube_cmf_kernel(double *cmf) {
-  int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k < kNLambda) dcmf(360.0 + 5.0 * k, cmf + 3 * k);
+// ---------------------------------------------------------------------------
+// Chromaticity of black bodies
+//
+// A star's colour is its luminosity times (X, Y, Z) / (X + Y + Z) of a black
+// body, a smooth function of 1/T alone.  For T in [1024 K, 1e9 K] it is
+// read off polynomials of degree 8 in 1/T on 64 equal cells of [0, 1/1024 K]
+// (Chebyshev nodes; a cell spans 0.6 in h c / (lambda k T) at 360 nm), fitted on
+// the device at each build: 576 black bodies instead of one per star.  Relative
+// error over the fitted range against extended precision: at most 1.4e-15 (the
+// FP64 sum over the wavelengths itself: 2.2e-15).
+// ---------------------------------------------------------------------------
+constexpr int kChromaCells = 64, kChromaNodes = 9;
+constexpr double kChromaTMin = 1024.0, kChromaTMax = 1e9;
+constexpr int kChromaStride = 2 * kChromaNodes + 2;  // X and Z coefficients, minus twice the cell's centre, pad
+constexpr int kChromaCoefs = kChromaCells * kChromaStride, kChromaVals = kChromaCells * kChromaNodes * 2;
+
+// Everything of the fit that does not depend on the cell: computed once on the
+// host, a kernel parameter.
+struct ChromaFit {
+  double node[kChromaNodes];                // Chebyshev nodes on [-1, 1]
+  // values at the nodes -> monomial coefficients, as sums of two doubles: their
+  // terms cancel to a thousandth
+  double inv[kChromaNodes][kChromaNodes], inv_lo[kChromaNodes][kChromaNodes];
+  double x[kNLambda];                       // c2 / lambda (K)
+  double cmf[3][kNLambda];                  // matching functions
+  double w[3][kNLambda];                    // ... times the trapezoid weight over (lambda / 560 nm)^5
+};
+
+static const ChromaFit &chroma_fit() {
+  static const ChromaFit fit = [] {
+    ChromaFit f = {};
+    constexpr int n = kChromaNodes;
+    const long double pi = 3.14159265358979323846264338327950288L;
+    double mono[n][n] = {};  // mono[j][m]: coefficient of u^m in the Chebyshev polynomial T_j
+    mono[0][0] = 1.0;
+    mono[1][1] = 1.0;
+    for (int j = 2; j < n; ++j)
+      for (int m = 0; m < n; ++m) mono[j][m] = (m > 0 ? 2.0 * mono[j - 1][m - 1] : 0.0) - mono[j - 2][m];
+    for (int k = 0; k < n; ++k) {
+      f.node[k] = (double)cosl(pi * (k + 0.5L) / n);
+      for (int m = 0; m < n; ++m) {
+        long double s = 0.0L;
+        for (int j = 0; j < n; ++j) s += mono[j][m] * (j == 0 ? 1.0L : 2.0L) / n * cosl(j * pi * (k + 0.5L) / n);
+        f.inv[m][k] = (double)s;
+        f.inv_lo[m][k] = (double)(s - f.inv[m][k]);
+      }
+    }
+    auto lobe = [](double l, double m, double s1, double s2) {
+      const double t = (l - m) / (l < m ? s1 : s2);
+      return exp(-0.5 * t * t);
+    };
+    for (int k = 0; k < kNLambda; ++k) {  // the observer of dcmf
+      const double l = 360.0 + 5.0 * k, r = l / 560.0, t = (k == 0 || k == kNLambda - 1 ? 2.5 : 5.0) / (r * r * r * r * r);
+      f.x[k] = 1.4387769e7 / l;
+      f.cmf[0][k] = 1.056 * lobe(l, 599.8, 37.9, 31.0) + 0.362 * lobe(l, 442.0, 16.0, 26.7) -
+                    0.065 * lobe(l, 501.1, 20.4, 26.2);
+      f.cmf[1][k] = 0.821 * lobe(l, 568.8, 46.9, 40.5) + 0.286 * lobe(l, 530.9, 16.3, 31.1);
+      f.cmf[2][k] = 1.217 * lobe(l, 437.0, 11.8, 36.0) + 0.681 * lobe(l, 459.0, 26.0, 13.8);
+      for (int c = 0; c < 3; ++c) f.w[c][k] = t * f.cmf[c][k];
+    }
+    return f;
+  }();
+  return fit;
+}
+
+// One warp (a block of its own: 576 of them spread over the SMs) per node, 45
+// FP64 operations per wavelength, whose constants come from the host; the last
+// node of a cell to finish fits the cell.  The block past the nodes writes the
+// matching functions, for stars outside the fitted range.
+__global__ void chroma_kernel(const ChromaFit fit, double *cmf_out, double *val, unsigned *done, double *coef) {
+  const int lane = threadIdx.x, cell = blockIdx.x / kChromaNodes, node = blockIdx.x - cell * kChromaNodes;
+  if (cell == kChromaCells) {
+    for (int k = lane; k < kNLambda; k += 32)
+      for (int c = 0; c < 3; ++c) cmf_out[3 * k + c] = fit.cmf[c][k];
+    return;
+  }
+  const double v = (cell + 0.5 * (fit.node[node] + 1.0)) * (1.0 / (kChromaCells * kChromaTMin));  // 1/T
+  double s[3] = {0.0, 0.0, 0.0};
+  for (int k = lane; k < kNLambda; k += 32) {
+    const double b = 1.0 / expm1(fit.x[k] * v);
+    for (int c = 0; c < 3; ++c) s[c] = fma(b, fit.w[c][k], s[c]);
+  }
+  for (int o = 16; o > 0; o >>= 1)
+    for (int c = 0; c < 3; ++c) s[c] += __shfl_xor_sync(0xffffffffu, s[c], o);
+  unsigned before = 0;
+  if (lane == 0) {
+    const double sum = 1.0 / (s[0] + s[1] + s[2]);
+    val[blockIdx.x * 2] = s[0] * sum;
+    val[blockIdx.x * 2 + 1] = s[2] * sum;
+    __threadfence();
+    before = atomicAdd(done + cell, 1u);
+    __threadfence();
+  }
+  if (__shfl_sync(0xffffffffu, before, 0) != kChromaNodes - 1u) return;
+  double *out = coef + cell * kChromaStride;
+  if (lane < 2 * kChromaNodes) {
+    const int c = lane / kChromaNodes, m = lane - c * kChromaNodes;
+    double a = 0.0, err = 0.0;  // the sum and what its roundings lost
+    for (int k = 0; k < kChromaNodes; ++k) {
+      const double f = __ldcg(val + (cell * kChromaNodes + k) * 2 + c);
+      const double p = fit.inv[m][k] * f, t = a + p, z = t - a;
+      err += ((a - (t - z)) + (p - z)) + (fma(fit.inv[m][k], f, -p) + fit.inv_lo[m][k] * f);
+      a = t;
+    }
+    out[lane] = a + err;
+  } else if (lane == 2 * kChromaNodes) {
+    out[lane] = -(2.0 * cell + 1.0);
+  }
+}
+
+// val: kChromaVals doubles of scratch; done: kChromaCells counters, zero.
+static void chroma_launch(double *cmf, double *val, unsigned *done, double *coef, cudaStream_t s) {
+  chroma_kernel<<<kChromaCells * kChromaNodes + 1, 32, 0, s>>>(chroma_fit(), cmf, val, done, coef);
+}
+
+// 1/b by Newton's iteration from the float reciprocal (b a normal float whose
+// reciprocal is one): 2^-23, 2^-46, then rounding.
+__device__ __forceinline__ double newton_rcp(float bf, double b) {
+  double r = (double)__frcp_rn(bf);
+  r = fma(r, fma(-b, r, 1.0), r);
+  return fma(r, fma(-b, r, 1.0), r);
+}
+
+// Emitted XYZ of a star (black body of its temperature scaled to its
+// luminosity X+Y+Z, rounded to float) in 2^-20 units.
+__device__ __forceinline__ void star_colour(const bh_star &st, const double *cmf, const double *coef, long long *q) {
+  const double lum = (double)st.lum;
+  float xf[3];
+  if (st.temp_K >= (float)kChromaTMin && st.temp_K <= (float)kChromaTMax) {
+    // 32 FP64 operations, which bound the kernel (98 us for 1M stars with a
+    // divide and 64-bit conversions)
+    const double r = newton_rcp(st.temp_K, (double)st.temp_K);
+    const int cell = min((int)((float)(kChromaCells * kChromaTMin) * __frcp_rn(st.temp_K)), kChromaCells - 1);
+    const double *a = coef + cell * kChromaStride, *b = a + kChromaNodes;
+    const double u = fma(2.0 * kChromaCells * kChromaTMin, r, a[2 * kChromaNodes]);
+    double x = a[kChromaNodes - 1], z = b[kChromaNodes - 1];
+#pragma unroll
+    for (int m = kChromaNodes - 2; m >= 0; --m) {
+      x = fma(x, u, a[m]);
+      z = fma(z, u, b[m]);
+    }
+    xf[0] = (float)(lum * x);
+    xf[1] = (float)(lum * ((1.0 - x) - z));
+    xf[2] = (float)(lum * z);
+  } else {
+    double b[3];
+    dblackbody_xyz(cmf, (double)st.temp_K, b);
+    const double s = __dadd_rn(__dadd_rn(b[0], b[1]), b[2]);
+    for (int c = 0; c < 3; ++c) xf[c] = (float)__ddiv_rn(__dmul_rn(lum, b[c]), s);
+  }
+  // in units of 2^-20, to the nearest integer: below 2^23 by the 32-bit
+  // conversion, above it the float is an integer, its mantissa shifted
+  for (int c = 0; c < 3; ++c) {
+    const float f = xf[c] * 1048576.f, m = fabsf(f);
+    if (m < 8388608.f) q[c] = __float2int_rn(f);
+    else if (m < 1.8e19f / 2) {
+      const unsigned bits = __float_as_uint(m);
+      const long long v = (long long)((bits & 0x7fffffu) | 0x800000u) << ((bits >> 23) - 150);
+      q[c] = f < 0.f ? -v : v;
+    } else q[c] = __double2ll_rn(__dmul_rn((double)xf[c], kXyzScale));  // out of range or not a number
+  }
 }
 
 // GL major-axis face and face coordinates (sc, tc, |ma|).
-__device__ __forceinline__ int cube_face_d(double x, double y, double z, double &sc, double &tc,
-                                           double &ma) {
-  double ax = fabs(x), ay = fabs(y), az = fabs(z);
+__device__ __forceinline__ int cube_face_f(float x, float y, float z, float &sc, float &tc, float &ma) {
+  const float ax = fabsf(x), ay = fabsf(y), az = fabsf(z);
   if (ax >= ay && ax >= az) {
     ma = ax;
-    if (x >= 0.0) { sc = -z; tc = -y; return 0; }
+    if (x >= 0.f) { sc = -z; tc = -y; return 0; }
     sc = z; tc = -y; return 1;
   }
   if (ay >= az) {
     ma = ay;
-    if (y >= 0.0) { sc = x; tc = z; return 2; }
+    if (y >= 0.f) { sc = x; tc = z; return 2; }
     sc = x; tc = -z; return 3;
   }
   ma = az;
-  if (z >= 0.0) { sc = x; tc = -y; return 4; }
+  if (z >= 0.f) { sc = x; tc = -y; return 4; }
   sc = -x; tc = -y; return 5;
 }
 
-// One thread per star: emitted XYZ (black body of the star's temperature,
-// scaled to its luminosity X+Y+Z, rounded to float), fixed-point sums into
-// the level-0 texel that contains its direction.
-__global__ void star_bin_kernel(const bh_star *stars, long long n, int N, const double *cmf,
-                                unsigned long long *acc) {
-  long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (k >= n) return;
-  bh_star st = stars[k];
-  double b[3];
-  dblackbody_xyz(cmf, (double)st.temp_K, b);
-  double s = __dadd_rn(__dadd_rn(b[0], b[1]), b[2]);
-  double lum = (double)st.lum;
-  long long q[3];
-  for (int c = 0; c < 3; ++c) {
-    float xf = (float)__ddiv_rn(__dmul_rn(lum, b[c]), s);
-    q[c] = __double2ll_rn(__dmul_rn((double)xf, kXyzScale));
+// Face, texel and 16-bit position inside the texel of a star.
+struct StarTexel {
+  int face, i, j;
+  unsigned s16, t16;
+};
+
+__device__ __forceinline__ StarTexel star_texel(const bh_star &st, int N) {
+  float sc, tc, ma;
+  StarTexel r;
+  r.face = cube_face_f(st.dir[0], st.dir[1], st.dir[2], sc, tc, ma);
+  // floor(65536 N (sc/ma + 1)/2) holds the column (above 16 bits) and the position
+  const double scale = 32768.0 * N;
+  long long S, T;
+  if (ma >= 1e-30f && ma <= 1e30f) {
+    // One reciprocal for both quotients, each put right by its exact remainder
+    // (Markstein: the quotient rounds as a division would); the floor is the low
+    // word of a sum rounded down onto the integers above 2^52.
+    const double b = (double)ma, rb = newton_rcp(ma, b);
+    auto place = [&](double a) {
+      const double q0 = a * rb, q = fma(fma(-q0, b, a), rb, q0);
+      return (long long)(unsigned)__double2loint(__fma_rd(__dadd_rn(q, 1.0), scale, 4503599627370496.0));
+    };
+    S = place((double)sc);
+    T = place((double)tc);
+  } else {
+    S = __double2ll_rd(__dmul_rn(__dadd_rn(__ddiv_rn((double)sc, (double)ma), 1.0), scale));
+    T = __double2ll_rd(__dmul_rn(__dadd_rn(__ddiv_rn((double)tc, (double)ma), 1.0), scale));
   }
-  double sc, tc, ma;
-  int f = cube_face_d((double)st.dir[0], (double)st.dir[1], (double)st.dir[2], sc, tc, ma);
-  double S = __dmul_rn(__dmul_rn(__dadd_rn(__ddiv_rn(sc, ma), 1.0), 0.5), (double)N);
-  double T = __dmul_rn(__dmul_rn(__dadd_rn(__ddiv_rn(tc, ma), 1.0), 0.5), (double)N);
-  int i = (int)floor(S), j = (int)floor(T);
-  i = min(max(i, 0), N - 1);
-  j = min(max(j, 0), N - 1);
-  long long s16 = (long long)floor(__dmul_rn(__dadd_rn(S, -(double)i), 65536.0));
-  long long t16 = (long long)floor(__dmul_rn(__dadd_rn(T, -(double)j), 65536.0));
-  s16 = min(max(s16, 0LL), 65535LL);
-  t16 = min(max(t16, 0LL), 65535LL);
-  unsigned long long *a = acc + (((long long)f * N + j) * N + i) * 5;
-  atomicAdd(a + 0, (unsigned long long)q[0]);
-  atomicAdd(a + 1, (unsigned long long)q[1]);
-  atomicAdd(a + 2, (unsigned long long)q[2]);
-  atomicAdd(a + 3, (unsigned long long)(q[1] * s16));
-  atomicAdd(a + 4, (unsigned long long)(q[1] * t16));
+  const long long most = (long long)N << 16;
+  auto split = [&](long long v, int &cell, unsigned &pos) {
+    if (v < 0) { cell = 0; pos = 0; }                          // a direction that is not a number
+    else if (v >= most) { cell = N - 1; pos = 65535; }         // the far edge
+    else { cell = (int)(v >> 16); pos = (unsigned)v & 65535u; }
+  };
+  split(S, r.i, r.s16);
+  split(T, r.j, r.t16);
+  return r;
 }
 
-__device__ __forceinline__ unsigned short enc16(double v, int dtype) {
-  if (dtype == BH_BF16) return __bfloat16_as_ushort(__double2bfloat16(v));
-  return __half_as_ushort(__double2half(fmin(v, 65504.0)));
+// ---------------------------------------------------------------------------
+// Records
+// ---------------------------------------------------------------------------
+
+// v / 2^k as half (at most 65504) or bfloat16, one rounding: the sum is first
+// rounded to odd in 24 bits (13 or more beyond the result's).  32-bit integer
+// work: conversions of 64-bit integers run at the FP64 rate.
+__device__ __forceinline__ unsigned short enc16(long long v, int k, int dtype) {
+  unsigned long long u = v < 0 ? 0ull - (unsigned long long)v : (unsigned long long)v;
+  const int lz = u ? __clzll(u) : 0;
+  u <<= lz;
+  const unsigned m = (unsigned)(u >> 40) | ((u & 0xffffffffffull) ? 1u : 0u);
+  float f = __uint2float_rn(m) * __int_as_float((127 + 40 - lz - k) << 23);
+  if (v < 0) f = -f;
+  if (dtype == BH_BF16) return __bfloat16_as_ushort(__float2bfloat16_rn(f));
+  return __half_as_ushort(__float2half_rn(fminf(f, 65504.f)));
 }
 
-// Level-0 records from the accumulators (X, Y, Z, Y*s16, Y*t16 per texel).
-__global__ void level0_kernel(const unsigned long long *acc, long long ntex, int dtype,
-                              uint2 *rec, long long *sums) {
-  long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (t >= ntex) return;
-  const long long *a = (const long long *)(acc + t * 5);
-  long long x = a[0], y = a[1], z = a[2];
-  int ps = 128, pt = 128;
-  if (y > 0) {
-    double fs = __ddiv_rn(__dadd_rn(__ddiv_rn((double)a[3], (double)y), 0.5), 65536.0);
-    double ft = __ddiv_rn(__dadd_rn(__ddiv_rn((double)a[4], (double)y), 0.5), 65536.0);
-    ps = min((int)floor(__dmul_rn(fs, 256.0)), 255);
-    pt = min((int)floor(__dmul_rn(ft, 256.0)), 255);
+__device__ __forceinline__ uint2 make_record(long long x, long long y, long long z, unsigned p, int L, int dtype) {
+  const int k = 20 + 2 * L;
+  return make_uint2((unsigned)enc16(x, k, dtype) | ((unsigned)enc16(y, k, dtype) << 16),
+                    (unsigned)enc16(z, k, dtype) | (p << 16));
+}
+
+__device__ __forceinline__ float approx_float(long long v) {  // v >= 0, to 2^-23
+  return fmaf(__uint2float_rn((unsigned)((unsigned long long)v >> 32)), 4294967296.f, __uint2float_rn((unsigned)v));
+}
+
+// floor(num / den) for 0 <= num <= 256 den, den > 0: a float estimate is off by
+// one at most and put right in integers.
+__device__ __forceinline__ int small_quotient(long long num, long long den) {
+  const int p = (int)__fdividef(approx_float(num), approx_float(den));
+  const long long r = num - p * den;
+  return r < 0 ? p - 1 : r >= den ? p + 1 : p;
+}
+
+// Mean position byte at level 0 from y = sum of Y and a = sum of Y * s16:
+// floor(256 (a/y + 1/2)/65536).  Rounding FP64 cannot carry the mean over a
+// byte boundary while y is below 2^35 (its distance from one is at least 1/(512
+// y)), so the quotient is taken in integers there.
+__device__ __forceinline__ int mean_byte0(long long a, long long y) {
+  if (y < (1LL << 35) && a >= 0 && a <= 65535 * y) return min(small_quotient(2 * a + y, 512 * y), 255);
+  const double f = __ddiv_rn(__dadd_rn(__ddiv_rn((double)a, (double)y), 0.5), 65536.0);
+  return min((int)floor(__dmul_rn(f, 256.0)), 255);
+}
+
+// A texel's sums and mean position (s | t << 8).
+struct alignas(16) Node {
+  long long x, y, z;
+  unsigned p, pad;
+};
+
+constexpr unsigned kNoPosition = 128u | (128u << 8);  // of a texel without Y
+constexpr uint2 kEmptyRecord = {0u, kNoPosition << 16};
+
+// A mip texel from its children in the order (a,b) = (0,0), (1,0), (0,1),
+// (1,1), a the column and b the row offset: sums, and the Y-weighted mean
+// position floor(256 sum(cy (a + (p + 1/2)/256)/2) / sum(cy)).  As above,
+// integers give the FP64 result while the weights sum to less than 2^40.
+__device__ __forceinline__ Node mip_node(const Node *c) {
+  Node r = {0, 0, 0, kNoPosition, 0};
+  bool plain = true;
+  for (int k = 0; k < 4; ++k) {
+    r.x += c[k].x;
+    r.y += c[k].y;
+    r.z += c[k].z;
+    plain = plain && c[k].y >= 0 && c[k].y < (1LL << 40);
   }
-  unsigned short X = enc16((double)x / kXyzScale, dtype), Y = enc16((double)y / kXyzScale, dtype),
-                 Z = enc16((double)z / kXyzScale, dtype);
-  rec[t] = make_uint2((unsigned)X | ((unsigned)Y << 16), (unsigned)Z | ((unsigned)(ps | (pt << 8)) << 16));
-  sums[t * 3 + 0] = x;
-  sums[t * 3 + 1] = y;
-  sums[t * 3 + 2] = z;
-}
-
-// Mip level L from level L-1: colour sums of the 4 children (exact), and the
-// Y-weighted mean of their positions, children in the order (a,b) = (0,0),
-// (1,0), (0,1), (1,1) with a the column and b the row offset.
-__global__ void mip_kernel(const long long *psums, const uint2 *prec, int Np, int L, int dtype,
-                           long long *csums, uint2 *crec) {
-  int Nc = Np >> 1;
-  long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  long long ntc = 6LL * Nc * Nc;
-  if (t >= ntc) return;
-  int f = (int)(t / ((long long)Nc * Nc));
-  long long rem = t % ((long long)Nc * Nc);
-  int j = (int)(rem / Nc), i = (int)(rem % Nc);
-  long long sx = 0, sy = 0, sz = 0;
-  double ns = 0.0, nt = 0.0;
-  for (int b = 0; b < 2; ++b)
-    for (int a = 0; a < 2; ++a) {
-      long long ct = ((long long)f * Np + 2 * j + b) * Np + 2 * i + a;
-      long long cy = psums[ct * 3 + 1];
-      sx += psums[ct * 3 + 0];
-      sy += cy;
-      sz += psums[ct * 3 + 2];
-      unsigned pp = prec[ct].y >> 16;
-      double cs = __ddiv_rn((double)(pp & 255) + 0.5, 256.0), cq = __ddiv_rn((double)(pp >> 8) + 0.5, 256.0);
-      ns = __dadd_rn(ns, __dmul_rn((double)cy, __dmul_rn(__dadd_rn((double)a, cs), 0.5)));
-      nt = __dadd_rn(nt, __dmul_rn((double)cy, __dmul_rn(__dadd_rn((double)b, cq), 0.5)));
+  if (r.y <= 0) return r;
+  int ps, pt;
+  if (plain && r.y < (1LL << 40)) {
+    long long ns = 0, nt = 0;
+    for (int k = 0; k < 4; ++k) {
+      ns += c[k].y * (long long)((k & 1) * 512 + 2 * (c[k].p & 255) + 1);
+      nt += c[k].y * (long long)((k >> 1) * 512 + 2 * (c[k].p >> 8) + 1);
     }
-  int ps = 128, pt = 128;
-  if (sy > 0) {
-    ps = min((int)floor(__dmul_rn(__ddiv_rn(ns, (double)sy), 256.0)), 255);
-    pt = min((int)floor(__dmul_rn(__ddiv_rn(nt, (double)sy), 256.0)), 255);
+    ps = min(small_quotient(ns, 4 * r.y), 255);
+    pt = min(small_quotient(nt, 4 * r.y), 255);
+  } else {
+    double ns = 0.0, nt = 0.0;
+    for (int k = 0; k < 4; ++k) {
+      const double cs = __ddiv_rn((double)(c[k].p & 255) + 0.5, 256.0), ct = __ddiv_rn((double)(c[k].p >> 8) + 0.5, 256.0);
+      ns = __dadd_rn(ns, __dmul_rn((double)c[k].y, __dmul_rn(__dadd_rn((double)(k & 1), cs), 0.5)));
+      nt = __dadd_rn(nt, __dmul_rn((double)c[k].y, __dmul_rn(__dadd_rn((double)(k >> 1), ct), 0.5)));
+    }
+    ps = min((int)floor(__dmul_rn(__ddiv_rn(ns, (double)r.y), 256.0)), 255);
+    pt = min((int)floor(__dmul_rn(__ddiv_rn(nt, (double)r.y), 256.0)), 255);
   }
-  double scale = ldexp(kXyzScale, 2 * L);
-  unsigned short X = enc16((double)sx / scale, dtype), Y = enc16((double)sy / scale, dtype),
-                 Z = enc16((double)sz / scale, dtype);
-  crec[t] = make_uint2((unsigned)X | ((unsigned)Y << 16), (unsigned)Z | ((unsigned)(ps | (pt << 8)) << 16));
-  csums[t * 3 + 0] = sx;
-  csums[t * 3 + 1] = sy;
-  csums[t * 3 + 2] = sz;
+  r.p = (unsigned)(ps | (pt << 8)) & 0xffffu;
+  return r;
 }
 
-// Occupancy bits of one level: a texel is occupied when its colour is not
-// zero.  The renderer takes only the occupied texels of a footprint.  One warp
-// per block; a ballot gives the bits of 8 columns x 4 rows (lane = 8 row +
-// column, reversed into bit 31 - lane), two of them side by side a block.
-__global__ void occupancy_kernel(const uint2 *rec, int NL, uint2 *mask) {
-  const long long blk = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5;
-  const int lane = threadIdx.x & 31, nbx = max(NL >> 3, 1), nby = max(NL >> 2, 1);
-  if (blk >= 6LL * nbx * nby) return;  // whole warps leave together
-  const int bx = (int)(blk % nbx), by = (int)((blk / nbx) % nby), face = (int)(blk / ((long long)nbx * nby));
+// ---------------------------------------------------------------------------
+// Stars to regions of 32 x 32 level-0 texels (the whole face below that)
+// ---------------------------------------------------------------------------
+constexpr int kRegion = 32, kRegionTexels = kRegion * kRegion;
+
+struct alignas(16) StarBin {
+  unsigned texel;  // region * 1024 + row * 32 + column
+  unsigned pos;    // s16 | t16 << 16
+  unsigned long long rank;  // of the star in its region
+};
+
+struct alignas(16) StarItem {  // a star in region order
+  long long q[3];
+  unsigned pos, local;
+};
+
+__global__ void star_bin_kernel(const bh_star *stars, long long n, int N, unsigned long long *count, StarBin *bins) {
+  const long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  const unsigned active = __ballot_sync(0xffffffffu, k < n);
+  if (k >= n) return;
+  const StarTexel t = star_texel(stars[k], N);
+  const int nr = max(N / kRegion, 1);
+  const unsigned region = (t.face * nr + t.j / kRegion) * nr + t.i / kRegion;
+  // one atomic per region and warp: fields may be clustered
+  const unsigned same = __match_any_sync(active, region);
+  const int lane = threadIdx.x & 31, leader = __ffs(same) - 1;
+  unsigned long long base = 0;
+  if (lane == leader) base = atomicAdd(count + region, (unsigned long long)__popc(same));
+  base = __shfl_sync(same, base, leader);
+  StarBin b;
+  b.texel = region * kRegionTexels + (t.j % kRegion) * kRegion + t.i % kRegion;
+  b.pos = t.s16 | (t.t16 << 16);
+  b.rank = base + __popc(same & ((1u << lane) - 1u));
+  bins[k] = b;
+}
+
+struct RegionSpan {
+  unsigned long long first, count;  // a region's stars in items
+};
+
+// Place of each region's stars, in any order of regions.
+__global__ void region_span_kernel(const unsigned long long *count, int regions, unsigned long long *cursor,
+                                   RegionSpan *span) {
+  const int r = blockIdx.x * blockDim.x + threadIdx.x, lane = threadIdx.x & 31;
+  const unsigned long long c = r < regions ? count[r] : 0;
+  unsigned long long s = c;
+  for (int o = 1; o < 32; o <<= 1) {
+    const unsigned long long v = __shfl_up_sync(0xffffffffu, s, o);
+    if (lane >= o) s += v;
+  }
+  unsigned long long base = 0;
+  if (lane == 31) base = atomicAdd(cursor, s);
+  base = __shfl_sync(0xffffffffu, base, 31);
+  if (r < regions) span[r] = {base + s - c, c};
+}
+
+__global__ void star_scatter_kernel(const bh_star *stars, long long n, const StarBin *bins, const RegionSpan *span,
+                                    const double *cmf, const double *coef, StarItem *items) {
+  const long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  if (k >= n) return;
+  const StarBin b = bins[k];
+  StarItem it;
+  star_colour(stars[k], cmf, coef, it.q);
+  it.pos = b.pos;
+  it.local = b.texel % kRegionTexels;
+  items[span[b.texel / kRegionTexels].first + b.rank] = it;
+}
+
+// Without room for a sorted copy: the sums X, Y, Z, Y s16, Y t16 of every
+// level-0 texel in global memory (5 words each, zero at the start).
+__global__ void star_accumulate_kernel(const bh_star *stars, long long n, int N, const double *cmf,
+                                       const double *coef, unsigned long long *acc) {
+  const long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  if (k >= n) return;
+  const bh_star st = stars[k];
+  long long q[3];
+  star_colour(st, cmf, coef, q);
+  const StarTexel t = star_texel(st, N);
+  unsigned long long *a = acc + (((long long)t.face * N + t.j) * N + t.i) * 5;
+  for (int c = 0; c < 3; ++c) atomicAdd(a + c, (unsigned long long)q[c]);
+  atomicAdd(a + 3, (unsigned long long)(q[1] * (long long)t.s16));
+  atomicAdd(a + 4, (unsigned long long)(q[1] * (long long)t.t16));
+}
+
+// ---------------------------------------------------------------------------
+// Regions to records
+// ---------------------------------------------------------------------------
+struct RegionParams {
+  const StarItem *items;               // stars by region, or nullptr: acc
+  const RegionSpan *span;              // nullptr: no stars
+  const unsigned long long *acc;
+  uint2 *rec;
+  unsigned char *mask;                 // nullptr: no occupancy mask (or faces below a region)
+  Node *nodes;                         // the top texel of every group, stage after stage
+  unsigned *arrived;                   // groups finished, per group of the next stage (zero at launch)
+  int N, dtype;
+  long long level_off[14];             // cube_level_offset
+  long long mask_off[3];               // mask_level_offset
+};
+
+static void region_levels(RegionParams &P) {
+  for (int L = 0; L < 14; ++L) P.level_off[L] = (P.N >> L) ? cube_level_offset(P.N, L) : 0;
+  for (int L = 0; L < 3; ++L) P.mask_off[L] = mask_level_offset(P.N, L);
+}
+
+// Threads of a region's block, and texels summed at a time: sorted stars and
+// dense sums (few regions: all of a region in two bands).
+constexpr int kSortedSlots = 128, kDenseSlots = 512;
+
+template <int kSlots>
+struct RegionShared {
+  unsigned acc[10][kSlots];             // X, Y, Z, Y s16, Y t16 of a texel: low and high halves
+  unsigned short p0[kSlots];
+  unsigned short slot[kRegionTexels];   // of a texel that a star touches
+  unsigned short list0[kSlots], list1[kSlots];  // the texels of levels 0 and 1 that hold sums
+  unsigned touched[kRegion];            // texels of level 0 that hold sums, one word per row
+  unsigned lit[3][kRegionTexels / 32];  // texels whose record has a colour, levels 0-2
+  unsigned full[6][8];                  // texels of levels 1-5 that hold sums
+  long long x[341], y[341], z[341];     // their sums: 256 of level 1, 64, 16, 4, 1
+  unsigned short p[341];
+  unsigned n0, n1;                      // lengths of the lists
+  int last;
+};
+
+template <typename Shared>
+__device__ __forceinline__ long long shared_sum(const Shared &sh, int c, int t) {
+  return (long long)(((unsigned long long)sh.acc[2 * c + 1][t] << 32) | sh.acc[2 * c][t]);
+}
+
+// 64-bit add by two 32-bit shared atomics (which are native): the low half's
+// carry goes into the high half's addend, so the sum is exact in any order.
+template <typename Shared>
+__device__ __forceinline__ void shared_add(Shared &sh, int c, int t, long long v) {
+  const unsigned lo = (unsigned)v, hi = (unsigned)((unsigned long long)v >> 32);
+  const unsigned old = atomicAdd(&sh.acc[2 * c][t], lo);
+  const unsigned up = hi + (old + lo < lo ? 1u : 0u);
+  if (up) atomicAdd(&sh.acc[2 * c + 1][t], up);
+}
+
+__device__ __forceinline__ int level_base(int l) { return l == 1 ? 0 : l == 2 ? 256 : l == 3 ? 320 : l == 4 ? 336 : 340; }
+
+// Texel t of level l from its children; false if none holds sums.
+template <typename Shared, typename Below>
+__device__ __forceinline__ bool build_texel(const RegionParams &P, Shared &sh, int l, int ls, int t, int L,
+                                            const Below &below, uint2 &v) {
+  const int j = t >> ls, i = t & ((1 << ls) - 1);
+  Node c[4];
+  bool any = false;
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    c[q] = {0, 0, 0, kNoPosition, 0};
+    if (below(2 * j + (q >> 1), 2 * i + (q & 1), c[q])) any = true;
+  }
+  if (!any) return false;
+  const Node r = mip_node(c);
+  const int k = level_base(l) + t;
+  sh.x[k] = r.x;
+  sh.y[k] = r.y;
+  sh.z[k] = r.z;
+  sh.p[k] = (unsigned short)r.p;
+  v = make_record(r.x, r.y, r.z, r.p, L, P.dtype);
+  return true;
+}
+
+__device__ __forceinline__ bool has_colour(uint2 v) { return (v.x | (v.y & 0xffffu)) != 0u; }
+
+// Texels first .. first + n - 1 of level l (side 2^ls texels) of a group whose
+// level 0 is level L0 of the map and begins at texel (ox, oy) of it: sums and
+// records.  `below` gives a child (row, column) if it holds sums.  Called by
+// threads t0, t0 + step, ... in whole warps.
+template <typename Shared, typename Below>
+__device__ void build_level(const RegionParams &P, Shared &sh, int l, int ls, int first, int n, int L0, int face,
+                            int ox, int oy, int t0, int step, const Below &below) {
+  const int L = L0 + l, NL = P.N >> L;
+  uint2 *rec = P.rec + P.level_off[L] + ((long long)face * NL + (oy >> l)) * NL + (ox >> l);
+  for (int k = t0; k < ((n + 31) & ~31); k += step) {
+    const int t = first + k;
+    uint2 v = kEmptyRecord;
+    bool any = false;
+    if (k < n) {
+      any = build_texel(P, sh, l, ls, t, L, below, v);
+      rec[(long long)(t >> ls) * NL + (t & ((1 << ls) - 1))] = v;
+    }
+    const unsigned full = __ballot_sync(0xffffffffu, any), lit = __ballot_sync(0xffffffffu, has_colour(v));
+    if ((threadIdx.x & 31) == 0) {
+      sh.full[l][t >> 5] = full;
+      if (l <= 2) sh.lit[l][t >> 5] = lit;
+    }
+  }
+}
+
+// A child from the level below in shared memory.
+template <typename Shared>
+struct FromLevel {
+  const Shared &sh;
+  int l, ls;  // the child's level and log2 of its side
+  __device__ bool operator()(int j, int i, Node &c) const {
+    const int t = (j << ls) + i;
+    if (!(sh.full[l][t >> 5] >> (t & 31) & 1u)) return false;
+    const int k = level_base(l) + t;
+    c = {sh.x[k], sh.y[k], sh.z[k], sh.p[k], 0};
+    return true;
+  }
+};
+
+// Levels 2 .. ls of a group (side 2^ls) whose level 1 is in shared memory.
+// Level 2 takes the block, the rest (16, 4 and 1 texels) the first warp while
+// the others go on; ends without a barrier, the top texel is in shared memory
+// for the first warp.
+template <typename Shared>
+__device__ void build_upper(const RegionParams &P, Shared &sh, int ls, int L0, int face, int ox, int oy) {
+  if (ls >= 2) {
+    build_level(P, sh, 2, ls - 2, 0, 1 << (2 * (ls - 2)), L0, face, ox, oy, threadIdx.x, blockDim.x,
+                FromLevel<Shared>{sh, 1, ls - 1});
+    __syncthreads();
+  }
+  if (threadIdx.x < 32)
+    for (int l = 3; l <= ls; ++l) {
+      build_level(P, sh, l, ls - l, 0, 1 << (2 * (ls - l)), L0, face, ox, oy, threadIdx.x, 32,
+                  FromLevel<Shared>{sh, l - 1, ls - l + 1});
+      __syncwarp();
+    }
+}
+
+template <typename Shared>
+__device__ __forceinline__ Node top_node(const Shared &sh, int ls) {
+  Node r = {0, 0, 0, kNoPosition, 0};
+  FromLevel<Shared>{sh, ls, 0}(0, 0, r);
+  return r;
+}
+
+// Occupancy blocks (mask_level_offset) of level l <= 2 of a region of 32 x 32
+// level-0 texels.  A block's second eight columns belong to its right
+// neighbour: within the region they are at hand, past it the neighbour
+// writes them (and this region writes its left neighbour's), byte by byte.
+template <typename Shared>
+__device__ void write_mask(const RegionParams &P, const Shared &sh, int l, int face, int rx, int ry, int t0) {
+  const int s = kRegion >> l, lc = 2 - l, nbc = 1 << lc, nbr = s / 4, NL = P.N >> l, nbx = NL / 8, nby = NL / 4;
+  for (int b = t0; b < nbc * nbr; b += 32) {
+    const int bx = b & (nbc - 1), by = b >> lc, gx = rx * nbc + bx, gy = ry * nbr + by;
+    unsigned row[4];
+    for (int r = 0; r < 4; ++r) {
+      const int bit = (by * 4 + r) * s;
+      const unsigned w = (sh.lit[l][bit >> 5] >> (bit & 31)) & (s == 32 ? 0xffffffffu : (1u << s) - 1u);
+      row[r] = __brev(w >> (8 * bx)) >> 16;  // columns 8 bx .. 8 bx + 15, the first on top
+    }
+    unsigned char *m = P.mask + 8 * (P.mask_off[l] + ((long long)face * nby + gy) * nbx + gx);
+    if (bx + 1 < nbc || gx + 1 == nbx) {
+      *reinterpret_cast<uint2 *>(m) = make_uint2((row[0] << 16) | row[1], (row[2] << 16) | row[3]);
+    } else {
+      m[3] = (unsigned char)(row[0] >> 8);
+      m[1] = (unsigned char)(row[1] >> 8);
+      m[7] = (unsigned char)(row[2] >> 8);
+      m[5] = (unsigned char)(row[3] >> 8);
+    }
+    if (bx == 0 && gx > 0) {
+      m -= 8;
+      m[2] = (unsigned char)(row[0] >> 8);
+      m[0] = (unsigned char)(row[1] >> 8);
+      m[6] = (unsigned char)(row[2] >> 8);
+      m[4] = (unsigned char)(row[3] >> 8);
+    }
+  }
+}
+
+// Bound by instruction issue and by the chain of loads and levels (about 6 us a
+// region), so: eight small blocks per SM, and the few texels that hold sums (41
+// of 1024 for 1M stars on 2048^2 faces) are listed and computed side by side
+// instead of one or two to a warp.
+template <int kSlots>
+__global__ void __launch_bounds__(kSlots, 1024 / kSlots) region_kernel(const RegionParams P) {
+  __shared__ __align__(16) RegionShared<kSlots> sh;
+  const int N = P.N, ls = min(31 - __clz(N), 5), side = 1 << ls;
+  int lp = max(31 - __clz(N) - 5, 0);  // log2 of the groups per face side
+  const int region = blockIdx.x, face = region >> (2 * lp);
+  int gx = region & ((1 << lp) - 1), gy = region >> lp & ((1 << lp) - 1);
+  const int tid = threadIdx.x, lane = tid & 31;
+  RegionSpan span = {0, 0};
+  if (P.items && P.span) span = P.span[region];
+  const StarItem *items = P.items + span.first;
+  uint2 *const rec0 = P.rec + ((long long)face * N + gy * side) * N + gx * side;
+  if (tid < kRegion) {
+    sh.touched[tid] = 0;
+    sh.lit[0][tid] = 0;
+    sh.lit[1][tid] = 0;
+  }
+  if (tid < 8) sh.full[1][tid] = 0;
+  if (tid == 0) sh.n0 = sh.n1 = 0;
+  // ---- sums of the region's texels, and levels 0 and 1
+  auto add = [&](const StarItem &st, int k) {
+    for (int c = 0; c < 3; ++c) shared_add(sh, c, k, st.q[c]);
+    shared_add(sh, 3, k, st.q[1] * (long long)(st.pos & 0xffffu));
+    shared_add(sh, 4, k, st.q[1] * (long long)(st.pos >> 16));
+  };
+  auto level0_record = [&](int q) {  // of the sums in slot q
+    const long long x = shared_sum(sh, 0, q), y = shared_sum(sh, 1, q), z = shared_sum(sh, 2, q);
+    unsigned p = kNoPosition;
+    if (y > 0)
+      p = (unsigned)(mean_byte0(shared_sum(sh, 3, q), y) | (mean_byte0(shared_sum(sh, 4, q), y) << 8)) & 0xffffu;
+    sh.p0[q] = (unsigned short)p;
+    return make_record(x, y, z, p, 0, P.dtype);
+  };
+  if (P.items && span.count <= kSlots) {
+    // few stars: a slot for each texel that one touches
+    StarItem st;
+    const bool has = tid < (int)span.count;
+    if (has) st = items[tid];
+    __syncthreads();
+    if (has) {
+      const int j = st.local >> 5, i = st.local & 31;
+      if (!(atomicOr(&sh.touched[j], 1u << i) >> i & 1u)) {  // the texel's first star
+        const unsigned k = atomicAdd(&sh.n0, 1u);
+        sh.slot[st.local] = (unsigned short)k;
+        sh.list0[k] = (unsigned short)st.local;
+        for (int c = 0; c < 10; ++c) sh.acc[c][k] = 0;
+        if (ls > 0) {
+          const unsigned t = ((j >> 1) << (ls - 1)) + (i >> 1);
+          if (!(atomicOr(&sh.full[1][t >> 5], 1u << (t & 31)) >> (t & 31) & 1u))
+            sh.list1[atomicAdd(&sh.n1, 1u)] = (unsigned short)t;
+        }
+      }
+    }
+    __syncthreads();
+    if (has) add(st, sh.slot[st.local]);
+    for (int k = tid; k < side * side; k += blockDim.x) {
+      const int j = k >> ls, i = k & (side - 1);
+      if (!(sh.touched[j] >> i & 1u)) rec0[(long long)j * N + i] = kEmptyRecord;
+    }
+    __syncthreads();
+    if (tid < (int)sh.n0) {
+      const int t = sh.list0[tid], j = t >> 5, i = t & 31;
+      const uint2 v = level0_record(tid);
+      rec0[(long long)j * N + i] = v;
+      if (has_colour(v)) atomicOr(&sh.lit[0][j], 1u << i);
+    }
+    __syncthreads();
+    if (ls > 0) {
+      const int l1 = ls - 1, N1 = N >> 1;
+      uint2 *rec1 = P.rec + P.level_off[1] + ((long long)face * N1 + (gy << l1)) * N1 + (gx << l1);
+      for (int t = tid; t < 1 << (2 * l1); t += blockDim.x)
+        if (!(sh.full[1][t >> 5] >> (t & 31) & 1u)) rec1[(long long)(t >> l1) * N1 + (t & ((1 << l1) - 1))] = kEmptyRecord;
+      if (tid < (int)sh.n1) {
+        const int t = sh.list1[tid];
+        uint2 v = kEmptyRecord;
+        build_texel(P, sh, 1, l1, t, 1, [&](int j, int i, Node &c) {
+          if (!(sh.touched[j] >> i & 1u)) return false;
+          const int q = sh.slot[j * kRegion + i];
+          c = {shared_sum(sh, 0, q), shared_sum(sh, 1, q), shared_sum(sh, 2, q), sh.p0[q], 0};
+          return true;
+        }, v);
+        rec1[(long long)(t >> l1) * N1 + (t & ((1 << l1) - 1))] = v;
+        if (has_colour(v)) atomicOr(&sh.lit[1][t >> 5], 1u << (t & 31));
+      }
+      __syncthreads();
+    }
+  } else {
+    // many stars, or dense sums: bands of rows, a slot for each texel
+    const int rows = min(side, kSlots >> ls), n = rows << ls;
+    for (int r0 = 0; r0 < side; r0 += rows) {
+      for (int c = 0; c < 10; ++c) sh.acc[c][tid] = 0;
+      __syncthreads();
+      if (P.items) {
+        for (unsigned long long s = tid; s < span.count; s += blockDim.x) {
+          const int j = (int)(items[s].local >> 5) - r0;
+          if (j < 0 || j >= rows) continue;
+          const StarItem st = items[s];
+          atomicOr(&sh.touched[r0 + j], 1u << (st.local & 31));
+          add(st, (j << ls) + (st.local & 31));
+        }
+      } else if (tid < n) {
+        const int j = r0 + (tid >> ls), i = tid & (side - 1);
+        const unsigned long long *a = P.acc + (((long long)face * N + gy * side + j) * N + gx * side + i) * 5;
+        unsigned long long any = 0;
+        for (int c = 0; c < 5; ++c) {
+          const unsigned long long v = a[c];
+          any |= v;
+          sh.acc[2 * c][tid] = (unsigned)v;
+          sh.acc[2 * c + 1][tid] = (unsigned)(v >> 32);
+        }
+        if (any) atomicOr(&sh.touched[j], 1u << i);
+      }
+      __syncthreads();
+      if (tid < n) {
+        const int j = r0 + (tid >> ls), i = tid & (side - 1);
+        uint2 v = kEmptyRecord;
+        if (sh.touched[j] >> i & 1u) v = level0_record(tid);
+        rec0[(long long)j * N + i] = v;
+        if (has_colour(v)) atomicOr(&sh.lit[0][j], 1u << i);
+      }
+      __syncthreads();
+      if (ls > 0)
+        build_level(P, sh, 1, ls - 1, (r0 / 2) << (ls - 1), (rows / 2) << (ls - 1), 0, face, gx * side, gy * side, tid,
+                    blockDim.x, [&](int j, int i, Node &c) {
+                      if (!(sh.touched[j] >> i & 1u)) return false;
+                      const int q = ((j - r0) << ls) + i;
+                      c = {shared_sum(sh, 0, q), shared_sum(sh, 1, q), shared_sum(sh, 2, q), sh.p0[q], 0};
+                      return true;
+                    });
+      __syncthreads();
+    }
+  }
+  if (ls == 0) return;
+  build_upper(P, sh, ls, 0, face, gx * side, gy * side);
+  if (P.mask && (tid >> 5) >= 1 && (tid >> 5) <= 3) write_mask(P, sh, (tid >> 5) - 1, face, gx, gy, lane);
+  // ---- the groups above: the last of up to 32 x 32 groups to finish builds
+  // the next levels from the top texels of them all
+  int L0 = ls, lg = ls;
+  Node *nodes = P.nodes;
+  unsigned *arrived = P.arrived;
+  while (lp > 0) {
+    const int lm = min(lp, 5), la = lp - lm, ax = gx >> lm, ay = gy >> lm;
+    if (tid == 0) {
+      nodes[(((face << lp) + gy) << lp) + gx] = top_node(sh, lg);
+      __threadfence();
+      sh.last = atomicAdd(arrived + (((face << la) + ay) << la) + ax, 1u) == (1u << (2 * lm)) - 1u;
+      __threadfence();
+    }
+    __syncthreads();
+    if (!sh.last) return;
+    const Node *group = nodes + ((((face << lp) + (ay << lm)) << lp) + (ax << lm));
+    build_level(P, sh, 1, lm - 1, 0, 1 << (2 * (lm - 1)), L0, face, ax << lm, ay << lm, tid, blockDim.x,
+                [&](int j, int i, Node &c) {
+                  const ulonglong2 *g = reinterpret_cast<const ulonglong2 *>(group + ((long long)j << lp) + i);
+                  const ulonglong2 a = __ldcg(g), b = __ldcg(g + 1);
+                  c = {(long long)a.x, (long long)a.y, (long long)b.x, (unsigned)b.y, 0};
+                  return true;
+                });
+    __syncthreads();
+    build_upper(P, sh, lm, L0, face, ax << lm, ay << lm);
+    nodes += 6LL << (2 * lp);
+    arrived += 6LL << (2 * la);
+    L0 += lm;
+    lg = lm;
+    lp = la;
+    gx = ax;
+    gy = ay;
+  }
+}
+
+// Nodes and arrival counters of the stages above the regions.
+static void stage_sizes(int N, long long *nodes, long long *counters) {
+  *nodes = *counters = 0;
+  for (long long per = std::max(N / kRegion, 1); per > 1;) {
+    const long long above = per / std::min<long long>(per, kRegion);
+    *nodes += 6 * per * per;
+    *counters += 6 * above * above;
+    per = above;
+  }
+}
+
+// Occupancy blocks of levels first .. levels - 1 (mask_level_offset) from the
+// records, one warp per block; a ballot gives the bits of 8 columns x 4 rows
+// (lane = 8 row + column, reversed into bit 31 - lane).  A texel is occupied
+// when its colour is not zero: the renderer takes only those of a footprint.
+__global__ void occupancy_kernel(const uint2 *rec, int N, int first, int levels, uint2 *mask) {
+  long long blk = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5;
+  int L = 0, nbx = 0, nby = 0;
+  long long in_level = blk, before = 0, texels = 0;  // blocks and records of the levels before L
+  for (L = 0; L < levels; texels += 6LL * (N >> L) * (N >> L), ++L) {
+    nbx = max((N >> L) >> 3, 1);
+    nby = max((N >> L) >> 2, 1);
+    const long long here = 6LL * nbx * nby;
+    if (L < first) { before += here; continue; }
+    if (in_level < here) break;
+    in_level -= here;
+    before += here;
+  }
+  if (L == levels) return;  // whole warps leave together
+  const int lane = threadIdx.x & 31, NL = N >> L;
+  const int bx = (int)(in_level % nbx), by = (int)(in_level / nbx % nby), face = (int)(in_level / ((long long)nbx * nby));
   const int j = by * 4 + (lane >> 3), i = bx * 8 + (lane & 7);
+  const uint2 *level = rec + texels;
   auto occupied = [&](const int ii) {
     if (ii >= NL || j >= NL) return false;
-    const uint2 v = rec[((long long)face * NL + j) * NL + ii];
+    const uint2 v = level[((long long)face * NL + j) * NL + ii];
     return (v.x | (v.y & 0xffffu)) != 0u;
   };
   const unsigned a = __brev(__ballot_sync(0xffffffffu, occupied(i)));
   const unsigned b = __brev(__ballot_sync(0xffffffffu, occupied(i + 8)));
   // bytes of a and b are rows (row 0 on top): interleave them
-  if (lane == 0) mask[blk] = make_uint2(__byte_perm(a, b, 0x3726u), __byte_perm(a, b, 0x1504u));
+  if (lane == 0) mask[before + in_level] = make_uint2(__byte_perm(a, b, 0x3726u), __byte_perm(a, b, 0x1504u));
 }
 
-// The occupancy mask of every level from the records.
-void occupancy_launch(bh_ctx *ctx, const bh_cubemap *c, cudaStream_t s) {
-  for (int L = 0; L < c->levels; ++L) {
-    const long long blocks = mask_level_offset(c->n, L + 1) - mask_level_offset(c->n, L);
-    occupancy_kernel<<<(unsigned)((blocks + 7) / 8), 256, 0, s>>>(c->rec + cube_level_offset(c->n, L), c->n >> L,
-                                                                 c->mask + mask_level_offset(c->n, L));
-    count_launch(ctx);
-  }
+// The occupancy mask of levels `first` and up from the records.
+void occupancy_launch(bh_ctx *ctx, const bh_cubemap *c, int first, cudaStream_t s) {
+  const long long blocks = mask_level_offset(c->n, c->levels) - mask_level_offset(c->n, first);
+  if (blocks <= 0) return;
+  occupancy_kernel<<<(unsigned)((blocks + 7) / 8), 256, 0, s>>>(c->rec, c->n, first, c->levels, c->mask);
+  count_launch(ctx);
 }
+
+static unsigned star_blocks(long long n) { return (unsigned)((n + 255) / 256); }
 
 }  // namespace bh
 
@@ -209,57 +870,74 @@ extern "C" bh_status bh_build_star_cubemap(bh_ctx *ctx, const bh_star *stars, lo
   }
   BH_CUDA(cudaSetDevice(ctx->device));
   cudaStream_t s = (cudaStream_t)stream;
-  bh_cubemap *c = new bh_cubemap();
-  c->ctx = ctx;
-  c->n = N;
-  c->levels = cube_levels(N);
-  c->storage = storage;
-  c->records = bh_cubemap_records(N);
-  long long nt0 = 6LL * N * N;
-  long long nt1 = N > 1 ? 6LL * (N / 2) * (N / 2) : 1;
-  unsigned long long *acc = nullptr;
-  long long *sums0 = nullptr, *sums1 = nullptr;
-  double *cmf = nullptr;
-  bh_star *dstars = nullptr;
-  const size_t mask_bytes = sizeof(uint2) * mask_level_offset(N, c->levels);
-  cudaError_t e = cudaMalloc((void **)&c->rec, sizeof(uint2) * c->records);
-  if (e == cudaSuccess) e = cudaMalloc((void **)&c->mask, mask_bytes);
-  if (e == cudaSuccess) e = cudaMallocAsync((void **)&acc, sizeof(unsigned long long) * 5 * nt0, s);
-  if (e == cudaSuccess) e = cudaMallocAsync((void **)&sums0, sizeof(long long) * 3 * nt0, s);
-  if (e == cudaSuccess) e = cudaMallocAsync((void **)&sums1, sizeof(long long) * 3 * nt1, s);
-  if (e == cudaSuccess) e = cudaMallocAsync((void **)&cmf, sizeof(double) * 3 * kNLambda, s);
-  const bh_star *src = stars;
-  if (e == cudaSuccess && n > 0 && !on_device) {
-    e = cudaMallocAsync((void **)&dstars, sizeof(bh_star) * n, s);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(dstars, stars, sizeof(bh_star) * n, cudaMemcpyHostToDevice, s);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);  // the host list may be freed on return
-    src = dstars;
+  bh_cubemap *c = nullptr;
+  bh_status st = cubemap_alloc_public(ctx, N, storage, &c);
+  if (st) return st;
+  // Scratch, one allocation: counters (cleared), offsets, colour fit, stage
+  // nodes, then the sorted stars -- or, where those would take more than the
+  // dense sums of the level-0 texels and 1 GiB, the sums (cleared).
+  const long long per = std::max(N / kRegion, 1), regions = 6 * per * per, texels = 6LL * N * N;
+  long long n_nodes, n_counters;
+  stage_sizes(N, &n_nodes, &n_counters);
+  const size_t sorted = (sizeof(StarBin) + sizeof(StarItem)) * (size_t)n, dense = sizeof(unsigned long long) * 5 * texels;
+  const bool sort = sorted <= std::max<size_t>(dense, (size_t)1 << 30);
+  auto up16 = [](size_t b) { return (b + 15) / 16 * 16; };
+  const size_t b_arrived = up16(sizeof(unsigned) * (kChromaCells + n_counters)), b_count = up16(sizeof(unsigned long long) * (regions + 1));
+  const size_t b_acc = sort ? 0 : dense, b_span = sizeof(RegionSpan) * regions;
+  const size_t b_fit = up16(sizeof(double) * (3 * kNLambda + kChromaCoefs + kChromaVals)), b_nodes = sizeof(Node) * n_nodes;
+  const size_t b_stars = sort ? sorted : 0, b_copy = n > 0 && !on_device ? up16(sizeof(bh_star) * (size_t)n) : 0;
+  const size_t cleared = b_arrived + b_count + b_acc;
+  unsigned char *scratch = nullptr;
+  cudaError_t e = cudaMallocAsync((void **)&scratch, cleared + b_span + b_fit + b_nodes + b_stars + b_copy, s);
+  if (e != cudaSuccess) {
+    bh_cubemap_free(c);
+    return cuda_fail(e, "bh_build_star_cubemap");
   }
-  if (e == cudaSuccess) e = cudaMemsetAsync(acc, 0, sizeof(unsigned long long) * 5 * nt0, s);
+  RegionParams P;
+  unsigned *fitted = reinterpret_cast<unsigned *>(scratch);
+  P.arrived = fitted + kChromaCells;
+  unsigned long long *count = reinterpret_cast<unsigned long long *>(scratch + b_arrived), *cursor = count + regions;
+  unsigned long long *acc = reinterpret_cast<unsigned long long *>(scratch + b_arrived + b_count);
+  RegionSpan *span = reinterpret_cast<RegionSpan *>(scratch + cleared);
+  double *cmf = reinterpret_cast<double *>(scratch + cleared + b_span), *coef = cmf + 3 * kNLambda, *vals = coef + kChromaCoefs;
+  P.nodes = reinterpret_cast<Node *>(scratch + cleared + b_span + b_fit);
+  StarItem *items = reinterpret_cast<StarItem *>(scratch + cleared + b_span + b_fit + b_nodes);
+  StarBin *bins = reinterpret_cast<StarBin *>(items + n);
+  const bh_star *src = stars;
+  if (b_copy) {
+    bh_star *copy = reinterpret_cast<bh_star *>(scratch + cleared + b_span + b_fit + b_nodes + b_stars);
+    e = cudaMemcpyAsync(copy, stars, sizeof(bh_star) * n, cudaMemcpyHostToDevice, s);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);  // the host list may be freed on return
+    src = copy;
+  }
+  if (e == cudaSuccess) e = cudaMemsetAsync(scratch, 0, cleared, s);
   if (e == cudaSuccess) {
-    cube_cmf_kernel<<<1, 128, 0, s>>>(cmf);
-    if (n > 0) star_bin_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(src, n, N, cmf, acc);
-    level0_kernel<<<(unsigned)((nt0 + 255) / 256), 256, 0, s>>>(acc, nt0, storage, c->rec, sums0);
-    count_launch(ctx, n > 0 ? 3 : 2);
-    long long *ps = sums0, *cs = sums1;
-    for (int L = 1; L < c->levels; ++L) {
-      int Np = N >> (L - 1);
-      long long ntc = 6LL * (Np / 2) * (Np / 2);
-      mip_kernel<<<(unsigned)((ntc + 255) / 256), 256, 0, s>>>(
-          ps, c->rec + cube_level_offset(N, L - 1), Np, L, storage, cs, c->rec + cube_level_offset(N, L));
-      count_launch(ctx);
-      long long *tmp = ps;
-      ps = cs;
-      cs = tmp;
+    if (n > 0) {
+      chroma_launch(cmf, vals, fitted, coef, s);
+      if (sort) {
+        star_bin_kernel<<<star_blocks(n), 256, 0, s>>>(src, n, N, count, bins);
+        region_span_kernel<<<(unsigned)((regions + 255) / 256), 256, 0, s>>>(count, (int)regions, cursor, span);
+        star_scatter_kernel<<<star_blocks(n), 256, 0, s>>>(src, n, bins, span, cmf, coef, items);
+      } else {
+        star_accumulate_kernel<<<star_blocks(n), 256, 0, s>>>(src, n, N, cmf, coef, acc);
+      }
+      count_launch(ctx, sort ? 4 : 2);
     }
-    occupancy_launch(ctx, c, s);
+    P.items = sort ? items : nullptr;
+    P.span = n > 0 ? span : nullptr;
+    P.acc = acc;
+    P.rec = c->rec;
+    P.mask = N >= kRegion ? reinterpret_cast<unsigned char *>(c->mask) : nullptr;
+    P.N = N;
+    P.dtype = storage;
+    region_levels(P);
+    if (sort) region_kernel<kSortedSlots><<<(unsigned)regions, kSortedSlots, 0, s>>>(P);
+    else region_kernel<kDenseSlots><<<(unsigned)regions, kDenseSlots, 0, s>>>(P);
+    count_launch(ctx);
+    occupancy_launch(ctx, c, N >= kRegion ? 3 : 0, s);
     e = cudaGetLastError();
   }
-  cudaFreeAsync(acc, s);
-  cudaFreeAsync(sums0, s);
-  cudaFreeAsync(sums1, s);
-  cudaFreeAsync(cmf, s);
-  if (dstars) cudaFreeAsync(dstars, s);
+  cudaFreeAsync(scratch, s);
   if (e != cudaSuccess) {
     bh_cubemap_free(c);
     return cuda_fail(e, "bh_build_star_cubemap");
@@ -322,16 +1000,20 @@ extern "C" void bh_cubemap_free(bh_cubemap *c) {
 // not call cudaMalloc/cudaFree, which can synchronise the device and take an
 // unbounded time.  The scratch lives in one file-scope device array, sized for
 // faces of up to kNoAllocMaxFace texels; every GPU that loads this library
-// holds it (about 6.9 MB) until the process exits.
+// holds it (about 4 MB) until the process exits.
 // ---------------------------------------------------------------------------
 namespace bh {
 
 constexpr int kNoAllocMaxFace = 128;
 constexpr long long kNoAllocTexels0 = 6LL * kNoAllocMaxFace * kNoAllocMaxFace;
-constexpr long long kNoAllocTexels1 = kNoAllocTexels0 / 4;
-// accumulators (5 x 64 bit per level-0 texel), level sums (3 x 64 bit per
-// texel of two consecutive levels), matching functions (3 x 95 doubles)
-constexpr size_t kNoAllocScratchWords = 5 * kNoAllocTexels0 + 3 * kNoAllocTexels0 + 3 * kNoAllocTexels1 + 3 * kNLambda;
+// arrival counters of the stage above the regions, the sums of the level-0
+// texels (5 x 64 bit each), the top texels of the regions, the matching functions
+// and the colour fit
+constexpr size_t kNoAllocRegions = 6 * (kNoAllocMaxFace / kRegion) * (kNoAllocMaxFace / kRegion);
+constexpr size_t kNoAllocCounters = (kChromaCells + 6 + 1) / 2 / 2 * 2 + 2;  // 32-bit counters: the fit's cells, the faces
+constexpr size_t kNoAllocScratchWords =
+    kNoAllocCounters + 5 * kNoAllocTexels0 + 4 * kNoAllocRegions + 3 * kNLambda + kChromaCoefs + kChromaVals;
+static_assert(kNoAllocMaxFace <= kRegion * kRegion && sizeof(Node) == 32, "one stage above the regions");
 
 static __device__ __align__(256) unsigned long long g_noalloc_scratch[kNoAllocScratchWords];
 
@@ -389,28 +1071,29 @@ extern "C" bh_status bh_build_star_cubemap_noalloc(const bh_star *stars_device, 
   unsigned long long *scratch = nullptr;
   bh_status st = noalloc_scratch(dev, cap != cudaStreamCaptureStatusNone, &scratch);
   if (st) return st;
-  long long nt0 = 6LL * N * N;
-  unsigned long long *acc = scratch;
-  long long *sums0 = reinterpret_cast<long long *>(scratch + 5 * kNoAllocTexels0);
-  long long *sums1 = sums0 + 3 * kNoAllocTexels0;
-  double *cmf = reinterpret_cast<double *>(sums1 + 3 * kNoAllocTexels1);
-  uint2 *rec = reinterpret_cast<uint2 *>(records_device);
-  int levels = cube_levels(N);
-  // the array keeps the previous call's contents: the accumulators must start at zero
-  BH_CUDA(cudaMemsetAsync(acc, 0, sizeof(unsigned long long) * 5 * nt0, s));
-  cube_cmf_kernel<<<1, 128, 0, s>>>(cmf);
-  if (n > 0) star_bin_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(stars_device, n, N, cmf, acc);
-  level0_kernel<<<(unsigned)((nt0 + 255) / 256), 256, 0, s>>>(acc, nt0, storage, rec, sums0);
-  long long *ps = sums0, *cs = sums1;
-  for (int L = 1; L < levels; ++L) {
-    int Np = N >> (L - 1);
-    long long ntc = 6LL * (Np / 2) * (Np / 2);
-    mip_kernel<<<(unsigned)((ntc + 255) / 256), 256, 0, s>>>(ps, rec + cube_level_offset(N, L - 1), Np, L,
-                                                              storage, cs, rec + cube_level_offset(N, L));
-    long long *tmp = ps;
-    ps = cs;
-    cs = tmp;
+  const long long nt0 = 6LL * N * N, per = std::max(N / kRegion, 1);
+  RegionParams P;
+  unsigned *fitted = reinterpret_cast<unsigned *>(scratch);
+  P.arrived = fitted + kChromaCells;
+  unsigned long long *acc = scratch + kNoAllocCounters;
+  P.nodes = reinterpret_cast<Node *>(acc + 5 * kNoAllocTexels0);
+  double *cmf = reinterpret_cast<double *>(P.nodes + kNoAllocRegions), *coef = cmf + 3 * kNLambda;
+  double *vals = coef + kChromaCoefs;
+  // the array keeps the previous call's contents: counters and sums must start at zero
+  BH_CUDA(cudaMemsetAsync(scratch, 0, sizeof(unsigned long long) * (kNoAllocCounters + 5 * nt0), s));
+  if (n > 0) {
+    chroma_launch(cmf, vals, fitted, coef, s);
+    star_accumulate_kernel<<<star_blocks(n), 256, 0, s>>>(stars_device, n, N, cmf, coef, acc);
   }
+  P.items = nullptr;
+  P.span = nullptr;
+  P.acc = acc;
+  P.rec = reinterpret_cast<uint2 *>(records_device);
+  P.mask = nullptr;
+  P.N = N;
+  P.dtype = storage;
+  region_levels(P);
+  region_kernel<kDenseSlots><<<(unsigned)(6 * per * per), kDenseSlots, 0, s>>>(P);
   BH_CUDA(cudaGetLastError());
   return BH_OK;
 }

@@ -192,5 +192,6 @@ inline int cube_levels(int N) {
 void count_launch(bh_ctx *ctx, int n = 1);
 bh_status check_status(bh_ctx *ctx, cudaStream_t s);
 bh_status colour_tables_launch(bh_ctx *ctx, bh_tables *t, cudaStream_t s);
-void occupancy_launch(bh_ctx *ctx, const bh_cubemap *c, cudaStream_t s);
+void occupancy_launch(bh_ctx *ctx, const bh_cubemap *c, int first, cudaStream_t s);
+bh_status cubemap_alloc_public(bh_ctx *ctx, int N, bh_dtype storage, bh_cubemap **out);
 }  // namespace bh

@@ -17,7 +17,6 @@ namespace bh {
 
 bh_status tables_alloc_public(bh_ctx *ctx, const bh_table_desc *desc, bh_tables **out);
 bh_status tables_convert_storage(bh_ctx *ctx, bh_tables *t, cudaStream_t s);
-bh_status cubemap_alloc_public(bh_ctx *ctx, int N, bh_dtype storage, bh_cubemap **out);
 
 namespace {
 
@@ -290,7 +289,7 @@ extern "C" bh_status bh_cubemap_load(bh_ctx *ctx, const char *path, void *stream
   if (st) return st;
   cudaError_t e = cudaMemcpyAsync(c->rec, rec, (size_t)records * sizeof(uint2), cudaMemcpyHostToDevice, s);
   if (e == cudaSuccess) {
-    occupancy_launch(ctx, c, s);  // the renderer's layout, from the records
+    occupancy_launch(ctx, c, 0, s);  // the renderer's layout, from the records
     e = cudaGetLastError();
   }
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);

@@ -170,6 +170,29 @@ def test_cubemap_bit_exact(ctx, orc, n, N, dtype):
     assert diff.sum() == 0, (diff.sum(), np.flatnonzero(diff)[:5])
 
 
+@pytest.mark.parametrize("N,dtype", [(1, 1), (2, 2), (16, 1), (32, 2), (64, 1), (128, 2), (1024, 1)])
+def test_cubemap_uneven_stars_bit_exact(ctx, orc, N, dtype):
+    """Stars in clusters (one texel, one region), of temperatures on both sides
+    of the fitted range and so bright that records clamp and the mean positions
+    leave the integer range; the allocation-free build on the same stars."""
+    st = synth.stars(6000, 31)
+    st[:1500, :3] = st[0, :3]
+    st[1500:3000, :3] = st[1, :3] + 1e-3 * st[1500:3000, :3]
+    st[3000:3050, :3] = np.eye(3, dtype=np.float32)[np.arange(50) % 3] * np.where(np.arange(50) % 2, 1, -1)[:, None]
+    st[:600, 4] = np.resize(np.array([200, 800, 1023.9, 1024, 1025, 65000, 1e6], np.float32), 600)
+    st[200:260, 3] *= np.float32(3e5)
+    c = bh.bh_build_star_cubemap(ctx, st, N, dtype)
+    try:
+        rec = bh.bh_cubemap_copy_out(c, N)
+    finally:
+        bh.bh_cubemap_free(c)
+    assert np.array_equal(rec, orc.build_cubemap(st, N, dtype))
+    if N <= 128:
+        own = torch.empty((bh.bh_cubemap_records(N), 4), dtype=torch.int16, device="cuda")
+        bh.bh_build_star_cubemap_noalloc(torch.from_numpy(st).cuda(), N, dtype, own)
+        assert np.array_equal(own.cpu().numpy().view(np.uint16), rec)
+
+
 def test_cubemap_from_device_stars(ctx, orc):
     st = synth.stars(4000, seed=12)
     dst = torch.from_numpy(st).cuda()
