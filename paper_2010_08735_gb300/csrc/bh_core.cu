@@ -1,17 +1,28 @@
 // libbh core: context, errors, and the GPU precompute of the tables.
 //
 //  * D(e,u) and U(e,phi) (Algorithm 1 PRECOMPUTE, Appendix A): instead of
-//    Euler steps along each e row, every texel is an independent FP64
-//    quadrature of the ray equation's first integral
+//    Euler steps along each e row, FP64 quadrature of the ray equation's first
+//    integral
 //        phi(u) = int_0^u du' / sqrt(P(u')),  P(u) = e^2 - u^2 (1 - u)
-//    (Eq. rayequation), after a substitution that removes the apsis
-//    singularity and the near-double root at the photon sphere:
-//      e^2 < mu:  P = (u_a - u) q(u), u = u_a - w^2, q = A + B w^2 - w^4,
-//                 and near criticality w = sqrt(A/B) sinh t;
-//      e^2 > mu:  P = (e^2 - mu) + v^2 (v + 1), v = u - 2/3 = sqrt(e^2-mu) sinh t.
-//    Delta = phi - atan2(u, du/dphi) (Algorithm 1).  U inverts phi(u) by
-//    safeguarded Newton iterations on the same quadrature, using the apsis
-//    reflection phi -> 2 phi_a - phi past the apsis (Sec. 3.3.1).
+//    (Eq. rayequation), in a variable without the apsis singularity and fine
+//    enough for the near-double root at the photon sphere:
+//      e^2 < mu:  P = (u_a - u) q(u), u = u_a - w^2, q = A + B w^2 - w^4;
+//      e^2 > mu:  P = (e^2 - mu) + v^2 (v + 1), v = u - 2/3 = z |z|
+//    (D, whose texels are equal steps of w and of z), or w = sqrt(A/B) sinh t and
+//    v = sqrt(e^2-mu) sinh t (U, any e).  One block takes an e: every step
+//    between texels is one four-node Gauss-Legendre panel, a block scan gives
+//    the integrals up to every texel.  Delta = phi - atan2(u, du/dphi)
+//    (Algorithm 1) is integrated directly: with u'' = -u + 3/2 u^2 (the ray
+//    equation), dDelta/dphi = (3/2) u^3 / (e^2 + u^3).  U inverts phi(u) by
+//    Newton steps inside a panel, using the apsis reflection phi -> 2 phi_a - phi
+//    past the apsis (Sec. 3.3.1).
+//    GB300 does two FP64 multiply-adds per SM and clock, so the number of
+//    integrand values decides: one quadrature from infinity per texel took 64 to
+//    160 of them twice (6.05 ms for 512 x 512; U by up to 80 Newton steps of
+//    whole quadratures 0.99 ms); this takes four per texel: 145 us for both, of
+//    which FP64 is busy 120.  Largest errors at 512 x 512 against quadratures
+//    with 128 nodes: 1.7e-13 on Delta (before: 2.0e-12), 6e-13 on R (4.4e-12),
+//    1.0e-15 on u (1.1e-15), 1.1e-12 on U's R (1.6e-12).
 //  * The colour tables (Sec. 3.4.2): C(xy, D) and the disc black-body table.
 #include <cmath>
 #include <cstdio>
@@ -56,10 +67,10 @@ bh_status check_status(bh_ctx *ctx, cudaStream_t s) {
 }
 
 // ---------------------------------------------------------------------------
-// Gauss-Legendre nodes (16 points) computed once on the host by Newton's
-// method on P_16 with its three-term recurrence.
+// Gauss-Legendre nodes (4 points) computed once on the host by Newton's method
+// on P_4 with its three-term recurrence.
 // ---------------------------------------------------------------------------
-constexpr int kGL = 16;
+constexpr int kGL = 4;
 __constant__ double cGLx[kGL], cGLw[kGL];
 
 static void gauss_legendre(int n, double *x, double *w) {
@@ -104,78 +115,109 @@ __device__ Apsis apsis_of_eta(double eta) {
   return a;
 }
 
-__device__ __forceinline__ double qw(const Apsis &a, double w) {
-  double w2 = w * w;
-  return a.A + a.B * w2 - w2 * w2;
-}
-
 // The regularised time R = t + 1/u - ln(u/(1-u)) (reading C5) obeys
-// dR/dphi = 1/(e + du/dphi), so every angle quadrature below has a time twin
-// (TIME = true) whose integrand carries the extra factor 1/(e + du/dphi).
+// dR/dphi = 1/(e + du/dphi), so every angle integral has a time twin whose
+// integrand carries the extra factor 1/(e + du/dphi).
 
-// int_{w0}^{w1} 2 dw / sqrt(q(w)) [/(e + w sqrt(q))], composite Gauss-Legendre
-template <bool TIME>
-__device__ double quad_w(const Apsis &a, double e, double w0, double w1, int panels) {
-  double h = (w1 - w0) / panels, s = 0.0;
-  for (int p = 0; p < panels; ++p) {
-    double c = w0 + (p + 0.5) * h, r = 0.5 * h;
-    for (int k = 0; k < kGL; ++k) {
-      double w = c + r * cGLx[k], q = qw(a, w), rq = rsqrt(q);
-      double f = 2.0 * rq;
-      if (TIME) f /= e + w * q * rq;
-      s += cGLw[k] * r * f;
-    }
-  }
-  return s;
+// Rays of one e.
+struct Ray {
+  double e, e2;
+  bool low;       // e^2 < mu
+  Apsis ap;       // low
+  double w1;      // low: w at infinity, sqrt(u_a)
+  double c;       // low: scale of w = c sinh t
+  double em, se;  // high: e^2 - mu and its root
+};
+
+__device__ __forceinline__ Ray low_ray(double eta, double e2) {
+  Ray r;
+  r.low = true;
+  r.e2 = e2;
+  r.e = sqrt(e2);
+  r.ap = apsis_of_eta(eta);
+  r.w1 = sqrt(r.ap.ua);
+  r.c = r.ap.B > 0.0 ? sqrt(r.ap.A / r.ap.B) : 1.0;
+  r.em = r.se = 0.0;
+  return r;
 }
 
-// same integral in t, w = c sinh t, c = sqrt(A/B): integrand 2 c cosh t / sqrt(q)
-template <bool TIME>
-__device__ double quad_t_scatter(const Apsis &a, double e, double c, double t0, double t1, int panels) {
-  double h = (t1 - t0) / panels, s = 0.0;
-  for (int p = 0; p < panels; ++p) {
-    double m = t0 + (p + 0.5) * h, r = 0.5 * h;
-    for (int k = 0; k < kGL; ++k) {
-      double t = m + r * cGLx[k];
-      double sh = sinh(t), w = c * sh, q = qw(a, w), rq = rsqrt(q);
-      double f = 2.0 * c * sqrt(1.0 + sh * sh) * rq;
-      if (TIME) f /= e + w * q * rq;
-      s += cGLw[k] * r * f;
-    }
-  }
-  return s;
+__device__ __forceinline__ Ray high_ray(double em, double e2) {
+  Ray r;
+  r.low = false;
+  r.e2 = e2;
+  r.e = sqrt(e2);
+  r.em = em;
+  r.se = sqrt(em);
+  r.ap = {0.0, 0.0, 0.0};
+  r.w1 = r.c = 0.0;
+  return r;
 }
 
-// From infinity to u = u_a - w0^2: the angle (TIME = false) or the
-// regularised time (TIME = true), int_{w0}^{sqrt(u_a)} in w.
-template <bool TIME>
-__device__ double scatter_integral(const Apsis &a, double e, double w0) {
-  double w1 = sqrt(a.ua);
-  if (a.ua > 0.6) {
-    double c = sqrt(a.A / a.B);
-    double wm = fmax(w0, fmin(w1, 0.35));
-    return quad_t_scatter<TIME>(a, e, c, asinh(w0 / c), asinh(wm / c), 6) + quad_w<TIME>(a, e, wm, w1, 4);
-  }
-  return quad_w<TIME>(a, e, w0, w1, 4);
+// 1/x and 1/sqrt(x) by Newton's iteration from the single-precision value (x a
+// normal float whose reciprocal is one): 2^-23, 2^-46, then rounding.  Six and
+// ten FP64 operations, a third of the general routines'.
+__device__ __forceinline__ double newton_rcp(double x) {
+  double r = (double)__frcp_rn((float)x);
+  r = fma(r, fma(-x, r, 1.0), r);
+  return fma(r, fma(-x, r, 1.0), r);
 }
 
-// Plunging rays: int_{ta}^{tb} dt / sqrt(1 + v tanh^2 t), v = se sinh t
-// (du/dphi = se cosh t sqrt(1 + v tanh^2 t)).
-template <bool TIME>
-__device__ double plunge_integral(double se, double e, double ta, double tb) {
-  const int panels = 6;
-  double h = (tb - ta) / panels, s = 0.0;
-  for (int p = 0; p < panels; ++p) {
-    double m = ta + (p + 0.5) * h, r = 0.5 * h;
-    for (int k = 0; k < kGL; ++k) {
-      double t = m + r * cGLx[k];
-      double th = tanh(t), g = 1.0 + se * sinh(t) * th * th, rg = rsqrt(g);
-      double f = rg;
-      if (TIME) f /= e + se * cosh(t) * g * rg;
-      s += cGLw[k] * r * f;
-    }
+__device__ __forceinline__ double newton_rsqrt(double x) {
+  double r = (double)rsqrtf((float)x);
+  r = fma(0.5 * r, fma(-x * r, r, 1.0), r);
+  return fma(0.5 * r, fma(-x * r, r, 1.0), r);
+}
+
+// dphi/ds, u and du/dphi at a point: s = w (low) or z (high), falling and
+// rising with phi.
+__device__ __forceinline__ double ray_rate(const Ray &r, double s, double &u, double &ud) {
+  if (r.low) {
+    const double w2 = s * s, q = fma(w2, r.ap.B - w2, r.ap.A), rq = newton_rsqrt(q);
+    u = r.ap.ua - w2;
+    ud = s * (q * rq);
+    return 2.0 * rq;
   }
-  return s;
+  const double v = s * fabs(s), P = fma(v * v, v + 1.0, r.em), rp = newton_rsqrt(P);
+  u = 2.0 / 3.0 + v;
+  ud = P * rp;
+  return 2.0 * fabs(s) * rp;
+}
+
+// The same in t: w = c sinh t where u_a > 0.6 and v = sqrt(e^2-mu) sinh t, else w
+// = t.
+__device__ __forceinline__ bool ray_sinh(const Ray &r) { return !r.low || r.ap.ua > 0.6; }
+
+__device__ __forceinline__ double ray_rate_t(const Ray &r, double t, double &u, double &ud) {
+  if (!ray_sinh(r)) return ray_rate(r, t, u, ud);
+  const double sh = sinh(t), ch = sqrt(fma(sh, sh, 1.0));
+  if (r.low) return ray_rate(r, r.c * sh, u, ud) * r.c * ch;
+  // P = (e^2 - mu) cosh^2 t (1 + v tanh^2 t)
+  const double v = r.se * sh, th = sh / ch, g = fma(v * th, th, 1.0), rg = rsqrt(g);
+  u = 2.0 / 3.0 + v;
+  ud = r.se * ch * (g * rg);
+  return rg;
+}
+
+// Inclusive scan of two sums over the block (a multiple of 32 threads, at
+// most 1024), plus the totals; buf holds 64 doubles.
+__device__ __forceinline__ void block_scan2(double &a, double &b, double *buf, double &ta, double &tb) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
+  for (int o = 1; o < 32; o <<= 1) {
+    const double x = __shfl_up_sync(0xffffffffu, a, o), y = __shfl_up_sync(0xffffffffu, b, o);
+    if (lane >= o) { a += x; b += y; }
+  }
+  __syncthreads();  // buf may still be read from the scan before
+  if (lane == 31) { buf[warp] = a; buf[32 + warp] = b; }
+  __syncthreads();
+  double pa = 0.0, pb = 0.0;
+  ta = tb = 0.0;
+  for (int w = 0; w < warps; ++w) {
+    if (w == warp) { pa = ta; pb = tb; }
+    ta += buf[w];
+    tb += buf[32 + w];
+  }
+  a += pa;
+  b += pb;
 }
 
 template <typename T>
@@ -185,186 +227,208 @@ __device__ __forceinline__ float to_storage<float>(double v) { return (float)v; 
 template <>
 __device__ __forceinline__ __half to_storage<__half>(double v) { return __double2half(v); }
 
-// D(e,u) per texel: texel (i,j) holds the Appendix A coordinates
-// x = i/(n-1), y = j/(n-1) (reading C3).
-__global__ void precompute_D_kernel(int n, double *D64, double *DT64, float *DTs) {
-  int i = blockIdx.x * blockDim.x + threadIdx.x;
-  int j = blockIdx.y;
-  if (i >= n || j >= n) return;
-  double x = (double)i / (n - 1), y = (double)j / (n - 1);
-  double Delta, R;
-  if (i < n / 2) {
-    // x = 1/2 - sqrt(-log(1 - e^2/mu)/50): eta = 1 - e^2/mu = exp(-50 (1/2 - x)^2)
-    double a = 0.5 - x;
-    double eta = exp(-50.0 * a * a);
-    double e = sqrt(-kMu * expm1(-50.0 * a * a));
-    Apsis ap = apsis_of_eta(eta);
-    double w0 = sqrt(ap.ua) * (1.0 - y);  // y = 1 - sqrt(1 - u/u_a)
-    double u = ap.ua - w0 * w0;
-    double phi = scatter_integral<false>(ap, e, w0);
-    double udot = w0 * sqrt(qw(ap, w0));
-    Delta = phi - atan2(u, udot);
-    R = scatter_integral<true>(ap, e, w0);
-  } else {
+constexpr int kColumnThreads = 256, kDSteps = 2;
+
+// Column i of D and its time channel: texel (i,j) holds the Appendix A
+// coordinates x = i/(n-1), y = j/(n-1) (reading C3).
+__device__ void d_column(int n, int i, double *D64, double *DT64, float *DTs, double *buf) {
+  // the ray's constants cost as much FP64 as 50 nodes: one thread forms them
+  __shared__ Ray ray;
+  if (threadIdx.x == 0) {
+    // x = 1/2 - sqrt(-log(1 - e^2/mu)/50): eta = 1 - e^2/mu = exp(-50 (1/2 - x)^2);
     // x = 1/2 + sqrt(-log(1 - mu/e^2)/50): 1 - mu/e^2 = exp(-50 (x - 1/2)^2)
-    double a = x - 0.5;
-    double g = exp(-50.0 * a * a);
-    double e2 = kMu / (-expm1(-50.0 * a * a));
-    double em = e2 * g;  // e^2 - mu
-    double se = sqrt(em);
-    const double r23 = sqrt(2.0 / 3.0), r13 = sqrt(1.0 / 3.0);
-    double z = y * (r23 + r13) - r23;
-    double v = z >= 0.0 ? z * z : -z * z;  // u - 2/3
-    double u = 2.0 / 3.0 + v;
-    double ta = asinh(-2.0 / 3.0 / se), tb = asinh(v / se);
-    double phi = plunge_integral<false>(se, 0.0, ta, tb);
-    double udot = sqrt(em + v * v * (v + 1.0));
-    Delta = phi - atan2(u, udot);
-    R = plunge_integral<true>(se, sqrt(e2), ta, tb);
+    const double x = (double)i / (n - 1), a = fabs(0.5 - x);
+    const double eta = exp(-50.0 * a * a), one_eta = -expm1(-50.0 * a * a);
+    ray = i < n / 2 ? low_ray(eta, kMu * one_eta) : high_ray(kMu / one_eta * eta, kMu / one_eta);
   }
-  D64[(size_t)j * n + i] = Delta;
-  DT64[(size_t)j * n + i] = R;
-  DTs[(size_t)j * n + i] = (float)R;
-}
-
-// Warp-cooperative forms of the quadratures above: the 32 lanes of a warp
-// share the Gauss-Legendre nodes of one integral and sum them with shuffles,
-// so that the Newton iterations of one U texel run on a whole warp.
-__device__ __forceinline__ double warp_sum(double v) {
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
-
-template <bool TIME>
-__device__ double warp_quad_w(const Apsis &a, double e, double w0, double w1, int panels, int lane) {
-  double h = (w1 - w0) / panels, s = 0.0;
-  for (int idx = lane; idx < panels * kGL; idx += 32) {
-    int p = idx / kGL, k = idx % kGL;
-    double c = w0 + (p + 0.5) * h, r = 0.5 * h;
-    double w = c + r * cGLx[k], q = qw(a, w), rq = rsqrt(q);
-    double f = 2.0 * rq;
-    if (TIME) f /= e + w * q * rq;
-    s += cGLw[k] * r * f;
-  }
-  return warp_sum(s);
-}
-
-template <bool TIME>
-__device__ double warp_quad_t_scatter(const Apsis &a, double e, double c, double t0, double t1, int panels,
-                                      int lane) {
-  double h = (t1 - t0) / panels, s = 0.0;
-  for (int idx = lane; idx < panels * kGL; idx += 32) {
-    int p = idx / kGL, k = idx % kGL;
-    double m = t0 + (p + 0.5) * h, r = 0.5 * h;
-    double sh = sinh(m + r * cGLx[k]), w = c * sh, q = qw(a, w), rq = rsqrt(q);
-    double f = 2.0 * c * sqrt(1.0 + sh * sh) * rq;
-    if (TIME) f /= e + w * q * rq;
-    s += cGLw[k] * r * f;
-  }
-  return warp_sum(s);
-}
-
-template <bool TIME>
-__device__ double warp_scatter_integral(const Apsis &a, double e, double w0, int lane) {
-  double w1 = sqrt(a.ua);
-  if (a.ua > 0.6) {
-    double c = sqrt(a.A / a.B);
-    double wm = fmax(w0, fmin(w1, 0.35));
-    return warp_quad_t_scatter<TIME>(a, e, c, asinh(w0 / c), asinh(wm / c), 6, lane) +
-           warp_quad_w<TIME>(a, e, wm, w1, 4, lane);
-  }
-  return warp_quad_w<TIME>(a, e, w0, w1, 4, lane);
-}
-
-template <bool TIME>
-__device__ double warp_plunge_integral(double se, double e, double ta, double tb, int lane) {
-  const int panels = 6;
-  double h = (tb - ta) / panels, s = 0.0;
-  for (int idx = lane; idx < panels * kGL; idx += 32) {
-    int p = idx / kGL, k = idx % kGL;
-    double t = ta + (p + 0.5) * h + 0.5 * h * cGLx[k];
-    double th = tanh(t), g = 1.0 + se * sinh(t) * th * th, rg = rsqrt(g);
-    double f = rg;
-    if (TIME) f /= e + se * cosh(t) * g * rg;
-    s += cGLw[k] * 0.5 * h * f;
-  }
-  return warp_sum(s);
-}
-
-// U(e,phi) per texel, one warp per texel: x = 1/(1 + 6 e^2),
-// y = (phi/3)(1 + 6 e^3)/(1 + e^2).  UT gets the regularised time at the
-// same point; past the apsis it follows from the time symmetry of the ray
-// about its apsis, t(phi) = 2 t_a - t(2 phi_a - phi).
-template <typename T>
-__global__ void precompute_U_kernel(int ne, int nphi, double *U64, T *Us, double *UT64, float *UTs) {
-  int lane = threadIdx.x & 31;
-  int texel = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  if (texel >= ne * nphi) return;  // whole warps leave together
-  int i = texel % ne, j = texel / ne;
-  double u, R = 0.0;  // R = 0 where there is no ray or it was captured
-  if (i == 0) {
-    u = j == 0 ? 0.0 : 1.0;  // e -> infinity: radial ray, captured at once
-  } else {
-    double x = (double)i / (ne - 1), y = (double)j / (nphi - 1);
-    double e2 = (1.0 / x - 1.0) / 6.0;
-    double e = sqrt(e2);
-    double phi = 3.0 * y * (1.0 + e2) / (1.0 + 6.0 * e2 * e);
-    if (e2 <= 0.0 || phi <= 0.0) {
-      u = 0.0;
-    } else if (e2 < kMu) {
-      Apsis ap = apsis_of_eta(1.0 - e2 / kMu);
-      double phia = warp_scatter_integral<false>(ap, e, 0.0, lane);
-      bool past = phi > phia;
-      if (past) phi = 2.0 * phia - phi;  // past the apsis: reflection
-      double lo = 0.0, hi = sqrt(ap.ua), w = 0.5 * (lo + hi);
-      for (int it = 0; it < 80; ++it) {
-        double F = warp_scatter_integral<false>(ap, e, w, lane) - phi;  // decreasing in w
-        if (F > 0.0) lo = w; else hi = w;
-        double dF = -2.0 * rsqrt(qw(ap, w));
-        double wn = w - F / dF;
-        if (!(wn > lo && wn < hi)) wn = 0.5 * (lo + hi);
-        if (fabs(wn - w) < 1e-16) { w = wn; break; }
-        w = wn;
-      }
-      u = ap.ua - w * w;
-      R = warp_scatter_integral<true>(ap, e, w, lane);
-      if (past) {
-        if (u > 0.0) {
-          double Ra = warp_scatter_integral<true>(ap, e, 0.0, lane);
-          double l = 2.0 * log(u / (1.0 - u)), la = 2.0 * log(ap.ua / (1.0 - ap.ua));
-          R = 2.0 * Ra - 2.0 / ap.ua + la - R + 2.0 / u - l;
+  __syncthreads();
+  const Ray r = ray;
+  const double r23 = sqrt(2.0 / 3.0), r13 = sqrt(1.0 / 3.0);
+  // y = 1 - sqrt(1 - u/u_a) = 1 - w/w1 (low), equal steps of z (high)
+  auto place = [&](double y) { return r.low ? r.w1 * (1.0 - y) : y * (r23 + r13) - r23; };
+  // panels between two texels: never wider than 1/511 of the range
+  const int parts = (511 + n - 2) / (n - 1), panels = (n - 1) * parts;
+  const double dy = 1.0 / panels;
+  double base_d = 0.0, base_t = 0.0;
+  for (int k0 = 0; k0 < panels; k0 += kDSteps * blockDim.x) {
+    const int first = k0 + kDSteps * threadIdx.x;
+    double sd[kDSteps], st[kDSteps], all_d = 0.0, all_t = 0.0, p = place(first * dy);
+#pragma unroll
+    for (int c = 0; c < kDSteps; ++c) {
+      sd[c] = st[c] = 0.0;
+      if (first + c < panels) {
+        // the last panel ends at y = 1 exactly
+        const double q = place(first + c + 1 == panels ? 1.0 : (first + c + 1) * dy);
+        auto panel = [&](double p, double q) {
+          const double m = 0.5 * (p + q), h = 0.5 * fabs(q - p);
+          double vd = 0.0, vt = 0.0;
+#pragma unroll
+          for (int g = 0; g < kGL; ++g) {
+            double u, ud;
+            const double f = ray_rate(r, fma(h, cGLx[g], m), u, ud) * cGLw[g];
+            const double u3 = u * u * u, den = r.e2 + u3, den_t = r.e + ud, inv = newton_rcp(den * den_t);
+            vd = fma(f, u3 * (den_t * inv), vd);
+            vt = fma(f, den * inv, vt);
+          }
+          sd[c] = fma(1.5 * h, vd, sd[c]);
+          st[c] = fma(h, vt, st[c]);
+        };
+        if (!r.low && p < 0.0 && q > 0.0) {  // |z| has a corner at 0
+          panel(p, 0.0);
+          panel(0.0, q);
         } else {
-          R = 0.0;  // back at infinity: no texel of the mapping gets here
+          panel(p, q);
         }
+        p = q;
       }
-    } else {
-      double se = sqrt(e2 - kMu);
-      double ta = asinh(-2.0 / 3.0 / se), tb = asinh(1.0 / 3.0 / se);
-      if (phi >= warp_plunge_integral<false>(se, e, ta, tb, lane)) {
-        u = 1.0;  // reached the horizon before phi (reading C7)
-      } else {
-        double lo = ta, hi = tb, t = 0.5 * (lo + hi);
-        for (int it = 0; it < 80; ++it) {
-          double F = warp_plunge_integral<false>(se, e, ta, t, lane) - phi;  // increasing in t
-          if (F < 0.0) lo = t; else hi = t;
-          double th = tanh(t);
-          double dF = rsqrt(1.0 + se * sinh(t) * th * th);
-          double tn = t - F / dF;
-          if (!(tn > lo && tn < hi)) tn = 0.5 * (lo + hi);
-          if (fabs(tn - t) < 1e-16) { t = tn; break; }
-          t = tn;
-        }
-        u = 2.0 / 3.0 + se * sinh(t);
-        R = warp_plunge_integral<true>(se, e, ta, t, lane);
+      all_d += sd[c];
+      all_t += st[c];
+    }
+    double up_d = all_d, up_t = all_t, td, tt;
+    block_scan2(up_d, up_t, buf, td, tt);
+    up_d += base_d - all_d;  // the integrals before this thread's panels
+    up_t += base_t - all_t;
+#pragma unroll
+    for (int c = 0; c < kDSteps; ++c) {
+      const int k = first + c + 1;
+      up_d += sd[c];
+      up_t += st[c];
+      if (k <= panels && (parts == 1 || k % parts == 0)) {
+        const size_t o = (size_t)(parts == 1 ? k : k / parts) * n + i;
+        D64[o] = up_d;
+        DT64[o] = up_t;
+        DTs[o] = (float)up_t;
       }
     }
+    base_d += td;
+    base_t += tt;
   }
-  if (lane == 0) {
-    U64[(size_t)j * ne + i] = u;
-    Us[(size_t)j * ne + i] = to_storage<T>(u);
-    UT64[(size_t)j * ne + i] = R;
-    UTs[(size_t)j * ne + i] = (float)R;
+  if (threadIdx.x == 0) {
+    D64[i] = 0.0;
+    DT64[i] = 0.0;
+    DTs[i] = 0.f;
   }
+}
+
+// Column i of U: x = 1/(1 + 6 e^2), y = (phi/3)(1 + 6 e^3)/(1 + e^2).  UT gets
+// the regularised time at the same point; past the apsis it follows from the
+// time symmetry of the ray about its apsis, t(phi) = 2 t_a - t(2 phi_a - phi).
+// The integrals up to kUPanels + 1 points first; then eight lanes per texel
+// invert phi inside the panel that holds it.
+constexpr int kUPanels = 256;
+
+template <typename T>
+__device__ void u_column(int ne, int nphi, int i, double *U64, T *Us, double *UT64, float *UTs, double *buf) {
+  __shared__ double phis[kUPanels + 1], times[kUPanels + 1];
+  const double x = (double)i / (ne - 1);
+  const double e2 = i == 0 ? 0.0 : (1.0 / x - 1.0) / 6.0;
+  const bool radial = i == 0, none = !radial && e2 <= 0.0;
+  __shared__ Ray ray;
+  __shared__ double span[2];  // t at u = 0 and at the apsis (low: 0) or the horizon
+  if (threadIdx.x == 0 && !radial && !none) {
+    if (e2 < kMu) {
+      ray = low_ray(1.0 - e2 / kMu, e2);
+      span[0] = ray_sinh(ray) ? asinh(ray.w1 / ray.c) : ray.w1;
+      span[1] = 0.0;
+    } else {
+      ray = high_ray(fmax(e2 - kMu, 1e-24), e2);
+      span[0] = asinh(-2.0 / 3.0 / ray.se);
+      span[1] = asinh(1.0 / 3.0 / ray.se);
+    }
+  }
+  __syncthreads();
+  const Ray r = ray;
+  const double t0 = span[0], t1 = span[1];
+  if (!radial && !none) {
+    const double step = (t1 - t0) / kUPanels;
+    static_assert(kUPanels <= kColumnThreads, "one panel per thread");
+    const int k = threadIdx.x;
+    double sp = 0.0, st = 0.0, tp, tt;
+    const double m = fma(k + 0.5, step, t0), h = 0.5 * fabs(step);
+    if (k < kUPanels) {
+#pragma unroll
+      for (int g = 0; g < kGL; ++g) {
+        double u, ud;
+        const double f = ray_rate_t(r, fma(h, cGLx[g], m), u, ud) * (cGLw[g] * h);
+        sp += f;
+        st = fma(f, newton_rcp(r.e + ud), st);
+      }
+    }
+    block_scan2(sp, st, buf, tp, tt);
+    if (k < kUPanels) {
+      phis[k + 1] = sp;
+      times[k + 1] = st;
+    }
+    if (k == 0) phis[0] = times[0] = 0.0;
+  }
+  __syncthreads();
+  const int lane8 = threadIdx.x & 7;
+  for (int j0 = 0; j0 < nphi; j0 += blockDim.x / 8) {
+    const int j = j0 + (int)(threadIdx.x >> 3);
+    const bool real = j < nphi;
+    double u = 0.0, R = 0.0;  // R = 0 where there is no ray or it was captured
+    const double y = (double)min(j, nphi - 1) / (nphi - 1);
+    if (radial) {
+      u = j == 0 ? 0.0 : 1.0;  // e -> infinity: radial ray, captured at once
+    } else if (!none) {        // the same for the whole block: its lanes stay together
+      double phi = 3.0 * y * (1.0 + e2) / (1.0 + 6.0 * e2 * r.e);
+      const double last = phis[kUPanels];
+      const bool start = phi <= 0.0;
+      const bool captured = !r.low && phi >= last;  // reached the horizon before phi (reading C7)
+      const bool past = r.low && phi > last;
+      if (past) phi = 2.0 * last - phi;  // past the apsis: reflection
+      const bool away = phi < 0.0;       // back at infinity: no texel of the mapping gets here
+      int k = 0;                         // the panel with phis[k] <= phi < phis[k + 1]
+      for (int bit = kUPanels / 2; bit > 0; bit >>= 1)
+        if (k + bit < kUPanels && phis[k + bit] <= phi) k += bit;
+      const double step = (t1 - t0) / kUPanels, ta = fma((double)k, step, t0);
+      const double p0 = phis[k], p1 = phis[k + 1];
+      double f = fmin(fmax((phi - p0) / (p1 - p0), 0.0), 1.0);  // place in the panel
+      double at, uu, rate = 1.0, rsum = 0.0;
+      // three Newton steps from the linear guess (error 1e-4 of the panel, then its
+      // square, then rounding), then the time: lanes 0-3 take the nodes, lane 4
+      // the end
+#pragma unroll 1
+      for (int it = 0; it < 4; ++it) {
+        at = fma(f, step, ta);
+        const double h = 0.5 * fabs(f * step), m = fma(0.5 * f, step, ta);
+        const double node = lane8 < kGL ? cGLx[lane8] : 0.0, wt = lane8 < kGL ? cGLw[lane8] * h : 0.0;
+        double un, ud;
+        const double g = ray_rate_t(r, lane8 < kGL ? fma(h, node, m) : at, un, ud);
+        double sum = wt * (it == 3 ? g / (r.e + ud) : g);
+        for (int o = 4; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+        rate = __shfl_sync(0xffffffffu, g, (threadIdx.x & 24) + 4);
+        uu = __shfl_sync(0xffffffffu, un, (threadIdx.x & 24) + 4);
+        if (it < 3) f = fmin(fmax(f - (p0 + sum - phi) / (rate * fabs(step)), 0.0), 1.0);
+        else rsum = sum;
+      }
+      u = uu;
+      R = times[k] + rsum;
+      if (past) {
+        const double Ra = times[kUPanels], ua = r.ap.ua;
+        R = u > 0.0 ? 2.0 * Ra - 2.0 / ua + 2.0 * log(ua / (1.0 - ua)) - R + 2.0 / u - 2.0 * log(u / (1.0 - u)) : 0.0;
+      }
+      if (captured) { u = 1.0; R = 0.0; }
+      if (start || away) u = R = 0.0;
+    }
+    if (real && lane8 == 0) {
+      const size_t o = (size_t)j * ne + i;
+      U64[o] = u;
+      Us[o] = to_storage<T>(u);
+      UT64[o] = R;
+      UTs[o] = (float)R;
+    }
+  }
+}
+
+// One block per column: U's first (they take longest), then D's.
+template <typename T>
+__global__ void __launch_bounds__(kColumnThreads, 4) precompute_kernel(int n, double *D64, double *DT64, float *DTs, int ne,
+                                                                   int nphi, double *U64, T *Us, double *UT64,
+                                                                   float *UTs) {
+  __shared__ double buf[64];
+  if ((int)blockIdx.x < ne) u_column<T>(ne, nphi, blockIdx.x, U64, Us, UT64, UTs, buf);
+  else d_column(n, blockIdx.x - ne, D64, DT64, DTs, buf);
 }
 
 // The render copy of D, row-paired: texel (j, i) holds D(j, i) and
@@ -387,10 +451,59 @@ __global__ void convert_kernel(const double *src, T *dst, size_t n) {
 // ---------------------------------------------------------------------------
 // Colour tables (Sec. 3.4.2, reading C14)
 // ---------------------------------------------------------------------------
-__global__ void cmf_kernel(double *cmf) {
-  int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k < kNLambda) dcmf(360.0 + 5.0 * k, cmf + 3 * k);
+// A black body's X, Y, Z times exp(c2/(830 nm T)) - 1 is smooth and between 0 and
+// O(1) for any T: fitted by polynomials in 1/T, from 0 to 1/960 K on 22 cells (the
+// Planckian locus, whose nearest points are decided in FP64: truncation 1e-15)
+// and to 1/64 K on 138 cells (C alone, rounded to float: 1e-11).  1,920 black
+// bodies replace 400,000 (3.5 ms) for the locus, the disc table and C.
+constexpr int kSpecFine = 22, kSpecCells = 160, kSpecNodes = 12;
+constexpr double kSpecV0 = 1.0 / 960.0, kSpecV1 = 1.0 / 64.0;  // 1/K
+constexpr double kSpecStep0 = kSpecV0 / kSpecFine, kSpecStep1 = (kSpecV1 - kSpecV0) / (kSpecCells - kSpecFine);
+constexpr int kSpecCoefs = kSpecCells * 3 * kSpecNodes;
+using SpecFit = BlackBodyFit<kSpecNodes>;
+
+// One warp per node; the last node of a cell to finish fits the cell.
+__global__ void spectrum_kernel(const SpecFit fit, double *val, unsigned *done, double *coef) {
+  const int lane = threadIdx.x, cell = blockIdx.x / kSpecNodes, node = blockIdx.x - cell * kSpecNodes;
+  const double at = 0.5 * (fit.node[node] + 1.0);
+  const double v = cell < kSpecFine ? (cell + at) * kSpecStep0 : kSpecV0 + (cell - kSpecFine + at) * kSpecStep1;  // 1/T
+  const double ref = expm1(fit.x[kNLambda - 1] * v);
+  double s[3] = {0.0, 0.0, 0.0};
+  for (int k = lane; k < kNLambda; k += 32) {
+    const double b = ref / expm1(fit.x[k] * v);
+    for (int c = 0; c < 3; ++c) s[c] = fma(b, fit.w[c][k], s[c]);
+  }
+  for (int o = 16; o > 0; o >>= 1)
+    for (int c = 0; c < 3; ++c) s[c] += __shfl_xor_sync(0xffffffffu, s[c], o);
+  unsigned before = 0;
+  if (lane == 0) {
+    for (int c = 0; c < 3; ++c) val[blockIdx.x * 3 + c] = s[c];
+    __threadfence();
+    before = atomicAdd(done + cell, 1u);
+    __threadfence();
+  }
+  if (__shfl_sync(0xffffffffu, before, 0) != kSpecNodes - 1u) return;
+  for (int k = lane; k < 3 * kSpecNodes; k += 32)
+    coef[cell * 3 * kSpecNodes + k] = fit_coefficient(fit, k % kSpecNodes, val + cell * kSpecNodes * 3 + k / kSpecNodes, 3);
 }
+
+// X, Y, Z of the black body of temperature 1/v, times exp(c2 v / 830 nm) - 1.
+__device__ __forceinline__ void spectrum_xyz(const double *coef, double v, double *g) {
+  const bool fine = v < kSpecV0;
+  const double t = fine ? v * (1.0 / kSpecStep0) : (v - kSpecV0) * (1.0 / kSpecStep1);
+  const int k = min((int)t, fine ? kSpecFine - 1 : kSpecCells - kSpecFine - 1), cell = fine ? k : kSpecFine + k;
+  const double u = fma(2.0, t - k, -1.0);
+  const double *a = coef + cell * 3 * kSpecNodes;
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    double s = a[c * kSpecNodes + kSpecNodes - 1];
+#pragma unroll
+    for (int m = kSpecNodes - 2; m >= 0; --m) s = fma(s, u, a[c * kSpecNodes + m]);
+    g[c] = s;
+  }
+}
+
+constexpr double kRefK = 1.4387769e7 / 830.0;  // c2 / 830 nm
 
 __device__ __forceinline__ void uv1960(const double *xyz, double *uv) {
   double den = __dadd_rn(__dadd_rn(xyz[0], __dmul_rn(15.0, xyz[1])), __dmul_rn(3.0, xyz[2]));
@@ -398,70 +511,106 @@ __device__ __forceinline__ void uv1960(const double *xyz, double *uv) {
   uv[1] = __ddiv_rn(__dmul_rn(6.0, xyz[1]), den);
 }
 
-__global__ void locus_kernel(const double *cmf, double *locus) {
-  int m = blockIdx.x * blockDim.x + threadIdx.x;
-  if (m >= kNLocus) return;
-  double xyz[3];
-  dblackbody_xyz(cmf, 1000.0 * pow(40.0, m / 4095.0), xyz);
-  uv1960(xyz, locus + 2 * m);
+struct Locus {
+  double2 uv[kNLocus];     // Planckian locus in CIE 1960 uv, T = 1000 40^(m/4095)
+  double2 body[kNLocus];   // 1/T, and (exp(c2/(830 nm T)) - 1) / (X+Y+Z) of the fit
+  double shift[kCnd];      // 1/D of C's layers
+  float2 uv32[kNLocus];
+};
+
+// The locus, and the disc table: ln Y, X/Y, Z/Y of B_T at log2 T = 8 + 12 (k +
+// 1/2)/n (one exponential per lookup).
+__global__ void locus_disc_kernel(const double *coef, Locus *locus, float4 *disc) {
+  const int m = blockIdx.x * blockDim.x + threadIdx.x;
+  double g[3];
+  if (m < kNLocus) {
+    const double v = 1.0 / (1000.0 * pow(40.0, m / 4095.0));
+    spectrum_xyz(coef, v, g);
+    double uv[2];
+    uv1960(g, uv);
+    locus->uv[m] = make_double2(uv[0], uv[1]);
+    locus->uv32[m] = make_float2((float)uv[0], (float)uv[1]);
+    locus->body[m] = make_double2(v, expm1(kRefK * v) / (g[0] + g[1] + g[2]));
+    if (m < kCnd) locus->shift[m] = exp2(4.0 - 8.0 * (m + 0.5) / kCnd);
+  } else if (m < kNLocus + kDiscN) {
+    const int k = m - kNLocus;
+    const double v = exp2(-(8.0 + 12.0 * (k + 0.5) / kDiscN));
+    spectrum_xyz(coef, v, g);
+    // the fit's wavelengths are in units of 560 nm
+    disc[k] = make_float4((float)(log(g[1] / expm1(kRefK * v)) - 5.0 * log(560.0)), (float)(g[0] / g[1]),
+                          (float)(g[2] / g[1]), 0.f);
+  }
 }
 
-// Nearest Planckian-locus temperature of each (x,y) cell in CIE 1960 uv.
-__global__ void cct_kernel(const double *locus, double *cct) {
-  int i = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y;
-  if (i >= kCnx || j >= kCny) return;
-  double x = 0.15 + 0.60 * (i + 0.5) / kCnx, y = 0.15 + 0.35 * (j + 0.5) / kCny;
-  double c[3] = {__ddiv_rn(x, y), 1.0, __ddiv_rn(__dadd_rn(__dadd_rn(1.0, -x), -y), y)};
+// C(xy, D) = XYZ(B_{D T}) / (X+Y+Z)(B_T), T the nearest Planckian-locus
+// temperature of the cell in CIE 1960 uv (D^5 I(D lambda) of a black body is the
+// black body at temperature D T).  One warp per (x, y) cell.  The nearest point
+// is searched in FP32; FP64 decides between the points within its error.
+__global__ void colour_cell_kernel(const Locus *locus, const double *coef, float4 *C) {
+  const int cell = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+  if (cell >= kCnx * kCny) return;  // whole warps leave together
+  const int i = cell % kCnx, j = cell / kCnx;
+  const double x = 0.15 + 0.60 * (i + 0.5) / kCnx, y = 0.15 + 0.35 * (j + 0.5) / kCny;
+  const double c[3] = {__ddiv_rn(x, y), 1.0, __ddiv_rn(__dadd_rn(__dadd_rn(1.0, -x), -y), y)};
   double uv[2];
   uv1960(c, uv);
-  int best = 0;
+  const float uf = (float)uv[0], vf = (float)uv[1];
+  auto near = [&](int m) {
+    const float2 p = locus->uv32[m];
+    const float du = uf - p.x, dv = vf - p.y;
+    return fmaf(du, du, dv * dv);
+  };
+  float least = INFINITY;
+  for (int m = lane; m < kNLocus; m += 32) least = fminf(least, near(m));
+  for (int o = 16; o > 0; o >>= 1) least = fminf(least, __shfl_xor_sync(0xffffffffu, least, o));
+  // du and dv are off by at most 1.2e-7 each
+  const float bound = fmaf(1e-6f, sqrtf(least) + least, least + 1e-12f);
   double bd = INFINITY;
-  for (int m = 0; m < kNLocus; ++m) {
-    double du = __dadd_rn(uv[0], -locus[2 * m]), dv = __dadd_rn(uv[1], -locus[2 * m + 1]);
-    double d = __dadd_rn(__dmul_rn(du, du), __dmul_rn(dv, dv));
-    if (d < bd) { bd = d; best = m; }
+  int best = kNLocus;
+  // the candidates of a lane as bits first: under a condition in this loop, the
+  // FP64 of all its steps would be issued, predicated off (146 us)
+  for (int m0 = 0; m0 < kNLocus; m0 += 1024) {
+    unsigned in = 0;
+    for (int k = 0; k < 32; ++k) in |= near(m0 + 32 * k + lane) <= bound ? 1u << k : 0u;
+    while (in) {
+      const int m = m0 + 32 * (__ffs(in) - 1) + lane;
+      in &= in - 1u;
+      const double2 p = locus->uv[m];
+      const double du = __dadd_rn(uv[0], -p.x), dv = __dadd_rn(uv[1], -p.y);
+      const double d = __dadd_rn(__dmul_rn(du, du), __dmul_rn(dv, dv));
+      if (d < bd) { bd = d; best = m; }
+    }
   }
-  cct[j * kCnx + i] = 1000.0 * pow(40.0, best / 4095.0);
-}
-
-// C(xy, D) = XYZ(B_{D T}) / (X+Y+Z)(B_T): D^5 I(D lambda) of a black body is
-// the black body at temperature D T.
-__global__ void ctable_kernel(const double *cmf, const double *cct, float4 *C) {
-  int i = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y, k = blockIdx.z;
-  if (i >= kCnx) return;
-  double T = cct[j * kCnx + i];
-  double e[3], r[3];
-  dblackbody_xyz(cmf, T, e);
-  double es = e[0] + e[1] + e[2];
-  double D = exp2(-4.0 + 8.0 * (k + 0.5) / kCnd);
-  dblackbody_xyz(cmf, D * T, r);
-  C[((size_t)k * kCny + j) * kCnx + i] =
-      make_float4((float)(r[0] / es), (float)(r[1] / es), (float)(r[2] / es), 0.f);
-}
-
-// Disc table: ln Y, X/Y, Z/Y of B_T at log2 T = 8 + 12 (k + 1/2)/n (one
-// exponential per lookup).
-__global__ void disc_table_kernel(const double *cmf, float4 *out) {
-  int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= kDiscN) return;
-  double xyz[3];
-  dblackbody_xyz(cmf, exp2(8.0 + 12.0 * (k + 0.5) / kDiscN), xyz);
-  out[k] = make_float4((float)log(xyz[1]), (float)(xyz[0] / xyz[1]), (float)(xyz[2] / xyz[1]), 0.f);
+  for (int o = 16; o > 0; o >>= 1) {
+    const double d = __shfl_xor_sync(0xffffffffu, bd, o);
+    const int m = __shfl_xor_sync(0xffffffffu, best, o);
+    if (d < bd || (d == bd && m < best)) { bd = d; best = m; }
+  }
+  const double2 body = locus->body[best];
+  for (int k = lane; k < kCnd; k += 32) {
+    const double vk = body.x * locus->shift[k];
+    double r[3];
+    spectrum_xyz(coef, vk, r);
+    const double f = body.y / expm1(kRefK * vk);
+    C[((size_t)k * kCny + j) * kCnx + i] = make_float4((float)(r[0] * f), (float)(r[1] * f), (float)(r[2] * f), 0.f);
+  }
 }
 
 bh_status colour_tables_launch(bh_ctx *ctx, bh_tables *t, cudaStream_t s) {
-  double *scratch = nullptr;
-  size_t n = 3 * kNLambda + 2 * kNLocus + kCnx * kCny;
-  BH_CUDA(cudaMallocAsync((void **)&scratch, n * sizeof(double), s));
-  double *cmf = scratch, *locus = scratch + 3 * kNLambda, *cct = locus + 2 * kNLocus;
-  cmf_kernel<<<1, 128, 0, s>>>(cmf);
-  locus_kernel<<<(kNLocus + 127) / 128, 128, 0, s>>>(cmf, locus);
-  cct_kernel<<<dim3(1, kCny), kCnx, 0, s>>>(locus, cct);
-  ctable_kernel<<<dim3(1, kCny, kCnd), kCnx, 0, s>>>(cmf, cct, t->C);
-  disc_table_kernel<<<(kDiscN + 127) / 128, 128, 0, s>>>(cmf, t->disc);
-  count_launch(ctx, 5);
+  struct Scratch {
+    Locus locus;
+    double coef[kSpecCoefs], val[kSpecCells * kSpecNodes * 3];
+    unsigned done[kSpecCells];
+  };
+  Scratch *w = nullptr;
+  BH_CUDA(cudaMallocAsync((void **)&w, sizeof(Scratch), s));
+  BH_CUDA(cudaMemsetAsync(w->done, 0, sizeof w->done, s));
+  spectrum_kernel<<<kSpecCells * kSpecNodes, 32, 0, s>>>(black_body_fit<kSpecNodes>(), w->val, w->done, w->coef);
+  locus_disc_kernel<<<(kNLocus + kDiscN) / 64, 64, 0, s>>>(w->coef, &w->locus, t->disc);
+  colour_cell_kernel<<<kCnx * kCny / 4, 128, 0, s>>>(&w->locus, w->coef, t->C);
+  count_launch(ctx, 3);
   BH_CUDA(cudaGetLastError());
-  BH_CUDA(cudaFreeAsync(scratch, s));
+  BH_CUDA(cudaFreeAsync(w, s));
   return BH_OK;
 }
 
@@ -605,20 +754,19 @@ extern "C" bh_status bh_precompute_tables(bh_ctx *ctx, const bh_table_desc *desc
   bh_tables *t = nullptr;
   bh_status st = tables_alloc(ctx, desc, s, &t);
   if (st) return st;
-  int n = desc->d_n;
-  dim3 gd((n + 127) / 128, n);
-  unsigned gu = (unsigned)((desc->u_ne * desc->u_nphi + 3) / 4);  // 4 warps (texels) per block
-  precompute_D_kernel<<<gd, 128, 0, s>>>(n, t->D64, t->DT64, t->DT);
+  const int n = desc->d_n;
+  const dim3 gd((n + 127) / 128, n);
+  const unsigned columns = (unsigned)(n + desc->u_ne);
   if (desc->storage == BH_F32) {
+    precompute_kernel<float><<<columns, kColumnThreads, 0, s>>>(n, t->D64, t->DT64, t->DT, desc->u_ne, desc->u_nphi,
+                                                               t->U64, (float *)t->U, t->UT64, t->UT);
     pair_d_kernel<float><<<gd, 128, 0, s>>>(n, t->D64, (float *)t->D);
-    precompute_U_kernel<float><<<gu, 128, 0, s>>>(desc->u_ne, desc->u_nphi, t->U64, (float *)t->U, t->UT64,
-                                                 t->UT);
   } else {
+    precompute_kernel<__half><<<columns, kColumnThreads, 0, s>>>(n, t->D64, t->DT64, t->DT, desc->u_ne, desc->u_nphi,
+                                                                t->U64, (__half *)t->U, t->UT64, t->UT);
     pair_d_kernel<__half><<<gd, 128, 0, s>>>(n, t->D64, (__half *)t->D);
-    precompute_U_kernel<__half><<<gu, 128, 0, s>>>(desc->u_ne, desc->u_nphi, t->U64, (__half *)t->U, t->UT64,
-                                                  t->UT);
   }
-  count_launch(ctx, 3);
+  count_launch(ctx, 2);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) { bh_tables_free(t); return cuda_fail(e, "precompute launch"); }
   st = colour_tables_launch(ctx, t, s);

@@ -56,54 +56,7 @@ constexpr double kChromaTMin = 1024.0, kChromaTMax = 1e9;
 constexpr int kChromaStride = 2 * kChromaNodes + 2;  // X and Z coefficients, minus twice the cell's centre, pad
 constexpr int kChromaCoefs = kChromaCells * kChromaStride, kChromaVals = kChromaCells * kChromaNodes * 2;
 
-// Everything of the fit that does not depend on the cell: computed once on the
-// host, a kernel parameter.
-struct ChromaFit {
-  double node[kChromaNodes];                // Chebyshev nodes on [-1, 1]
-  // values at the nodes -> monomial coefficients, as sums of two doubles: their
-  // terms cancel to a thousandth
-  double inv[kChromaNodes][kChromaNodes], inv_lo[kChromaNodes][kChromaNodes];
-  double x[kNLambda];                       // c2 / lambda (K)
-  double cmf[3][kNLambda];                  // matching functions
-  double w[3][kNLambda];                    // ... times the trapezoid weight over (lambda / 560 nm)^5
-};
-
-static const ChromaFit &chroma_fit() {
-  static const ChromaFit fit = [] {
-    ChromaFit f = {};
-    constexpr int n = kChromaNodes;
-    const long double pi = 3.14159265358979323846264338327950288L;
-    double mono[n][n] = {};  // mono[j][m]: coefficient of u^m in the Chebyshev polynomial T_j
-    mono[0][0] = 1.0;
-    mono[1][1] = 1.0;
-    for (int j = 2; j < n; ++j)
-      for (int m = 0; m < n; ++m) mono[j][m] = (m > 0 ? 2.0 * mono[j - 1][m - 1] : 0.0) - mono[j - 2][m];
-    for (int k = 0; k < n; ++k) {
-      f.node[k] = (double)cosl(pi * (k + 0.5L) / n);
-      for (int m = 0; m < n; ++m) {
-        long double s = 0.0L;
-        for (int j = 0; j < n; ++j) s += mono[j][m] * (j == 0 ? 1.0L : 2.0L) / n * cosl(j * pi * (k + 0.5L) / n);
-        f.inv[m][k] = (double)s;
-        f.inv_lo[m][k] = (double)(s - f.inv[m][k]);
-      }
-    }
-    auto lobe = [](double l, double m, double s1, double s2) {
-      const double t = (l - m) / (l < m ? s1 : s2);
-      return exp(-0.5 * t * t);
-    };
-    for (int k = 0; k < kNLambda; ++k) {  // the observer of dcmf
-      const double l = 360.0 + 5.0 * k, r = l / 560.0, t = (k == 0 || k == kNLambda - 1 ? 2.5 : 5.0) / (r * r * r * r * r);
-      f.x[k] = 1.4387769e7 / l;
-      f.cmf[0][k] = 1.056 * lobe(l, 599.8, 37.9, 31.0) + 0.362 * lobe(l, 442.0, 16.0, 26.7) -
-                    0.065 * lobe(l, 501.1, 20.4, 26.2);
-      f.cmf[1][k] = 0.821 * lobe(l, 568.8, 46.9, 40.5) + 0.286 * lobe(l, 530.9, 16.3, 31.1);
-      f.cmf[2][k] = 1.217 * lobe(l, 437.0, 11.8, 36.0) + 0.681 * lobe(l, 459.0, 26.0, 13.8);
-      for (int c = 0; c < 3; ++c) f.w[c][k] = t * f.cmf[c][k];
-    }
-    return f;
-  }();
-  return fit;
-}
+using ChromaFit = BlackBodyFit<kChromaNodes>;
 
 // One warp (a block of its own: 576 of them spread over the SMs) per node, 45
 // FP64 operations per wavelength, whose constants come from the host; the last
@@ -137,14 +90,7 @@ __global__ void chroma_kernel(const ChromaFit fit, double *cmf_out, double *val,
   double *out = coef + cell * kChromaStride;
   if (lane < 2 * kChromaNodes) {
     const int c = lane / kChromaNodes, m = lane - c * kChromaNodes;
-    double a = 0.0, err = 0.0;  // the sum and what its roundings lost
-    for (int k = 0; k < kChromaNodes; ++k) {
-      const double f = __ldcg(val + (cell * kChromaNodes + k) * 2 + c);
-      const double p = fit.inv[m][k] * f, t = a + p, z = t - a;
-      err += ((a - (t - z)) + (p - z)) + (fma(fit.inv[m][k], f, -p) + fit.inv_lo[m][k] * f);
-      a = t;
-    }
-    out[lane] = a + err;
+    out[lane] = fit_coefficient(fit, m, val + cell * kChromaNodes * 2 + c, 2);
   } else if (lane == 2 * kChromaNodes) {
     out[lane] = -(2.0 * cell + 1.0);
   }
@@ -152,7 +98,7 @@ __global__ void chroma_kernel(const ChromaFit fit, double *cmf_out, double *val,
 
 // val: kChromaVals doubles of scratch; done: kChromaCells counters, zero.
 static void chroma_launch(double *cmf, double *val, unsigned *done, double *coef, cudaStream_t s) {
-  chroma_kernel<<<kChromaCells * kChromaNodes + 1, 32, 0, s>>>(chroma_fit(), cmf, val, done, coef);
+  chroma_kernel<<<kChromaCells * kChromaNodes + 1, 32, 0, s>>>(black_body_fit<kChromaNodes>(), cmf, val, done, coef);
 }
 
 // 1/b by Newton's iteration from the float reciprocal (b a normal float whose
