@@ -14,6 +14,9 @@
  *  - Handles (bh_ctx, bh_tables, bh_cubemap) are owned by the library and
  *    released by their _free / bh_destroy call.  Image buffers are owned by
  *    the caller.
+ *  - A context keeps up to 512 MiB of the device memory of freed tables, cube
+ *    maps and build scratch for the next ones; bh_destroy gives it back, and so
+ *    does an allocation of the context that would fail otherwise.
  *  - "device" pointers are CUDA device pointers of the context's device;
  *    "host" pointers are ordinary (preferably pinned) host memory.
  *  - Streams are passed as void* holding a cudaStream_t (NULL = the legacy
@@ -199,7 +202,7 @@ typedef struct {
  * stars: host array (stars_on_device = 0) or device array (1).  Enqueued on
  * `stream` (a host star list is staged synchronously first).  Uses
  * 48 bytes of scratch per star -- where that is more than 1 GiB, at most
- * 240 * face_size^2 bytes --, freed before return. */
+ * 240 * face_size^2 bytes --, given back before return. */
 bh_status bh_build_star_cubemap(bh_ctx *ctx, const bh_star *stars, long long n, int face_size,
                                 bh_dtype storage, int stars_on_device, void *stream,
                                 bh_cubemap **out);

@@ -52,6 +52,84 @@ bh_status cuda_fail(cudaError_t e, const char *what) {
 
 void count_launch(bh_ctx *ctx, int n) { ctx->launches.fetch_add(n, std::memory_order_relaxed); }
 
+static void pool_release(bh_ctx *ctx) {  // pool_mu held
+  for (PoolBlock &b : ctx->pool) {
+    if (b.ready) {
+      cudaEventSynchronize(b.ready);
+      cudaEventDestroy(b.ready);
+    }
+    cudaFree(b.p);
+  }
+  ctx->pool.clear();
+  ctx->pool_bytes = 0;
+}
+
+cudaError_t pool_get(bh_ctx *ctx, size_t bytes, cudaStream_t s, PoolBlock *out) {
+  std::lock_guard<std::mutex> lk(ctx->pool_mu);
+  int best = -1;  // the smallest that fits and wastes less than its half
+  for (int k = 0; k < (int)ctx->pool.size(); ++k) {
+    const size_t have = ctx->pool[k].bytes;
+    if (have >= bytes && have / 2 <= bytes && (best < 0 || have < ctx->pool[best].bytes)) best = k;
+  }
+  if (best >= 0) {
+    PoolBlock b = ctx->pool[best];
+    if (b.ready) {
+      const cudaError_t e = cudaStreamWaitEvent(s, b.ready, 0);
+      if (e != cudaSuccess) return e;
+      cudaEventDestroy(b.ready);  // takes effect once the event has completed
+      b.ready = nullptr;
+    }
+    ctx->pool.erase(ctx->pool.begin() + best);
+    ctx->pool_bytes -= b.bytes;
+    *out = b;
+    return cudaSuccess;
+  }
+  PoolBlock b;
+  b.bytes = bytes;
+  cudaError_t e = cudaMalloc(&b.p, bytes);
+  if (e == cudaErrorMemoryAllocation && !ctx->pool.empty()) {
+    cudaGetLastError();
+    pool_release(ctx);
+    e = cudaMalloc(&b.p, bytes);
+  }
+  if (e == cudaSuccess) *out = b;
+  return e;
+}
+
+static void pool_keep(bh_ctx *ctx, PoolBlock b) {  // b.ready behind its last use, or idle
+  {
+    std::lock_guard<std::mutex> lk(ctx->pool_mu);
+    if (ctx->pool_bytes + b.bytes <= kPoolBytes) {
+      ctx->pool.push_back(b);
+      ctx->pool_bytes += b.bytes;
+      return;
+    }
+  }
+  if (b.ready) {
+    cudaEventSynchronize(b.ready);
+    cudaEventDestroy(b.ready);
+  }
+  cudaFree(b.p);
+}
+
+void pool_put(bh_ctx *ctx, PoolBlock b, cudaStream_t s) {
+  if (!b.p) return;
+  b.ready = nullptr;
+  if (cudaEventCreateWithFlags(&b.ready, cudaEventDisableTiming) != cudaSuccess || cudaEventRecord(b.ready, s) != cudaSuccess) {
+    if (b.ready) cudaEventDestroy(b.ready);
+    b.ready = nullptr;
+    cudaFree(b.p);  // waits for the device
+    return;
+  }
+  pool_keep(ctx, b);
+}
+
+void pool_put_idle(bh_ctx *ctx, PoolBlock b) {
+  if (!b.p) return;
+  b.ready = nullptr;
+  pool_keep(ctx, b);
+}
+
 bh_status check_status(bh_ctx *ctx, cudaStream_t s) {
   unsigned st = 0;
   BH_CUDA(cudaMemcpyAsync(&st, ctx->status_dev, sizeof st, cudaMemcpyDeviceToHost, s));
@@ -602,16 +680,17 @@ bh_status colour_tables_launch(bh_ctx *ctx, bh_tables *t, cudaStream_t s) {
     double coef[kSpecCoefs], val[kSpecCells * kSpecNodes * 3];
     unsigned done[kSpecCells];
   };
-  Scratch *w = nullptr;
-  BH_CUDA(cudaMallocAsync((void **)&w, sizeof(Scratch), s));
-  BH_CUDA(cudaMemsetAsync(w->done, 0, sizeof w->done, s));
+  PoolBlock mem;
+  BH_CUDA(pool_get(ctx, sizeof(Scratch), s, &mem));
+  Scratch *w = static_cast<Scratch *>(mem.p);
+  cudaError_t e = cudaMemsetAsync(w->done, 0, sizeof w->done, s);
   spectrum_kernel<<<kSpecCells * kSpecNodes, 32, 0, s>>>(black_body_fit<kSpecNodes>(), w->val, w->done, w->coef);
   locus_disc_kernel<<<(kNLocus + kDiscN) / 64, 64, 0, s>>>(w->coef, &w->locus, t->disc);
   colour_cell_kernel<<<kCnx * kCny / 4, 128, 0, s>>>(&w->locus, w->coef, t->C);
   count_launch(ctx, 3);
-  BH_CUDA(cudaGetLastError());
-  BH_CUDA(cudaFreeAsync(w, s));
-  return BH_OK;
+  if (e == cudaSuccess) e = cudaGetLastError();
+  pool_put(ctx, mem, s);
+  return e == cudaSuccess ? BH_OK : cuda_fail(e, "colour tables");
 }
 
 }  // namespace bh
@@ -676,6 +755,10 @@ extern "C" void bh_destroy(bh_ctx *c) {
   bh::serve_destroy(c);
   cudaDeviceSynchronize();
   c->graph.reset();
+  {
+    std::lock_guard<std::mutex> lk(c->pool_mu);
+    bh::pool_release(c);
+  }
   if (c->status_dev) cudaFree(c->status_dev);
   if (c->sched_dev) cudaFree(c->sched_dev);
   if (c->aux) cudaStreamDestroy(c->aux);
@@ -723,22 +806,33 @@ static bh_status tables_alloc(bh_ctx *ctx, const bh_table_desc *desc, cudaStream
   t->ctx = ctx;
   t->desc = *desc;
   size_t nd = (size_t)desc->d_n * desc->d_n, nu = (size_t)desc->u_ne * desc->u_nphi;
-  size_t es = desc->storage == BH_F32 ? 4 : 2;
-  cudaError_t e = cudaMalloc((void **)&t->D64, nd * 8);
-  if (e == cudaSuccess) e = cudaMalloc((void **)&t->U64, nu * 8);
-  if (e == cudaSuccess) e = cudaMalloc(&t->D, 2 * nd * es);  // row-paired render copy
-  if (e == cudaSuccess) e = cudaMalloc(&t->U, ((nu * es + 15) / 16) * 16);
-  if (e == cudaSuccess) e = cudaMalloc((void **)&t->DT64, nd * 8);
-  if (e == cudaSuccess) e = cudaMalloc((void **)&t->UT64, nu * 8);
-  if (e == cudaSuccess) e = cudaMalloc((void **)&t->DT, nd * 4);
-  if (e == cudaSuccess) e = cudaMalloc((void **)&t->UT, nu * 4);
-  if (e == cudaSuccess) e = cudaMalloc((void **)&t->C, sizeof(float4) * kCnx * kCny * kCnd);
-  if (e == cudaSuccess) e = cudaMalloc((void **)&t->disc, sizeof(float4) * kDiscN);
+  const size_t es = desc->storage == BH_F32 ? 4 : 2;
+  // one allocation, every array on a 256-byte line
+  size_t bytes = 0;
+  auto place = [&](size_t b) {
+    const size_t at = bytes;
+    bytes += (b + 255) / 256 * 256;
+    return at;
+  };
+  const size_t o_D64 = place(nd * 8), o_U64 = place(nu * 8), o_D = place(2 * nd * es) /* row-paired render copy */,
+               o_U = place(nu * es), o_DT64 = place(nd * 8), o_UT64 = place(nu * 8), o_DT = place(nd * 4),
+               o_UT = place(nu * 4), o_C = place(sizeof(float4) * kCnx * kCny * kCnd), o_disc = place(sizeof(float4) * kDiscN);
+  const cudaError_t e = pool_get(ctx, bytes, s, &t->mem);
   if (e != cudaSuccess) {
-    bh_tables_free(t);
+    delete t;
     return cuda_fail(e, "table allocation");
   }
-  (void)s;
+  char *p = static_cast<char *>(t->mem.p);
+  t->D64 = reinterpret_cast<double *>(p + o_D64);
+  t->U64 = reinterpret_cast<double *>(p + o_U64);
+  t->D = p + o_D;
+  t->U = p + o_U;
+  t->DT64 = reinterpret_cast<double *>(p + o_DT64);
+  t->UT64 = reinterpret_cast<double *>(p + o_UT64);
+  t->DT = reinterpret_cast<float *>(p + o_DT);
+  t->UT = reinterpret_cast<float *>(p + o_UT);
+  t->C = reinterpret_cast<float4 *>(p + o_C);
+  t->disc = reinterpret_cast<float4 *>(p + o_disc);
   *out = t;
   return BH_OK;
 }
@@ -776,8 +870,8 @@ extern "C" bh_status bh_precompute_tables(bh_ctx *ctx, const bh_table_desc *desc
 }
 
 namespace bh {
-bh_status tables_alloc_public(bh_ctx *ctx, const bh_table_desc *desc, bh_tables **out) {
-  return tables_alloc(ctx, desc, nullptr, out);
+bh_status tables_alloc_public(bh_ctx *ctx, const bh_table_desc *desc, cudaStream_t s, bh_tables **out) {
+  return tables_alloc(ctx, desc, s, out);
 }
 
 // Storage copies of D and U (the table's storage type) and FP32 copies of the
@@ -890,15 +984,6 @@ extern "C" void bh_tables_free(bh_tables *t) {
   if (!t) return;
   cudaSetDevice(t->ctx->device);
   cudaDeviceSynchronize();
-  cudaFree(t->D64);
-  cudaFree(t->U64);
-  cudaFree(t->D);
-  cudaFree(t->U);
-  cudaFree(t->DT64);
-  cudaFree(t->UT64);
-  cudaFree(t->DT);
-  cudaFree(t->UT);
-  cudaFree(t->C);
-  cudaFree(t->disc);
+  pool_put_idle(t->ctx, t->mem);
   delete t;
 }

@@ -817,7 +817,7 @@ extern "C" bh_status bh_build_star_cubemap(bh_ctx *ctx, const bh_star *stars, lo
   BH_CUDA(cudaSetDevice(ctx->device));
   cudaStream_t s = (cudaStream_t)stream;
   bh_cubemap *c = nullptr;
-  bh_status st = cubemap_alloc_public(ctx, N, storage, &c);
+  bh_status st = cubemap_alloc_public(ctx, N, storage, s, &c);
   if (st) return st;
   // Scratch, one allocation: counters (cleared), offsets, colour fit, stage
   // nodes, then the sorted stars -- or, where those would take more than the
@@ -833,8 +833,9 @@ extern "C" bh_status bh_build_star_cubemap(bh_ctx *ctx, const bh_star *stars, lo
   const size_t b_fit = up16(sizeof(double) * (3 * kNLambda + kChromaCoefs + kChromaVals)), b_nodes = sizeof(Node) * n_nodes;
   const size_t b_stars = sort ? sorted : 0, b_copy = n > 0 && !on_device ? up16(sizeof(bh_star) * (size_t)n) : 0;
   const size_t cleared = b_arrived + b_count + b_acc;
-  unsigned char *scratch = nullptr;
-  cudaError_t e = cudaMallocAsync((void **)&scratch, cleared + b_span + b_fit + b_nodes + b_stars + b_copy, s);
+  PoolBlock mem;
+  cudaError_t e = pool_get(ctx, cleared + b_span + b_fit + b_nodes + b_stars + b_copy, s, &mem);
+  unsigned char *scratch = static_cast<unsigned char *>(mem.p);
   if (e != cudaSuccess) {
     bh_cubemap_free(c);
     return cuda_fail(e, "bh_build_star_cubemap");
@@ -883,7 +884,7 @@ extern "C" bh_status bh_build_star_cubemap(bh_ctx *ctx, const bh_star *stars, lo
     occupancy_launch(ctx, c, N >= kRegion ? 3 : 0, s);
     e = cudaGetLastError();
   }
-  cudaFreeAsync(scratch, s);
+  pool_put(ctx, mem, s);
   if (e != cudaSuccess) {
     bh_cubemap_free(c);
     return cuda_fail(e, "bh_build_star_cubemap");
@@ -907,22 +908,21 @@ extern "C" bh_status bh_cubemap_copy_out(const bh_cubemap *c, uint16_t *h, long 
 namespace bh {
 // An empty map of face size N (all levels and the occupancy mask allocated,
 // contents undefined), for loading from a checkpoint.
-bh_status cubemap_alloc_public(bh_ctx *ctx, int N, bh_dtype storage, bh_cubemap **out) {
+bh_status cubemap_alloc_public(bh_ctx *ctx, int N, bh_dtype storage, cudaStream_t s, bh_cubemap **out) {
   bh_cubemap *c = new bh_cubemap();
   c->ctx = ctx;
   c->n = N;
   c->levels = cube_levels(N);
   c->storage = storage;
   c->records = bh_cubemap_records(N);
-  const size_t mask_bytes = sizeof(uint2) * mask_level_offset(N, c->levels);
-  cudaError_t e = cudaMalloc((void **)&c->rec, sizeof(uint2) * c->records);
-  if (e == cudaSuccess) e = cudaMalloc((void **)&c->mask, mask_bytes);
+  const size_t rec_bytes = (sizeof(uint2) * c->records + 255) / 256 * 256;
+  const cudaError_t e = pool_get(ctx, rec_bytes + sizeof(uint2) * mask_level_offset(N, c->levels), s, &c->mem);
   if (e != cudaSuccess) {
-    cudaFree(c->rec);
-    cudaFree(c->mask);
     delete c;
     return cuda_fail(e, "cube map allocation");
   }
+  c->rec = static_cast<uint2 *>(c->mem.p);
+  c->mask = reinterpret_cast<uint2 *>(static_cast<char *>(c->mem.p) + rec_bytes);
   *out = c;
   return BH_OK;
 }
@@ -932,8 +932,7 @@ extern "C" void bh_cubemap_free(bh_cubemap *c) {
   if (!c) return;
   cudaSetDevice(c->ctx->device);
   cudaDeviceSynchronize();
-  cudaFree(c->rec);
-  cudaFree(c->mask);
+  pool_put_idle(c->ctx, c->mem);
   delete c;
 }
 

@@ -15,7 +15,7 @@
 
 namespace bh {
 
-bh_status tables_alloc_public(bh_ctx *ctx, const bh_table_desc *desc, bh_tables **out);
+bh_status tables_alloc_public(bh_ctx *ctx, const bh_table_desc *desc, cudaStream_t s, bh_tables **out);
 bh_status tables_convert_storage(bh_ctx *ctx, bh_tables *t, cudaStream_t s);
 
 namespace {
@@ -207,7 +207,7 @@ extern "C" bh_status bh_tables_load(bh_ctx *ctx, const char *path, void *stream,
   BH_CUDA(cudaSetDevice(ctx->device));
   cudaStream_t s = (cudaStream_t)stream;
   bh_tables *t = nullptr;
-  bh_status st = tables_alloc_public(ctx, &desc, &t);
+  bh_status st = tables_alloc_public(ctx, &desc, s, &t);
   if (st) return st;
   cudaError_t e = cudaMemcpyAsync(t->D64, D, nd * 8, cudaMemcpyHostToDevice, s);
   if (e == cudaSuccess) e = cudaMemcpyAsync(t->U64, U, nu * 8, cudaMemcpyHostToDevice, s);
@@ -285,7 +285,7 @@ extern "C" bh_status bh_cubemap_load(bh_ctx *ctx, const char *path, void *stream
   BH_CUDA(cudaSetDevice(ctx->device));
   cudaStream_t s = (cudaStream_t)stream;
   bh_cubemap *c = nullptr;
-  bh_status st = cubemap_alloc_public(ctx, N, storage, &c);
+  bh_status st = cubemap_alloc_public(ctx, N, storage, s, &c);
   if (st) return st;
   cudaError_t e = cudaMemcpyAsync(c->rec, rec, (size_t)records * sizeof(uint2), cudaMemcpyHostToDevice, s);
   if (e == cudaSuccess) {

@@ -193,6 +193,56 @@ def test_cubemap_uneven_stars_bit_exact(ctx, orc, N, dtype):
         assert np.array_equal(own.cpu().numpy().view(np.uint16), rec)
 
 
+def test_memory_kept_by_a_context_is_bounded_and_given_back():
+    """Maps and tables built and freed over and over, from two threads on streams
+    of their own: every result is that of a fresh context, at most 512 MiB stay
+    with the context, and bh_destroy gives them back."""
+    from concurrent.futures import ThreadPoolExecutor
+    fields = [(synth.stars(n, n), face) for n, face in ((3000, 64), (500, 1024), (20000, 256), (900, 2048))]
+
+    def records(c, k, stream):
+        cube = bh.bh_build_star_cubemap(c, fields[k][0], fields[k][1], 1, stream)
+        try:
+            return bh.bh_cubemap_copy_out(cube, fields[k][1])
+        finally:
+            bh.bh_cubemap_free(cube)
+
+    expect = []
+    for k in range(len(fields)):
+        c = bh.bh_create(0, 0)
+        expect.append(records(c, k, None))
+        bh.bh_destroy(c)
+    c = bh.bh_create(0, 0)
+    first = bh.bh_precompute_tables(c, 66, 10, 6, bh.BH_F32)
+    tables = bh.bh_tables_copy_out(first, 66, 10, 6)
+    bh.bh_tables_free(first)
+    bh.bh_destroy(c)
+
+    def work(c, seed, stream):
+        rng = np.random.default_rng(seed)
+        for _ in range(12):
+            k = int(rng.integers(len(fields)))
+            assert np.array_equal(records(c, k, stream), expect[k])
+            t = bh.bh_precompute_tables(c, 66, 10, 6, bh.BH_F32, stream)
+            stream.synchronize()
+            assert all(np.array_equal(a, b) for a, b in zip(bh.bh_tables_copy_out(t, 66, 10, 6), tables))
+            bh.bh_tables_free(t)
+
+    # twice: what the driver itself allocates for streams and kernels (once) is not measured
+    streams = [torch.cuda.Stream() for _ in range(2)]
+    with ThreadPoolExecutor(2) as ex:
+        for again in (False, True):
+            free0 = torch.cuda.mem_get_info()[0]
+            c = bh.bh_create(0, 0)
+            list(ex.map(work, (c, c), (1, 2), streams))
+            torch.cuda.synchronize()
+            kept = free0 - torch.cuda.mem_get_info()[0]
+            bh.bh_destroy(c)
+            if again:
+                assert kept <= (512 << 20) + (64 << 20)
+                assert torch.cuda.mem_get_info()[0] >= free0 - (64 << 20)
+
+
 def test_cubemap_from_device_stars(ctx, orc):
     st = synth.stars(4000, seed=12)
     dst = torch.from_numpy(st).cuda()
