@@ -41,23 +41,13 @@ constexpr int kBloomTile = 64;                      // output texels per tile si
 constexpr int kBloomHalo = 3;                       // blur radius
 constexpr int kBloomSpan = kBloomTile + 2 * kBloomHalo;
 constexpr int kBloomThreads = 1024;
-// composite tiles: per level at most ceil((kCompH - 1) 2^-k) + 2 staged texel rows of kCompW entries
-constexpr int kCompW = 256, kCompH = 32;
-constexpr int comp_rows() {
-  int n = 0;
-  for (int k = 1; k <= kBloomMaxLevels; ++k) n += ((kCompH - 1) + (1 << k) - 1) / (1 << k) + 2;
-  return n;
-}
 // shared-memory row strides, padded so that lanes on consecutive rows of sD
 // or sH address distinct 16-byte bank groups
 constexpr int kSDStride = kBloomSpan + 1, kSHStride = kBloomTile + 1;
 constexpr int kBlurRun = 8;  // consecutive outputs per thread in each blur pass (a sliding window of taps)
 constexpr size_t kBlurSmem = sizeof(float4) * (kBloomSpan * kSDStride + kBloomSpan * kSHStride);
-constexpr size_t kCompSmem = sizeof(float4) * kCompW * comp_rows();
-constexpr size_t kBloomSmem = kBlurSmem > kCompSmem ? kBlurSmem : kCompSmem;
-// with the composite's per-row tables (2 x kCompH x kBloomMaxLevels words) and
-// the barrier flag in static shared memory
-static_assert(kBloomSmem + 2 * 4 * kCompH * kBloomMaxLevels + 16 <= 227 * 1024, "bloom shared memory");
+constexpr size_t kBloomSmem = kBlurSmem;
+static_assert(kBloomSmem + 64 <= 227 * 1024, "bloom shared memory");
 
 struct BloomParams {
   const float4 *in;
@@ -105,20 +95,6 @@ __device__ bool grid_barrier(const BloomParams &P, unsigned phase) {
   return ok != 0;
 }
 
-// Pull the frame rows of composite tile `tile` into L2 (one bulk prefetch per
-// pixel row, issued by the lanes of warp 0): the composite of that tile then
-// finds them there.  Rows start 16-byte aligned and span whole pixels.
-__device__ __forceinline__ void prefetch_comp_tile(const BloomParams &P, int tile, int kw, int kh) {
-  const int W = P.w[0], H = P.h[0];
-  const int tcx = (W + kw - 1) / kw, ntiles = tcx * ((H + kh - 1) / kh);
-  if (threadIdx.x >= 32 || tile >= ntiles) return;
-  const int X0 = (tile % tcx) * kw, y = (tile / tcx) * kh + (int)threadIdx.x;
-  if ((int)threadIdx.x >= kh || y >= H) return;
-  const float4 *src = P.in + ((size_t)y * W + X0);
-  const unsigned bytes = (unsigned)(sizeof(float4) * min(kw, W - X0));
-  asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(src), "r"(bytes) : "memory");
-}
-
 // Pull the frame rows that region `reg` reads (its level-1 texels with their
 // 3-texel halo: 140 x 140 pixels, clamped to the frame) into L2, one bulk
 // prefetch per pixel row.
@@ -161,16 +137,58 @@ constexpr int kBloomRegionLevels = 7;
 // whose box texels, with a 3-texel halo at clamped coordinates, are in sD.
 __device__ void blur_staged(const BloomParams &P, int k, int x0, int y0, const float4 *sD, float4 *sH);
 
-// The same, the box texels read from level k in global memory.
-__device__ void blur_tile(const BloomParams &P, int k, int x0, int y0, float4 *sD, float4 *sH) {
-  const int w = P.w[k], h = P.h[k];
-  const float4 *Dk = P.D[k];
-  for (int i = threadIdx.x; i < kBloomSpan * kBloomSpan; i += blockDim.x) {
-    const int r = i / kBloomSpan, c = i - r * kBloomSpan;
-    const int x = min(max(x0 + c - kBloomHalo, 0), w - 1), y = min(max(y0 + r - kBloomHalo, 0), h - 1);
-    sD[r * kSDStride + c] = Dk[(size_t)y * w + x];
+// The blur of levels 2 and up (a twelfth of the frame's texels in all), straight
+// from L2: two outputs of a column per thread, eight rows of seven texels each,
+// in the order of blur_staged's sums.  Tiles staged in shared memory kept 58 of
+// the 152 blocks busy with three barriers each (12 us at 1080p).
+__device__ void blur_upper(const BloomParams &P) {
+  long long before[kBloomMaxLevels + 2];
+  before[2] = 0;
+#pragma unroll
+  for (int k = 2; k <= kBloomMaxLevels; ++k) before[k + 1] = before[k] + (k <= P.n ? (long long)P.w[k] * ((P.h[k] + 1) / 2) : 0);
+  for (long long it = (long long)blockIdx.x * blockDim.x + threadIdx.x; it < before[P.n + 1];
+       it += (long long)gridDim.x * blockDim.x) {
+    int k = 2;
+#pragma unroll
+    for (int l = 3; l <= kBloomMaxLevels; ++l)
+      if (l <= P.n && it >= before[l]) k = l;
+    const int w = P.w[k], h = P.h[k];
+    long long first = 0;
+#pragma unroll
+    for (int l = 3; l <= kBloomMaxLevels; ++l)
+      if (l == k) first = before[l];
+    const int rest = (int)(it - first), y = rest / w * 2, x = rest - (y >> 1) * w;
+    const float4 *Dk = P.D[k];
+    int xs[2 * kBloomHalo + 1];
+#pragma unroll
+    for (int t = -kBloomHalo; t <= kBloomHalo; ++t) xs[t + kBloomHalo] = min(max(x + t, 0), w - 1);
+    float3 acc[2] = {{0.f, 0.f, 0.f}, {0.f, 0.f, 0.f}};
+#pragma unroll
+    for (int r = -kBloomHalo; r <= kBloomHalo + 1; ++r) {
+      const float4 *row = Dk + (size_t)min(max(y + r, 0), h - 1) * w;
+      float3 s = {0.f, 0.f, 0.f};
+#pragma unroll
+      for (int t = 0; t <= 2 * kBloomHalo; ++t) {
+        const float4 v = row[xs[t]];
+        const float kt = cBloomTaps[t < kBloomHalo ? kBloomHalo - t : t - kBloomHalo];
+        s.x = fmaf(kt, v.x, s.x);
+        s.y = fmaf(kt, v.y, s.y);
+        s.z = fmaf(kt, v.z, s.z);
+      }
+#pragma unroll
+      for (int o = 0; o < 2; ++o) {
+        const int t = r - o;  // this row is tap t of output o
+        if (t >= -kBloomHalo && t <= kBloomHalo) {
+          const float kt = cBloomTaps[t < 0 ? -t : t];
+          acc[o].x = fmaf(kt, s.x, acc[o].x);
+          acc[o].y = fmaf(kt, s.y, acc[o].y);
+          acc[o].z = fmaf(kt, s.z, acc[o].z);
+        }
+      }
+    }
+    P.B[k][(size_t)y * w + x] = make_float4(acc[0].x, acc[0].y, acc[0].z, 1.f);
+    if (y + 1 < h) P.B[k][(size_t)(y + 1) * w + x] = make_float4(acc[1].x, acc[1].y, acc[1].z, 1.f);
   }
-  blur_staged(P, k, x0, y0, sD, sH);
 }
 
 __device__ void blur_staged(const BloomParams &P, int k, int x0, int y0, const float4 *sD, float4 *sH) {
@@ -237,6 +255,91 @@ __device__ void blur_staged(const BloomParams &P, int k, int x0, int y0, const f
   __syncthreads();
 }
 
+// Composite of the column x of the rows y0 .. y0 + 7 (y0 a multiple of 8):
+//   out = w_0 in + sum_k w_k bilinear(B_k).
+// The bilinear lookup of level k is a lerp along v of two lerps along u.  The
+// lerps along u of a texel row serve every pixel of the run between two texel
+// rows, and where those rows lie in an aligned run of 8 is fixed: 6, 4 and 3
+// rows at levels 1-3, two at each level above (whose rows change only at
+// multiples of 8 pixels).  So a run takes 19 pairs of texels for six levels
+// where a pixel alone would take 12 each; the sums of a pixel are added in the
+// order of its levels.  Bound by the frame's 66 MB; staging the rows in shared
+// memory for tiles of 256 x 32 pixels read 12 staged values per pixel (27 us of
+// the bloom's 57 at 1080p).
+constexpr int kCompRun = 8;
+
+struct CompLevel {
+  const float4 *B;
+  int w, h, i0, i1;
+  float tu;
+  __device__ CompLevel(const BloomParams &P, int k, int x) {
+    const float s = __int_as_float((127 - k) << 23);  // 2^-k
+    B = P.B[k];
+    w = P.w[k];
+    h = P.h[k];
+    const float u = fmaf((float)x + 0.5f, s, -0.5f), fu = floorf(u);
+    tu = u - fu;
+    i0 = min(max((int)fu, 0), w - 1);
+    i1 = min(max((int)fu + 1, 0), w - 1);
+  }
+  __device__ float3 row(int j) const {  // texel row j (clamped) at the column
+    const float4 *r = B + (size_t)min(max(j, 0), h - 1) * w;
+    const float4 a = r[i0], b = r[i1];
+    return make_float3(fmaf(tu, b.x - a.x, a.x), fmaf(tu, b.y - a.y, a.y), fmaf(tu, b.z - a.z, a.z));
+  }
+};
+
+__device__ __forceinline__ void comp_add(float3 &acc, float wk, float tv, const float3 &h0, const float3 &h1) {
+  acc.x = fmaf(wk, fmaf(tv, h1.x - h0.x, h0.x), acc.x);
+  acc.y = fmaf(wk, fmaf(tv, h1.y - h0.y, h0.y), acc.y);
+  acc.z = fmaf(wk, fmaf(tv, h1.z - h0.z, h0.z), acc.z);
+}
+
+// Level K <= 3: pixel p of the run has v = (2 p + 1) 2^-(K+1) - 1/2 texel rows
+// past y0 2^-K.
+template <int K>
+__device__ __forceinline__ void comp_low(const BloomParams &P, int x, int y0, float3 *acc) {
+  const CompLevel L(P, K, x);
+  const float wk = P.wt[K];
+  const int j0 = y0 >> K;
+  float3 h0, h1 = L.row(j0 - 1);
+#pragma unroll
+  for (int p = 0; p < kCompRun; ++p) {
+    const int num = 2 * p + 1 - (1 << K), j = num >> (K + 1);  // floor(v)
+    const float tv = (float)(num - (j << (K + 1))) / (float)(1 << (K + 1));
+    if (p == 0 || j != (num - 2) >> (K + 1)) {
+      h0 = h1;
+      h1 = L.row(j0 + j + 1);
+    }
+    comp_add(acc[p], wk, tv, h0, h1);
+  }
+}
+
+__device__ void composite_run(const BloomParams &P, int x, int y0) {
+  const int W = P.w[0], H = P.h[0];
+  const size_t at = (size_t)y0 * W + x;
+  float3 acc[kCompRun];
+#pragma unroll
+  for (int p = 0; p < kCompRun; ++p) {
+    const float4 c = y0 + p < H ? P.in[at + (size_t)p * W] : make_float4(0.f, 0.f, 0.f, 0.f);
+    acc[p] = make_float3(P.wt[0] * c.x, P.wt[0] * c.y, P.wt[0] * c.z);
+  }
+  if (P.n >= 1) comp_low<1>(P, x, y0, acc);
+  if (P.n >= 2) comp_low<2>(P, x, y0, acc);
+  if (P.n >= 3) comp_low<3>(P, x, y0, acc);
+  for (int k = 4; k <= P.n; ++k) {
+    const CompLevel L(P, k, x);
+    const float s = __int_as_float((127 - k) << 23), wk = P.wt[k];
+    const float v0 = fmaf((float)y0 + 0.5f, s, -0.5f), fv = floorf(v0);
+    const float3 h0 = L.row((int)fv), h1 = L.row((int)fv + 1);
+#pragma unroll
+    for (int p = 0; p < kCompRun; ++p) comp_add(acc[p], wk, fmaf((float)(y0 + p) + 0.5f, s, -0.5f) - fv, h0, h1);
+  }
+#pragma unroll
+  for (int p = 0; p < kCompRun; ++p)
+    if (y0 + p < H) P.out[at + (size_t)p * W] = make_float4(acc[p].x, acc[p].y, acc[p].z, 1.f);
+}
+
 // One launch for the whole bloom, in three phases separated by grid
 // barriers: the box levels (regions of the frame reduced in shared memory;
 // levels past the seventh one grid-wide pass each), the blur of every tile of
@@ -264,7 +367,6 @@ __device__ void bloom_body(const BloomParams &P) {
   float4 *sH = sb + kBloomSpan * kSDStride;     // kBloomSpan rows x kBloomTile blurred along x (stride kSHStride)
   unsigned phase = 0;
   if (P.n > 0) prefetch_region(P, blockIdx.x);        // read at once
-  prefetch_comp_tile(P, blockIdx.x, kCompW, kCompH);  // read after the pyramid is built
   if (P.n > 0) {
     // ---- box levels 1..7 by regions.  Level 1 of a region (64 x 64 texels)
     // is built with a 3-texel halo at clamped coordinates straight from the
@@ -329,87 +431,16 @@ __device__ void bloom_body(const BloomParams &P) {
       }
     }
     if (!grid_barrier(P, ++phase)) return;
-    // ---- blur every 64x64 tile of levels 2.. (level 1 was blurred by regions)
-    int tiles_before[kBloomMaxLevels + 2];
-    tiles_before[1] = tiles_before[2] = 0;
-    for (int k = 2; k <= P.n; ++k)
-      tiles_before[k + 1] = tiles_before[k] + ((P.w[k] + kBloomTile - 1) / kBloomTile) * ((P.h[k] + kBloomTile - 1) / kBloomTile);
-    for (int tile = blockIdx.x; tile < tiles_before[P.n + 1]; tile += gridDim.x) {
-      int k = 2;
-      while (tile >= tiles_before[k + 1]) ++k;
-      const int t = tile - tiles_before[k], tx = (P.w[k] + kBloomTile - 1) / kBloomTile;
-      blur_tile(P, k, (t % tx) * kBloomTile, (t / tx) * kBloomTile, sD, sH);
-    }
+    blur_upper(P);  // level 1 was blurred by regions
     if (!grid_barrier(P, ++phase)) return;
   }
-  // composite at full resolution, by tiles of kCompW x kCompH pixels.  The
-  // bilinear lookup of level k at pixel (x, y) is a lerp along v of two
-  // lerps along u; the lerps along u depend only on the pixel's column and
-  // the texel row, so for each level the tile's texel rows are first
-  // interpolated along u at every pixel column of the tile and staged in
-  // shared memory (hrow), and each pixel then takes one lerp along v per
-  // level from two staged values.  The arithmetic per pixel is exactly that
-  // of interpolating alone.
-  const int W = P.w[0], H = P.h[0];
-  const int tcx = (W + kCompW - 1) / kCompW, ntiles = tcx * ((H + kCompH - 1) / kCompH);
-  float4 *hrow = sb;
-  // per tile row and level: tv, and the staged index of the row's upper texel row
-  __shared__ float s_tv[kCompH][kBloomMaxLevels];  // [row][k - 1]
-  __shared__ int s_ri[kCompH][kBloomMaxLevels];
-  static_assert(kBloomThreads % kCompW == 0 && kBloomThreads / 32 == kCompH, "composite thread mapping");
-  const int cc = threadIdx.x % kCompW, rstep = kBloomThreads / kCompW;
-  for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-    const int X0 = (tile % tcx) * kCompW, Y0 = (tile / tcx) * kCompH;
-    __syncthreads();  // the previous tile's staged rows have been read
-    prefetch_comp_tile(P, tile + gridDim.x, kCompW, kCompH);
-    int off = 0;
-    for (int k = 1; k <= P.n; ++k) {
-      const float s = __int_as_float((127 - k) << 23);  // 2^-k
-      const int w = P.w[k], h = P.h[k];
-      // texel rows jb .. jb + nr - 1 (contents clamped) serve the tile's pixel rows
-      const int jb = (int)floorf(fmaf((float)Y0 + 0.5f, s, -0.5f));
-      const int nr = (int)floorf(fmaf((float)(Y0 + kCompH - 1) + 0.5f, s, -0.5f)) - jb + 2;
-      if ((int)threadIdx.x < kCompH) {
-        const float v = fmaf((float)(Y0 + (int)threadIdx.x) + 0.5f, s, -0.5f);
-        const float fv = floorf(v);
-        s_tv[threadIdx.x][k - 1] = v - fv;
-        s_ri[threadIdx.x][k - 1] = off + (int)fv - jb;
-      }
-      // this thread's column of the tile: its u, once per level
-      const float u = fmaf((float)(X0 + cc) + 0.5f, s, -0.5f);
-      const float fu = floorf(u), tu = u - fu;
-      const int i0 = min(max((int)fu, 0), w - 1), i1 = min(max((int)fu + 1, 0), w - 1);
-      const float4 *Bk = P.B[k];
-      for (int r = threadIdx.x / kCompW; r < nr; r += rstep) {
-        const float4 *row = Bk + (size_t)min(max(jb + r, 0), h - 1) * w;
-        const float4 a = row[i0], b = row[i1];
-        hrow[(off + r) * kCompW + cc] =
-            make_float4(fmaf(tu, b.x - a.x, a.x), fmaf(tu, b.y - a.y, a.y), fmaf(tu, b.z - a.z, a.z), 0.f);
-      }
-      off += nr;
-    }
-    __syncthreads();
-    // warp yy takes tile row yy, its lanes every 32nd column
-    const int yy = threadIdx.x >> 5, y = Y0 + yy;
-    if (y < H) {
-      for (int c = threadIdx.x & 31; c < kCompW; c += 32) {
-        const int x = X0 + c;
-        if (x >= W) break;
-        const long long p = (long long)y * W + x;
-        const float4 cp = P.in[p];
-        float r = P.wt[0] * cp.x, g = P.wt[0] * cp.y, b = P.wt[0] * cp.z;
-        for (int k = 1; k <= P.n; ++k) {
-          const float tv = s_tv[yy][k - 1];
-          const int ri = s_ri[yy][k - 1];
-          const float4 h0 = hrow[ri * kCompW + c], h1 = hrow[(ri + 1) * kCompW + c];
-          const float wk = P.wt[k];
-          r = fmaf(wk, fmaf(tv, h1.x - h0.x, h0.x), r);
-          g = fmaf(wk, fmaf(tv, h1.y - h0.y, h0.y), g);
-          b = fmaf(wk, fmaf(tv, h1.z - h0.z, h0.z), b);
-        }
-        P.out[p] = make_float4(r, g, b, 1.f);
-      }
-    }
+  // ---- composite: a warp takes 32 columns x 8 rows of the frame, neighbouring
+  // warps neighbouring columns
+  const int W = P.w[0], H = P.h[0], across = (W + 31) / 32, units = across * ((H + kCompRun - 1) / kCompRun);
+  const int warps = blockDim.x >> 5;
+  for (int unit = blockIdx.x * warps + (threadIdx.x >> 5); unit < units; unit += gridDim.x * warps) {
+    const int x = unit % across * 32 + (threadIdx.x & 31), y0 = unit / across * kCompRun;
+    if (x < W) composite_run(P, x, y0);
   }
 }
 
