@@ -773,8 +773,7 @@ extern "C" void bh_destroy(bh_ctx *c) {
   if (c->ring_copy) cudaStreamDestroy(c->ring_copy);
   if (c->bloom_dev) cudaFree(c->bloom_dev);
   if (c->bloom_bar) cudaFree(c->bloom_bar);
-  if (c->orb_outs_host) cudaFreeHost(c->orb_outs_host);
-  if (c->orb_outs_dev) cudaFree(c->orb_outs_dev);
+  if (c->orb_done) cudaEventDestroy(c->orb_done);
   if (c->orb_cams_dev) cudaFree(c->orb_cams_dev);
   delete c;
 }

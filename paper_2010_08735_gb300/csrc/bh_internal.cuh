@@ -124,10 +124,8 @@ struct bh_ctx {
   void *cam_dev = nullptr;
   int cam_cap = 0;
   bh::BatchGraph graph;               // bh_render_batch launches
-  void *orb_outs_host = nullptr;      // bh_render_orbits: pinned output pointers
-  void *orb_outs_dev = nullptr;       // device copy of them, then the tile count
-  void *orb_cams_dev = nullptr;       // per-orbit camera constants
-  int orb_cap = 0;
+  void *orb_cams_dev = nullptr;       // bh_render_orbits: per-orbit camera constants, then the tile count
+  cudaEvent_t orb_done = nullptr;     // behind the last launch that reads them
   float *frame_dev = nullptr;         // bh_render_to_host frame buffer
   size_t frame_cap = 0;
   // bh_render_to_host_async: two device frames; each is copied to the host

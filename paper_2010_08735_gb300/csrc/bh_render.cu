@@ -21,6 +21,7 @@
 namespace bh {
 
 constexpr int kMaxLevels = 14;
+constexpr int kMaxOrbits = 1024;  // of one bh_render_orbits call
 
 // Per-camera constants, computed on the host in FP64 (Eq. staticbasis,
 // Eq. camerabasis, the boost B(v) of Appendix C, Eq. d) and rounded to float.
@@ -989,8 +990,8 @@ extern "C" void bh_disc_particles_free(bh_particles *p) {
 
 // Camera frame in FP64: static basis (Eq. staticbasis), boost B(v) (the
 // camera's 4-velocity is gamma (1, v) on the static frame), user rotation O.
-__host__ __device__ static void camera_constants(const bh_camera *c, CamConst *k) {
-  double st = sin(c->theta), ct = cos(c->theta), sp = sin(c->phi), cph = cos(c->phi);
+__host__ __device__ static void camera_constants_at(const bh_camera *c, double st, double ct, double sp, double cph,
+                                                    CamConst *k) {  // sines and cosines of theta, phi
   double u = 1.0 / c->r;
   double rh[3] = {st * cph, st * sp, ct}, th[3] = {ct * cph, ct * sp, -st}, ph[3] = {-sp, cph, 0.0};
   const double *v = c->v;
@@ -1037,6 +1038,10 @@ __host__ __device__ static void camera_constants(const bh_camera *c, CamConst *k
   k->height = c->height;
   k->rgb = 0;  // RGBA float4 frames unless the host-bound form asks for packed RGB
   k->rgb_vec = 0;
+}
+
+__host__ __device__ static void camera_constants(const bh_camera *c, CamConst *k) {
+  camera_constants_at(c, sin(c->theta), cos(c->theta), sin(c->phi), cos(c->phi), k);
 }
 
 // XYZ -> linear sRGB from the Rec.709 primaries and the D65 white point.
@@ -1129,8 +1134,8 @@ static bh_status fill_params(bh_ctx *ctx, const bh_tables *t, const bh_cubemap *
 }
 
 // Warp tiles (8 x 4 pixels) of a w x h image.
-static inline int tiles_across(int w) { return (w + 7) / 8; }
-static inline int warp_tiles(int w, int h) { return tiles_across(w) * ((h + 3) / 4); }
+__host__ __device__ static inline int tiles_across(int w) { return (w + 7) / 8; }
+__host__ __device__ static inline int warp_tiles(int w, int h) { return tiles_across(w) * ((h + 3) / 4); }
 
 // Persistent grid: enough blocks to fill the GPU, no more than the work needs.
 static int render_grid(const bh_ctx *ctx, long long tiles) {
@@ -1291,35 +1296,97 @@ __host__ __device__ static void orbit_to_camera(const bh_orbit *o, bh_camera *c)
   c->height = o->height;
 }
 
+// The camera constants of an orbit state on the device, straight from the
+// position's direction (cos chi cos psi, sin psi, sin chi cos psi): the chain of
+// acos, atan2 and their sines again took half of a set-up that nothing overlaps
+// (one thread per orbit, FP64 latency).
+__device__ static void orbit_constants(const bh_orbit &o, int width, int height, float *out, CamConst *k) {
+  double sp, cp, sc, cc;
+  sincos(o.psi, &sp, &cp);
+  sincos(o.chi, &sc, &cc);
+  const double rx = cc * cp, ry = sp, ct = sc * cp, st = sqrt(fma(rx, rx, ry * ry));
+  const double ist = st > 0.0 ? 1.0 / st : 0.0;
+  const double cph = st > 0.0 ? rx * ist : 1.0, sph = ry * ist;
+  const double u = 1.0 / o.r, a = sc * ct * cph + cc * st, b = -sc * sph;
+  const double ie = 1.0 / o.e, vpsi = o.l * u * sqrt(1.0 - u) * ie;
+  bh_camera c;
+  c.r = o.r;
+  c.v[0] = o.rdot * ie;
+  c.v[1] = -b * vpsi;
+  c.v[2] = a * vpsi;
+  for (int i = 0; i < 3; ++i) {
+    const double *Or = o.orient + 3 * i;  // on (r', chi', psi')
+    c.orient[3 * i + 0] = Or[0];
+    c.orient[3 * i + 1] = a * Or[1] - b * Or[2];
+    c.orient[3 * i + 2] = b * Or[1] + a * Or[2];
+  }
+  c.fov_y = o.fov_y;
+  c.width = width;
+  c.height = height;
+  camera_constants_at(&c, st, ct, sph, cph, k);
+  k->tiles_x = (width + 7) / 8;  // 8 x 4 pixel warp tiles
+  k->inv_tiles_x = 1.f / (float)k->tiles_x;
+  k->out = reinterpret_cast<float4 *>(out);
+  k->dbg = nullptr;
+}
+
+// First tile of every camera from the cameras' tile counts (shared memory), by
+// the first warp.
+__device__ static void tile_offsets(const int *tiles, int n, CamConst *cams, int *total_tiles) {
+  if (threadIdx.x >= 32) return;
+  int base = 0;
+  for (int k0 = 0; k0 < n; k0 += 32) {
+    const int k = k0 + (int)threadIdx.x, t = k < n ? tiles[k] : 0;
+    int sum = t;
+    for (int o = 1; o < 32; o <<= 1) {
+      const int v = __shfl_up_sync(0xffffffffu, sum, o);
+      if ((int)threadIdx.x >= o) sum += v;
+    }
+    if (k < n) cams[k].tile0 = base + sum - t;
+    base += __shfl_sync(0xffffffffu, sum, 31);
+  }
+  if (threadIdx.x == 0) *total_tiles = base;
+}
+
 // d^2r/dtau^2 = (2 l^2 u^3 - 3 l^2 u^4 - u^2)/2, dpsi/dtau = l u^2,
 // dt/dtau = e/(1-u): RK4 in proper time, FP64, one thread per orbit.  An orbit
 // that would reach r <= 1.05 stops there (no static observer inside the
-// horizon, Sec. 5).
-__device__ static void orbit_rhs(const bh_orbit &o, const double *y, double *dy) {
-  double u = 1.0 / y[1], l2 = o.l * o.l;
-  dy[0] = o.e / (1.0 - u);
+// horizon, Sec. 5).  Bound by the latency of one chain, 4 x steps evaluations
+// long, so each is kept short: reciprocals by Newton's iteration from the
+// single-precision one (2^-23, 2^-46, then rounding), u^2 (l^2 u (2 - 3 u) - 1)/2.
+__device__ __forceinline__ double orbit_rcp(double x) {
+  if (!(fabs(x) > 1e-30 && fabs(x) < 1e30)) return 1.0 / x;
+  double r = (double)__frcp_rn((float)x);
+  r = fma(r, fma(-x, r, 1.0), r);
+  return fma(r, fma(-x, r, 1.0), r);
+}
+
+__device__ __forceinline__ static void orbit_rhs(const bh_orbit &o, double l2, const double *y, double *dy) {
+  const double u = orbit_rcp(y[1]), u2 = u * u;
+  dy[0] = o.e * orbit_rcp(1.0 - u);
   dy[1] = y[3];
-  dy[2] = o.l * u * u;
-  dy[3] = 0.5 * (2.0 * l2 * u * u * u - 3.0 * l2 * u * u * u * u - u * u);
+  dy[2] = o.l * u2;
+  dy[3] = 0.5 * u2 * fma(l2 * u, fma(-3.0, u, 2.0), -1.0);
 }
 
 __device__ static void orbit_advance_one(bh_orbit &o, double dtau, int steps) {
-  double h = dtau / steps;
+  const double h = dtau / steps, l2 = o.l * o.l, h6 = h / 6.0;
   for (int s = 0; s < steps; ++s) {
     double y[4] = {o.t, o.r, o.psi, o.rdot}, k1[4], k2[4], k3[4], k4[4], z[4];
-    orbit_rhs(o, y, k1);
-    for (int a = 0; a < 4; ++a) z[a] = y[a] + 0.5 * h * k1[a];
-    orbit_rhs(o, z, k2);
-    for (int a = 0; a < 4; ++a) z[a] = y[a] + 0.5 * h * k2[a];
-    orbit_rhs(o, z, k3);
-    for (int a = 0; a < 4; ++a) z[a] = y[a] + h * k3[a];
-    orbit_rhs(o, z, k4);
-    double r = y[1] + h / 6.0 * (k1[1] + 2 * k2[1] + 2 * k3[1] + k4[1]);
-    if (!(r > 1.05)) break;
-    o.t = y[0] + h / 6.0 * (k1[0] + 2 * k2[0] + 2 * k3[0] + k4[0]);
-    o.r = r;
-    o.psi = y[2] + h / 6.0 * (k1[2] + 2 * k2[2] + 2 * k3[2] + k4[2]);
-    o.rdot = y[3] + h / 6.0 * (k1[3] + 2 * k2[3] + 2 * k3[3] + k4[3]);
+    orbit_rhs(o, l2, y, k1);
+    for (int a = 0; a < 4; ++a) z[a] = fma(0.5 * h, k1[a], y[a]);
+    orbit_rhs(o, l2, z, k2);
+    for (int a = 0; a < 4; ++a) z[a] = fma(0.5 * h, k2[a], y[a]);
+    orbit_rhs(o, l2, z, k3);
+    for (int a = 0; a < 4; ++a) z[a] = fma(h, k3[a], y[a]);
+    orbit_rhs(o, l2, z, k4);
+    double next[4];
+    for (int a = 0; a < 4; ++a) next[a] = fma(h6, (k1[a] + k4[a]) + 2.0 * (k2[a] + k3[a]), y[a]);
+    if (!(next[1] > 1.05)) break;
+    o.t = next[0];
+    o.r = next[1];
+    o.psi = next[2];
+    o.rdot = next[3];
   }
 }
 
@@ -1335,6 +1402,7 @@ __global__ void orbit_advance_kernel(bh_orbit *orbits, int n, double dtau, int s
 // (its own, in place), then its camera constants at the request's image size,
 // then the tile offsets -- one block, ahead of the render launch.
 __global__ void serve_orbit_setup_kernel(const OrbitJob *jobs, int n, CamConst *cams, int *total_tiles) {
+  __shared__ int tiles[kMaxOrbits];
   for (int k = threadIdx.x; k < n; k += blockDim.x) {
     const OrbitJob j = jobs[k];
     bh_orbit o = *j.orbit;
@@ -1342,50 +1410,32 @@ __global__ void serve_orbit_setup_kernel(const OrbitJob *jobs, int n, CamConst *
       orbit_advance_one(o, j.dtau, j.steps);
       *j.orbit = o;
     }
-    o.width = j.width;
-    o.height = j.height;
-    bh_camera c;
-    orbit_to_camera(&o, &c);
-    camera_constants(&c, &cams[k]);
-    cams[k].tiles_x = (j.width + 7) / 8;
-    cams[k].inv_tiles_x = 1.f / (float)cams[k].tiles_x;
-    cams[k].out = reinterpret_cast<float4 *>(j.out);
-    cams[k].dbg = nullptr;
+    orbit_constants(o, j.width, j.height, j.out, &cams[k]);
+    tiles[k] = warp_tiles(j.width, j.height);
   }
   __syncthreads();
-  if (threadIdx.x == 0) {
-    int tiles = 0;
-    for (int k = 0; k < n; ++k) {
-      cams[k].tile0 = tiles;
-      tiles += cams[k].tiles_x * ((jobs[k].height + 3) / 4);
-    }
-    *total_tiles = tiles;
-  }
+  tile_offsets(tiles, n, cams, total_tiles);
 }
 
-// Camera constants of every orbit (one block), then the tile offsets (one
-// thread, in camera order) -- the same layout bh_render_batch stages from the
-// host.
-__global__ void orbit_camconst_kernel(const bh_orbit *orbits, int n, float *const *outs, CamConst *cams,
+// Camera constants of every orbit (one block), then the tile offsets -- the
+// same layout bh_render_batch stages from the host.  The output addresses are a
+// kernel parameter: no staging buffer that a call would have to wait for.
+template <int N>
+struct OrbitOuts {
+  float *p[N];
+};
+
+template <int N>
+__global__ void orbit_camconst_kernel(const bh_orbit *orbits, int n, const OrbitOuts<N> outs, CamConst *cams,
                                       int *total_tiles) {
+  __shared__ int tiles[N];
   for (int k = threadIdx.x; k < n; k += blockDim.x) {
-    bh_camera c;
-    orbit_to_camera(&orbits[k], &c);
-    camera_constants(&c, &cams[k]);
-    cams[k].tiles_x = (c.width + 7) / 8;  // 8 x 4 pixel warp tiles
-    cams[k].inv_tiles_x = 1.f / (float)cams[k].tiles_x;
-    cams[k].out = reinterpret_cast<float4 *>(outs[k]);
-    cams[k].dbg = nullptr;
+    const bh_orbit o = orbits[k];
+    orbit_constants(o, o.width, o.height, outs.p[k], &cams[k]);
+    tiles[k] = warp_tiles(o.width, o.height);
   }
   __syncthreads();
-  if (threadIdx.x == 0 && blockIdx.x == 0) {
-    int tiles = 0;
-    for (int j = 0; j < n; ++j) {
-      cams[j].tile0 = tiles;
-      tiles += cams[j].tiles_x * ((orbits[j].height + 3) / 4);
-    }
-    *total_tiles = tiles;
-  }
+  tile_offsets(tiles, n, cams, total_tiles);
 }
 
 // One served batch of orbit requests: jobs staged in pinned memory are
@@ -1723,7 +1773,7 @@ extern "C" bh_status bh_render_orbits(bh_ctx *ctx, const bh_tables *t, const bh_
                                       const bh_orbit *orbits_device, const bh_disc *disc,
                                       const bh_shading *sh, float *const *outs, void *stream) {
   TraceRange trace_("bh_render_orbits");
-  if (!ctx || !t || !orbits_device || !outs || n < 1 || n > 1024) {
+  if (!ctx || !t || !orbits_device || !outs || n < 1 || n > kMaxOrbits) {
     set_error("bh_render_orbits: bad argument (1 <= n <= 1024)");
     return BH_ERR_INVALID_ARG;
   }
@@ -1735,30 +1785,31 @@ extern "C" bh_status bh_render_orbits(bh_ctx *ctx, const bh_tables *t, const bh_
   if (!validate_disc(disc)) return BH_ERR_INVALID_ARG;
   BH_CUDA(cudaSetDevice(ctx->device));
   cudaStream_t s = (cudaStream_t)stream;
-  std::lock_guard<std::mutex> lk(ctx->mu);
-  BH_CUDA(cudaStreamSynchronize(s));  // the staging buffers are reused
-  if (n > ctx->orb_cap) {
-    cudaFreeHost(ctx->orb_outs_host);
-    cudaFree(ctx->orb_outs_dev);
-    cudaFree(ctx->orb_cams_dev);
-    ctx->orb_outs_host = nullptr;
-    ctx->orb_outs_dev = nullptr;
-    ctx->orb_cams_dev = nullptr;
-    ctx->orb_cap = 0;
-    BH_CUDA(cudaMallocHost(&ctx->orb_outs_host, sizeof(float *) * 1024));
-    BH_CUDA(cudaMalloc(&ctx->orb_outs_dev, sizeof(float *) * 1024 + 16));
-    BH_CUDA(cudaMalloc(&ctx->orb_cams_dev, sizeof(CamConst) * 1024));
-    ctx->orb_cap = 1024;
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  BH_CUDA(cudaStreamIsCapturing(s, &cap));
+  if (cap != cudaStreamCaptureStatusNone) {
+    set_error("bh_render_orbits: the stream is being captured");
+    return BH_ERR_CUDA;
   }
-  float **ph = static_cast<float **>(ctx->orb_outs_host);
-  for (int k = 0; k < n; ++k) ph[k] = outs[k];
-  float **pd = static_cast<float **>(ctx->orb_outs_dev);
-  int *total_dev = reinterpret_cast<int *>(pd + 1024);
-  BH_CUDA(cudaMemcpyAsync(pd, ph, sizeof(float *) * n, cudaMemcpyHostToDevice, s));
+  std::lock_guard<std::mutex> lk(ctx->mu);
+  if (!ctx->orb_done) BH_CUDA(cudaEventCreateWithFlags(&ctx->orb_done, cudaEventDisableTiming));
+  if (!ctx->orb_cams_dev) BH_CUDA(cudaMalloc(&ctx->orb_cams_dev, sizeof(CamConst) * kMaxOrbits + 16));
+  // the last call's launch may still read the constants, on another stream
+  BH_CUDA(cudaStreamWaitEvent(s, ctx->orb_done, 0));
   RenderParams P;
   fill_params(ctx, t, cube, disc, sh, P);
   CamConst *cams = static_cast<CamConst *>(ctx->orb_cams_dev);
-  orbit_camconst_kernel<<<1, 256, 0, s>>>(orbits_device, n, pd, cams, total_dev);
+  int *total_dev = reinterpret_cast<int *>(cams + kMaxOrbits);
+  const int setup_threads = std::min((n + 31) / 32 * 32, 256);
+  if (n <= 64) {
+    OrbitOuts<64> o = {};
+    for (int k = 0; k < n; ++k) o.p[k] = outs[k];
+    orbit_camconst_kernel<64><<<1, setup_threads, 0, s>>>(orbits_device, n, o, cams, total_dev);
+  } else {
+    OrbitOuts<kMaxOrbits> o = {};
+    for (int k = 0; k < n; ++k) o.p[k] = outs[k];
+    orbit_camconst_kernel<kMaxOrbits><<<1, setup_threads, 0, s>>>(orbits_device, n, o, cams, total_dev);
+  }
   count_launch(ctx);
   P.cams = cams;
   P.ncams = n;
@@ -1772,6 +1823,7 @@ extern "C" bh_status bh_render_orbits(bh_ctx *ctx, const bh_tables *t, const bh_
   BH_CUDA(cudaLaunchKernel(f, dim3(grid), dim3(threads), args, smem, s));
   count_launch(ctx);
   BH_CUDA(cudaGetLastError());
+  BH_CUDA(cudaEventRecord(ctx->orb_done, s));
   return BH_OK;
 }
 

@@ -989,6 +989,37 @@ def test_render_orbits_equals_batch(ctx, gpu_tables, static_scene):
         assert torch.allclose(a, b, rtol=1e-4, atol=1e-6)
 
 
+@pytest.mark.parametrize("n", [1, 33, 64, 65, 1024])
+def test_render_many_orbits_on_two_streams(ctx, gpu_tables, static_scene, n):
+    """Calls of any size, back to back on two streams without a wait between them
+    (they share the context's camera constants): every frame is the one that its
+    orbit gives alone."""
+    cube, _ = static_scene
+    rng = np.random.default_rng(n)
+    sizes = ((8, 4), (17, 9), (24, 13), (1, 1), (33, 20))
+    host = [bh.bh_orbit_init(rng.uniform(4.0, 20.0), math.pi / 2, 0.3, rng.uniform(-1.0, 1.0), None, 1.0,
+                             *sizes[k % len(sizes)]) for k in range(n)]
+    raw = bh.orbits_to_bytes(host)
+    size = len(raw) // n
+    buf = torch.frombuffer(bytearray(raw), dtype=torch.uint8).cuda()
+    sh, disc = bh.make_shading(1.0, EXPOSURE_STARS), synth.disc()
+    torch.cuda.synchronize()
+    streams = [torch.cuda.Stream() for _ in range(2)]
+    outs = [[torch.zeros((o.height, o.width, 4), device="cuda") for o in host] for _ in streams]
+    torch.cuda.synchronize()
+    for part, (first, count) in enumerate(((0, n), (n // 2, n - n // 2))):
+        bh.bh_render_orbits(ctx, gpu_tables, cube, count, buf.data_ptr() + first * size, disc, sh,
+                            outs[part][first:first + count], streams[part])
+    torch.cuda.synchronize()
+    for k in range(0, n, max(1, n // 40)):
+        one = torch.zeros_like(outs[0][k])
+        bh.bh_render_orbits(ctx, gpu_tables, cube, 1, buf.data_ptr() + k * size, disc, sh, [one])
+        torch.cuda.synchronize()
+        assert torch.equal(outs[0][k], one)
+        if k >= n // 2:
+            assert torch.equal(outs[1][k], one)
+
+
 def test_served_orbits_equal_advance_then_render(gpu_tables, static_scene):
     """Viewers served on device-resident orbits: each request advances the
     viewer's orbit on the device and renders it; after three rounds the orbits
