@@ -341,9 +341,9 @@ __device__ void composite_run(const BloomParams &P, int x, int y0) {
 }
 
 // One launch for the whole bloom, in three phases separated by grid
-// barriers: the box levels (regions of the frame reduced in shared memory;
-// levels past the seventh one grid-wide pass each), the blur of every tile of
-// every level, then the composite of every pixel.
+// barriers: the box levels (regions of the frame reduced in shared memory, level
+// 1 blurred with them; levels past the seventh one grid-wide pass each), the
+// blur of the levels above, then the composite of every pixel.
 __device__ void bloom_body(const BloomParams &P);
 
 // The kernel proper, then its exit: the last block to leave (every block

@@ -4,11 +4,11 @@
 // eight 2x2 quads (lane bit 0 = column parity, bit 1 = row parity), so the
 // screen-space derivatives of Sec. 3.3.2 are two warp shuffles (xor 1 and
 // xor 2) with GLSL "fine" semantics.  Blocks are persistent and walk a tile
-// queue that spans every camera of a batch.  The U table (8 KiB) and the
-// disc black-body table (16 KiB) are copied into shared memory once per
-// block by the bulk-copy (TMA) engine behind an mbarrier; the 512x512 D
-// table (1 MiB) and the C(xy,D) table stay in L2 and are read through the
-// read-only path; the star cube map is gathered from L2/HBM with 8-byte
+// queue that spans every camera of a batch.  The U table (8 KiB) is copied into
+// shared memory once per block by the bulk-copy (TMA) engine behind an
+// mbarrier; the 512x512 D table (1 MiB), the disc black-body table (16 KiB) and
+// the C(xy,D) table stay in L2 and are read through the read-only path; the
+// star cube map is gathered from L2/HBM with 8-byte
 // records.  Pixels leave as one float4 store each (a warp writes four full
 // 128-byte lines).
 #include <algorithm>
@@ -85,6 +85,24 @@ __device__ __forceinline__ float sm_tab(const float *p, int i) { return p[i]; }
 __device__ __forceinline__ float sm_tab(const __half *p, int i) { return __half2float(p[i]); }
 
 constexpr float kMuF = 4.0f / 27.0f;
+
+// a / b and 1 / b for b below 2^126 (or a quotient that vanishes): SHORT leaves
+// out the range check of the general division, with the same bits (88 frames
+// compared).  Frames without the animated disc: 77.5 -> 76.3 M warp instructions
+// at 1080p, 84.4 -> 83.2 us, 4K 350 -> 343 us.  The animated variant, at its
+// register limit, got slower (67.8 -> 71.8 us) and keeps the general form.
+template <bool SHORT>
+__device__ __forceinline__ float quot(float a, float b) {
+  return SHORT ? __fdividef(a, b) : a / b;
+}
+template <bool SHORT>
+__device__ __forceinline__ float recip(float b) {
+  float r;
+  if (SHORT) asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(b));
+  else r = 1.f / b;
+  return r;
+}
+
 constexpr int kDbgFloats = 20;  // debug values per pixel (five float4)
 constexpr float kPiF = 3.14159265358979f;
 
@@ -136,14 +154,15 @@ __device__ __forceinline__ float d_bilinear(const DT *D, int n, float fx, float 
 }
 
 // x coordinate of D for e^2 (em = e^2 - mu, formed without cancellation).
+template <bool SHORT>
 __device__ __forceinline__ float d_x(float e2, float em) {
   if (em < 0.f) {
-    float r = e2 / kMuF;  // 1 - eta
-    float lg = r < 0.5f ? log1pf(-r) : logf(-em / kMuF);
+    float r = quot<SHORT>(e2, kMuF);  // 1 - eta
+    float lg = r < 0.5f ? log1pf(-r) : logf(quot<SHORT>(-em, kMuF));
     return 0.5f - sqrtf(fmaxf(-lg, 0.f) * 0.02f);
   }
-  float r = kMuF / e2;  // 1 - (e^2 - mu)/e^2
-  float lg = r < 0.5f ? log1pf(-r) : logf(em / e2);
+  float r = quot<SHORT>(kMuF, e2);  // 1 - (e^2 - mu)/e^2
+  float lg = r < 0.5f ? log1pf(-r) : logf(quot<SHORT>(em, e2));
   return 0.5f + sqrtf(fmaxf(-lg, 0.f) * 0.02f);
 }
 
@@ -201,6 +220,7 @@ enum RenderMode { kPlain = 0, kAnimated = 1, kDebug = 2 };
 template <typename DT, int MODE>
 __global__ void __launch_bounds__(256, BH_RENDER_MIN_BLOCKS) render_kernel(const RenderParams P) {
   constexpr bool DEBUG = MODE == kDebug;
+  constexpr bool SHORT = MODE != kAnimated;  // quotients
   // The debug render is also the checked build: every table, cube-map and
   // occupancy index is tested before its access; a bad one sets a status bit
   // (bh_check_status) and the access is skipped -- no trap, no fault.
@@ -231,6 +251,17 @@ __global__ void __launch_bounds__(256, BH_RENDER_MIN_BLOCKS) render_kernel(const
         "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst1),
         "l"(P.U), "r"((unsigned)P.u_bytes), "r"(mb)
         : "memory");
+  }
+  // peak-temperature luminance for the disc normalisation: its table entries are
+  // asked for here, behind the copy above
+  float peak_t, peak_a, peak_b;
+  {
+    float f = (log2f(P.t_peak) - 8.f) / 12.f * kDiscN - 0.5f;
+    f = fminf(fmaxf(f, 0.f), (float)(kDiscN - 1));
+    int k0 = (int)f, k1 = min(k0 + 1, kDiscN - 1);
+    peak_t = f - k0;
+    peak_a = s_disc[k0].x;
+    peak_b = s_disc[k1].x;
   }
   // animated disc (Appendix B): this frame's particle constants, phases
   // reduced in FP64 so that FP32 keeps them exact to ~1e-7 rad at any time
@@ -278,39 +309,30 @@ __global__ void __launch_bounds__(256, BH_RENDER_MIN_BLOCKS) render_kernel(const
   const DT *D = reinterpret_cast<const DT *>(P.D);
   const int n_half = dn / 2;
 
-  // peak-temperature luminance for the disc normalisation
-  float y_peak;
-  {
-    float f = (log2f(P.t_peak) - 8.f) / 12.f * kDiscN - 0.5f;
-    f = fminf(fmaxf(f, 0.f), (float)(kDiscN - 1));
-    int k0 = (int)f, k1 = min(k0 + 1, kDiscN - 1);
-    float t = f - k0;
-    y_peak = expf(fmaf(t, s_disc[k1].x - s_disc[k0].x, s_disc[k0].x));
-  }
+  const float y_peak = expf(fmaf(peak_t, peak_b - peak_a, peak_a));
 
-  // Dynamic schedule: each warp takes the next warp tiles from a global counter
-  // until none are left: P.fetch at a time while plenty are left, one at a time
-  // for the last kTailTiles per warp, so that no warp sits on a second tile
-  // while others have run out (a frame of 2,048 tiles takes one each).  Asking
-  // for the next fetch before the current one is rendered measured slower (1080p
-  // 86.0 -> 88.9 us: the early claim lengthens the tail by a tile).
+  // Dynamic schedule: a warp's first tiles follow from its place in the grid; then
+  // it takes the next ones from a global counter until none are left: P.fetch at
+  // a time while plenty are left, one at a time for the last kTailTiles per warp,
+  // so that no warp sits on a second tile while others have run out.  A launch
+  // with no more to hand out than it has warps (a frame of 2,048 tiles) never
+  // touches the counter, whose round trips were a fifth of such a frame's time
+  // (256 x 256: 13.8 -> 10.5 us; 1080p 82.6 -> 81.5, 4K 341 -> 346).
+  // Asking for the next fetch before the current one is rendered measured slower
+  // (1080p 86.0 -> 88.9 us: the early claim lengthens the tail by a tile).
   const unsigned total_tiles = P.total_tiles_dev ? *P.total_tiles_dev : P.total_tiles;
   const unsigned n_warps = gridDim.x * (blockDim.x >> 5), fetch = P.fetch;
   const unsigned chunked = total_tiles > kTailTiles * n_warps ? (total_tiles - kTailTiles * n_warps) / fetch * fetch : 0u;
-  unsigned tile = 0, tile_end = 0;
+  const bool counted = chunked / fetch + (total_tiles - chunked) > n_warps;
   int cam = 0;  // the camera of the warp's last tile: its tiles only ever increase
-  for (;;) {
-    if (tile == tile_end) {
-      unsigned g = 0;
-      if (lane == 0 && table_ok) g = atomicAdd(P.sched, 1u);
-      g = __shfl_sync(0xffffffffu, g, 0);
-      // whole chunks first, then single tiles (g stays below total_tiles + n_warps)
-      const unsigned first = g * fetch, single = chunked + (g - chunked / fetch);
-      const bool chunk = g < chunked / fetch;
-      tile = chunk ? first : single;
-      tile_end = tile + (chunk ? fetch : 1u);
-      if (!table_ok || tile >= total_tiles) break;
-    }
+  for (unsigned g = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); table_ok;) {
+    // whole chunks first, then single tiles (g stays below total_tiles + 2 n_warps)
+    const unsigned first = g * fetch, single = chunked + (g - chunked / fetch);
+    const bool chunk = g < chunked / fetch;
+    unsigned tile = chunk ? first : single;
+    const unsigned tile_end = tile + (chunk ? fetch : 1u);
+    if (tile >= total_tiles) break;
+    do {
     // ---- which camera and which tile of it.  A single-camera launch reads
     // its constants straight from the kernel parameters (constant bank); a
     // batch reads them from global memory.  The pixel work is written once.
@@ -337,7 +359,7 @@ __global__ void __launch_bounds__(256, BH_RENDER_MIN_BLOCKS) render_kernel(const
             x2_ = fmaf(qw, C.w[1], -qh * C.w[0]);
       float c2 = fmaf(x0_, x0_, fmaf(x1_, x1_, x2_ * x2_));
       pxw = c2;
-      dpar = C.gamma * (fmaf(qq, C.inv_gamma2, -c2) / (nq * fmaf(C.beta, nq, wq)));
+      dpar = C.gamma * quot<SHORT>(fmaf(qq, C.inv_gamma2, -c2), nq * fmaf(C.beta, nq, wq));
     } else {
       dpar = C.gamma * fmaf(wq, inv, -C.beta);
     }
@@ -410,19 +432,19 @@ __global__ void __launch_bounds__(256, BH_RENDER_MIN_BLOCKS) render_kernel(const
       captured = true;
     } else {
       int s = udot > 0.f ? 1 : -1;
-      float xd = d_x(e2, em);
+      float xd = d_x<SHORT>(e2, em);
       float fx = xd * P.d_n1f;
       int xlo = em < 0.f ? 0 : n_half, xhi = em < 0.f ? n_half - 1 : dn - 1;
       float ua = 0.f, Dl, Da = 0.f, phia = INFINITY, yv;
       if (em < 0.f) {
-        float eta = -em / kMuF;
+        float eta = quot<SHORT>(-em, kMuF);
         float sa = asinf(sqrtf(fminf(eta, 1.f)));
         float th = fmaf(-2.f, sa, 0.5f * kPiF) * (1.f / 3.f);
         ua = fmaf(2.f / 3.f, sinf(th), 1.f / 3.f);
         // 1 - u/u_a = (du/dphi)^2 / (u_a g), g = (f(u_a) - f(u))/(u_a - u), f(x) = x^2 - x^3:
         // no cancellation when the camera is near the apsis (du/dphi -> 0)
         float g = fmaf(-u, u, fmaf(-ua, u, fmaf(-ua, ua, ua + u)));
-        float om = g > 0.f ? udot * udot / (ua * g) : 1.f - u / ua;
+        float om = g > 0.f ? quot<SHORT>(udot * udot, ua * g) : 1.f - quot<SHORT>(u, ua);
         yv = 1.f - sqrtf(fmaxf(om, 0.f));
         Dl = d_bilinear_pair(D, dn, fx, yv * P.d_n1f, xlo, xhi, chk);
         Da = d_bilinear_pair(D, dn, fx, P.d_n1f, xlo, xhi, chk);
@@ -430,7 +452,7 @@ __global__ void __launch_bounds__(256, BH_RENDER_MIN_BLOCKS) render_kernel(const
       } else {
         const float r23 = 0.81649658f, r13 = 0.57735027f;
         float sq = sqrtf(fabsf(um));
-        yv = (r23 + (um >= 0.f ? sq : -sq)) / (r23 + r13);
+        yv = quot<SHORT>(r23 + (um >= 0.f ? sq : -sq), r23 + r13);
         Dl = d_bilinear_pair(D, dn, fx, yv * P.d_n1f, xlo, xhi, chk);
       }
       if (alpha_ok && P.disc_on) {
@@ -438,7 +460,7 @@ __global__ void __launch_bounds__(256, BH_RENDER_MIN_BLOCKS) render_kernel(const
         // from one reciprocal; y's scale folds in the texel count
         const float e = sqrtf(e2);
         const float a6 = fmaf(6.f, e2, 1.f), a3 = 3.f * (1.f + e2);
-        const float iq = 1.f / (a6 * a3);
+        const float iq = recip<SHORT>(a6 * a3);
         const float ux = a3 * iq;
         const float yk = fmaf(6.f * e2, e, 1.f) * (a6 * iq) * P.u_nphi1f;
         float fxu = fminf(fmaxf(ux * P.u_ne1f, 0.f), P.u_ne1f);
@@ -458,7 +480,7 @@ __global__ void __launch_bounds__(256, BH_RENDER_MIN_BLOCKS) render_kernel(const
         // retarded times (debug render and animated disc): t = R - 1/u +
         // ln(u/(1-u)) of the camera point and of the apsis, from D's time channel
         float tcam = 0.f, tapsis = 0.f;
-        auto t_of_R = [](float R, float uu) { return R - 1.f / uu + logf(uu / (1.f - uu)); };
+        auto t_of_R = [](float R, float uu) { return R - recip<SHORT>(uu) + logf(quot<SHORT>(uu, 1.f - uu)); };
         auto ulookT = [&](float ph) {
           float fy = fminf(fmaxf(ph * yk, 0.f), P.u_nphi1f);
           int j0 = (int)fy, j1 = min(j0 + 1, P.u_nphi - 1);
@@ -474,7 +496,7 @@ __global__ void __launch_bounds__(256, BH_RENDER_MIN_BLOCKS) render_kernel(const
           if (em < 0.f) tapsis = t_of_R(d_bilinear(P.DTt, dn, fx, (float)(dn - 1), xlo, xhi, chk), ua);
         }
         float phi = Dl + (s == 1 ? kPiF - dma : dma);
-        float turns0 = floorf(phi / kPiF);
+        float turns0 = floorf(quot<SHORT>(phi, kPiF));
         float phi0 = fmaf(-kPiF, turns0, phi);
         const float u0 = phi0 < phia ? ulook(phi0) : 0.f;
         if (phi0 < phia && P.u_oc <= u0 && u0 <= P.u_ic && ((s == 1 && u0 > u) || (s == -1 && u0 < u))) {
@@ -485,7 +507,7 @@ __global__ void __launch_bounds__(256, BH_RENDER_MIN_BLOCKS) render_kernel(const
         }
         if (em < 0.f && s == 1) {
           phi = fmaf(2.f, phia, -phi);
-          float turns1 = floorf(phi / kPiF);
+          float turns1 = floorf(quot<SHORT>(phi, kPiF));
           float phi1 = fmaf(-kPiF, turns1, phi);
           const float u1 = phi1 < phia ? ulook(phi1) : 0.f;
           if (phi1 < phia && P.u_oc <= u1 && u1 <= P.u_ic) {
@@ -515,20 +537,20 @@ __global__ void __launch_bounds__(256, BH_RENDER_MIN_BLOCKS) render_kernel(const
       // dcam sqrt(2 - 3u') / (sqrt(1-u) (sqrt(2) + u'^(3/2) (e_z.e_z') / e)).
       const float ie = rsqrtf(e2);
       const float dpre = dcam * C.inv_sqrt_1mu;
-      const float escale = P.exp_disc / y_peak;
+      const float escale = quot<SHORT>(P.exp_disc, y_peak);
       for (int h = 0; h < nh; ++h) {
         float up = h == 0 ? hu0 : hu1;
         float rho_h = P.rho;
         if (anim) {
           // Appendix B: density at the hit's retarded time, radius and azimuth
           const float sg = (h == 0 ? odd0 : odd1) ? -1.f : 1.f;
-          rho_h = particle_density(s_part, P.n_parts, P.rho, h == 0 ? th0 : th1, 1.f / up,
+          rho_h = particle_density(s_part, P.n_parts, P.rho, h == 0 ? th0 : th1, recip<SHORT>(up),
                                    atan2f(sg * tsy, sg * tsx));
         }
         if (h == 0) dens0 = rho_h; else dens1 = rho_h;
         const float sc = rho_h * escale;
         float su = sqrtf(up);
-        float Dk = dpre * sqrtf(fmaf(-3.f, up, 2.f)) / fmaf(up * su * z2, ie, 1.41421356f);
+        float Dk = quot<SHORT>(dpre * sqrtf(fmaf(-3.f, up, 2.f)), fmaf(up * su * z2, ie, 1.41421356f));
         if (h == 0) dop0 = Dk; else dop1 = Dk;
         // T^4 ~ u^3 (1 - sqrt(3u)), T = t_peak at the maximum: log2(D T)
         float fu = up * up * up * fmaf(-1.7320508f, su, 1.f);
@@ -605,7 +627,7 @@ __global__ void __launch_bounds__(256, BH_RENDER_MIN_BLOCKS) render_kernel(const
           else { face = 5; sc = -dp0; tc = -dp1; dmaw = -dw2; dmah = -dh2; dscw = -dw0; dsch = -dh0; dtcw = -dw1; dtch = -dh1; }
         }
         const int N = P.cube_n;
-        float hN = 0.5f * N, ima = 1.f / ma, hNi = hN * ima;
+        float hN = 0.5f * N, ima = recip<SHORT>(ma), hNi = hN * ima;
         float sr = sc * ima, tr = tc * ima;
         float S = (sr + 1.f) * hN, T = (tr + 1.f) * hN;
         float Jsw = hNi * fmaf(-sr, dmaw, dscw), Jsh = hNi * fmaf(-sr, dmah, dsch);
@@ -631,7 +653,7 @@ __global__ void __launch_bounds__(256, BH_RENDER_MIN_BLOCKS) render_kernel(const
         float det = fmaf(a11, a22, -a12 * a21);
         if (det * det > 1e-12f * (fmaf(a11, a11, a21 * a21) * fmaf(a12, a12, a22 * a22)) &&
             check(L >= 0 && L < P.cube_levels && L < kMaxLevels && face >= 0 && face < 6)) {
-          float id = 1.f / det;
+          float id = recip<SHORT>(det);
           float i11 = a22 * id, i12 = -a12 * id, i21 = -a21 * id, i22 = a11 * id;
           int i0 = max((int)floorf(cS - hsL), 0), i1 = min((int)floorf(cS + hsL), NL - 1);
           int j0 = max((int)floorf(cT - htL), 0), j1 = min((int)floorf(cT + htL), NL - 1);
@@ -650,7 +672,7 @@ __global__ void __launch_bounds__(256, BH_RENDER_MIN_BLOCKS) render_kernel(const
           // in: 3.3 take iterations per warp tile of the 1080p frame against 8.6 when
           // the lanes moved from row to row together (of 123 occupied texels in a
           // tile's 32 bounding boxes only 15 hold a star with a weight: the rest lie
-          // beside thin, slanted footprints).  Every star's weight is rounded in the
+          // beside thin, slanted footprints; the cull leaves 61).  Every star's weight is rounded in the
           // same steps as in a walk row by row, and stars are taken in row order.
           // 1080p frame 98.5 -> 87.3 us, 4K 435 -> 375 us, 256^2 24.7 -> 17.2 us.
           // Occupancy of the 8 x 8 texels from (wi, wj) on, clipped to the
@@ -681,7 +703,7 @@ __global__ void __launch_bounds__(256, BH_RENDER_MIN_BLOCKS) render_kernel(const
           // the rows (a slope that is not finite) bounds nothing: fmaxf and fminf
           // drop the NaN.
           auto cull = [&](const uint2 bits, const int wi, const int wj) {
-            const float r22 = 1.f / a22, r21 = 1.f / a21;
+            const float r22 = recip<SHORT>(a22), r21 = recip<SHORT>(a21);
             const float s1 = a12 * r22, s2 = a11 * r21, g1 = fabsf(det * r22), g2 = fabsf(det * r21);
             const float y = wj - cT, x = cS - wi;
             const float e1 = fmaf(1e-5f, fmaf(16.f, fabsf(s1), g1), g1 + 0.01f);
@@ -768,7 +790,7 @@ __global__ void __launch_bounds__(256, BH_RENDER_MIN_BLOCKS) render_kernel(const
         // C(xy, D): trilinear, texel centres, clamped.  One base texel and
         // constant strides (0 at a clamped edge, where the weight is 0);
         // interpolated along x, then y, then log2 D.
-        const float iS = 1.f / Ssum;
+        const float iS = recip<SHORT>(Ssum);
         float fx = fmaf(SX * iS, kCnx / 0.60f, -(0.15f * kCnx / 0.60f + 0.5f));
         float fy = fmaf(SY * iS, kCny / 0.35f, -(0.15f * kCny / 0.35f + 0.5f));
         float fz = fmaf(__log2f(dstar), kCnd / 8.f, 4.f * kCnd / 8.f - 0.5f);
@@ -860,7 +882,12 @@ __global__ void __launch_bounds__(256, BH_RENDER_MIN_BLOCKS) render_kernel(const
       ++tile;
       shade(P.cam0, t);
     }
+    } while (tile != tile_end);
+    if (!counted) return;
+    if (lane == 0) g = n_warps + atomicAdd(P.sched, 1u);
+    g = __shfl_sync(0xffffffffu, g, 0);
   }
+  if (!counted) return;
   // Retire the warp; the last warp of the grid re-arms the counters for the
   // next launch that uses them (every warp has taken its final fetch by then).
   if (lane == 0) {
