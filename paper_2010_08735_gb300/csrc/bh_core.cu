@@ -52,56 +52,69 @@ bh_status cuda_fail(cudaError_t e, const char *what) {
 
 void count_launch(bh_ctx *ctx, int n) { ctx->launches.fetch_add(n, std::memory_order_relaxed); }
 
-static void pool_release(bh_ctx *ctx) {  // pool_mu held
-  for (PoolBlock &b : ctx->pool) {
+static void pool_release(Pool &pool) {  // pool.mu held
+  for (PoolBlock &b : pool.kept) {
     if (b.ready) {
       cudaEventSynchronize(b.ready);
       cudaEventDestroy(b.ready);
     }
     cudaFree(b.p);
   }
-  ctx->pool.clear();
-  ctx->pool_bytes = 0;
+  pool.kept.clear();
+  pool.bytes = 0;
 }
 
-cudaError_t pool_get(bh_ctx *ctx, size_t bytes, cudaStream_t s, PoolBlock *out) {
-  std::lock_guard<std::mutex> lk(ctx->pool_mu);
+cudaError_t pool_get(Pool &pool, size_t bytes, cudaStream_t s, PoolBlock *out, bool scratch) {
+  // Under stream capture nothing is taken from the pool (a block's event lies
+  // outside the capture) or put into it: a handle's memory is allocated, which
+  // only a relaxed capture allows, and scratch belongs to the graph.
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  const cudaError_t ce = cudaStreamIsCapturing(s, &cap);
+  if (ce != cudaSuccess) return ce;
+  if (cap != cudaStreamCaptureStatusNone) {
+    PoolBlock b;
+    b.bytes = scratch ? 0 : bytes;  // 0: freed on its stream
+    const cudaError_t e = scratch ? cudaMallocAsync(&b.p, bytes, s) : cudaMalloc(&b.p, bytes);
+    if (e == cudaSuccess) *out = b;
+    return e;
+  }
+  std::lock_guard<std::mutex> lk(pool.mu);
   int best = -1;  // the smallest that fits and wastes less than its half
-  for (int k = 0; k < (int)ctx->pool.size(); ++k) {
-    const size_t have = ctx->pool[k].bytes;
-    if (have >= bytes && have / 2 <= bytes && (best < 0 || have < ctx->pool[best].bytes)) best = k;
+  for (int k = 0; k < (int)pool.kept.size(); ++k) {
+    const size_t have = pool.kept[k].bytes;
+    if (have >= bytes && have / 2 <= bytes && (best < 0 || have < pool.kept[best].bytes)) best = k;
   }
   if (best >= 0) {
-    PoolBlock b = ctx->pool[best];
+    PoolBlock b = pool.kept[best];
     if (b.ready) {
       const cudaError_t e = cudaStreamWaitEvent(s, b.ready, 0);
       if (e != cudaSuccess) return e;
       cudaEventDestroy(b.ready);  // takes effect once the event has completed
       b.ready = nullptr;
     }
-    ctx->pool.erase(ctx->pool.begin() + best);
-    ctx->pool_bytes -= b.bytes;
+    pool.kept.erase(pool.kept.begin() + best);
+    pool.bytes -= b.bytes;
     *out = b;
     return cudaSuccess;
   }
   PoolBlock b;
   b.bytes = bytes;
   cudaError_t e = cudaMalloc(&b.p, bytes);
-  if (e == cudaErrorMemoryAllocation && !ctx->pool.empty()) {
+  if (e == cudaErrorMemoryAllocation && !pool.kept.empty()) {
     cudaGetLastError();
-    pool_release(ctx);
+    pool_release(pool);
     e = cudaMalloc(&b.p, bytes);
   }
   if (e == cudaSuccess) *out = b;
   return e;
 }
 
-static void pool_keep(bh_ctx *ctx, PoolBlock b) {  // b.ready behind its last use, or idle
+static void pool_keep(Pool &pool, PoolBlock b) {  // b.ready behind its last use, or idle
   {
-    std::lock_guard<std::mutex> lk(ctx->pool_mu);
-    if (ctx->pool_bytes + b.bytes <= kPoolBytes) {
-      ctx->pool.push_back(b);
-      ctx->pool_bytes += b.bytes;
+    std::lock_guard<std::mutex> lk(pool.mu);
+    if (pool.open && pool.bytes + b.bytes <= kPoolBytes) {
+      pool.kept.push_back(b);
+      pool.bytes += b.bytes;
       return;
     }
   }
@@ -112,8 +125,12 @@ static void pool_keep(bh_ctx *ctx, PoolBlock b) {  // b.ready behind its last us
   cudaFree(b.p);
 }
 
-void pool_put(bh_ctx *ctx, PoolBlock b, cudaStream_t s) {
+void pool_put(Pool &pool, PoolBlock b, cudaStream_t s) {
   if (!b.p) return;
+  if (b.bytes == 0) {
+    cudaFreeAsync(b.p, s);
+    return;
+  }
   b.ready = nullptr;
   if (cudaEventCreateWithFlags(&b.ready, cudaEventDisableTiming) != cudaSuccess || cudaEventRecord(b.ready, s) != cudaSuccess) {
     if (b.ready) cudaEventDestroy(b.ready);
@@ -121,13 +138,13 @@ void pool_put(bh_ctx *ctx, PoolBlock b, cudaStream_t s) {
     cudaFree(b.p);  // waits for the device
     return;
   }
-  pool_keep(ctx, b);
+  pool_keep(pool, b);
 }
 
-void pool_put_idle(bh_ctx *ctx, PoolBlock b) {
+void pool_put_idle(Pool &pool, PoolBlock b) {
   if (!b.p) return;
   b.ready = nullptr;
-  pool_keep(ctx, b);
+  pool_keep(pool, b);
 }
 
 bh_status check_status(bh_ctx *ctx, cudaStream_t s) {
@@ -681,7 +698,7 @@ bh_status colour_tables_launch(bh_ctx *ctx, bh_tables *t, cudaStream_t s) {
     unsigned done[kSpecCells];
   };
   PoolBlock mem;
-  BH_CUDA(pool_get(ctx, sizeof(Scratch), s, &mem));
+  BH_CUDA(pool_get(*ctx->pool, sizeof(Scratch), s, &mem, true));
   Scratch *w = static_cast<Scratch *>(mem.p);
   cudaError_t e = cudaMemsetAsync(w->done, 0, sizeof w->done, s);
   spectrum_kernel<<<kSpecCells * kSpecNodes, 32, 0, s>>>(black_body_fit<kSpecNodes>(), w->val, w->done, w->coef);
@@ -689,7 +706,7 @@ bh_status colour_tables_launch(bh_ctx *ctx, bh_tables *t, cudaStream_t s) {
   colour_cell_kernel<<<kCnx * kCny / 4, 128, 0, s>>>(&w->locus, w->coef, t->C);
   count_launch(ctx, 3);
   if (e == cudaSuccess) e = cudaGetLastError();
-  pool_put(ctx, mem, s);
+  pool_put(*ctx->pool, mem, s);
   return e == cudaSuccess ? BH_OK : cuda_fail(e, "colour tables");
 }
 
@@ -713,7 +730,7 @@ extern "C" bh_status bh_create(int device, size_t budget, bh_ctx **out) {
   }
   BH_CUDA(cudaSetDevice(device));
   bh_ctx *c = new bh_ctx();
-  c->device = device;
+  c->device = c->pool->device = device;
   c->budget = budget;
   cudaError_t e = cudaDeviceGetAttribute(&c->sm_count, cudaDevAttrMultiProcessorCount, device);
   if (e == cudaSuccess) e = cudaMalloc((void **)&c->status_dev, sizeof(unsigned));
@@ -756,8 +773,9 @@ extern "C" void bh_destroy(bh_ctx *c) {
   cudaDeviceSynchronize();
   c->graph.reset();
   {
-    std::lock_guard<std::mutex> lk(c->pool_mu);
-    bh::pool_release(c);
+    std::lock_guard<std::mutex> lk(c->pool->mu);
+    c->pool->open = false;
+    bh::pool_release(*c->pool);
   }
   if (c->status_dev) cudaFree(c->status_dev);
   if (c->sched_dev) cudaFree(c->sched_dev);
@@ -803,6 +821,7 @@ static bh_status tables_alloc(bh_ctx *ctx, const bh_table_desc *desc, cudaStream
                               bh_tables **out) {
   bh_tables *t = new bh_tables();
   t->ctx = ctx;
+  t->pool = ctx->pool;
   t->desc = *desc;
   size_t nd = (size_t)desc->d_n * desc->d_n, nu = (size_t)desc->u_ne * desc->u_nphi;
   const size_t es = desc->storage == BH_F32 ? 4 : 2;
@@ -816,7 +835,7 @@ static bh_status tables_alloc(bh_ctx *ctx, const bh_table_desc *desc, cudaStream
   const size_t o_D64 = place(nd * 8), o_U64 = place(nu * 8), o_D = place(2 * nd * es) /* row-paired render copy */,
                o_U = place(nu * es), o_DT64 = place(nd * 8), o_UT64 = place(nu * 8), o_DT = place(nd * 4),
                o_UT = place(nu * 4), o_C = place(sizeof(float4) * kCnx * kCny * kCnd), o_disc = place(sizeof(float4) * kDiscN);
-  const cudaError_t e = pool_get(ctx, bytes, s, &t->mem);
+  const cudaError_t e = pool_get(*ctx->pool, bytes, s, &t->mem);
   if (e != cudaSuccess) {
     delete t;
     return cuda_fail(e, "table allocation");
@@ -981,8 +1000,8 @@ extern "C" bh_status bh_tables_copy_colour(const bh_tables *t, float *Ch, float 
 
 extern "C" void bh_tables_free(bh_tables *t) {
   if (!t) return;
-  cudaSetDevice(t->ctx->device);
+  cudaSetDevice(t->pool->device);
   cudaDeviceSynchronize();
-  pool_put_idle(t->ctx, t->mem);
+  pool_put_idle(*t->pool, t->mem);
   delete t;
 }

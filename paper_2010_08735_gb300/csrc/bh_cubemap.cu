@@ -834,7 +834,7 @@ extern "C" bh_status bh_build_star_cubemap(bh_ctx *ctx, const bh_star *stars, lo
   const size_t b_stars = sort ? sorted : 0, b_copy = n > 0 && !on_device ? up16(sizeof(bh_star) * (size_t)n) : 0;
   const size_t cleared = b_arrived + b_count + b_acc;
   PoolBlock mem;
-  cudaError_t e = pool_get(ctx, cleared + b_span + b_fit + b_nodes + b_stars + b_copy, s, &mem);
+  cudaError_t e = pool_get(*ctx->pool, cleared + b_span + b_fit + b_nodes + b_stars + b_copy, s, &mem, true);
   unsigned char *scratch = static_cast<unsigned char *>(mem.p);
   if (e != cudaSuccess) {
     bh_cubemap_free(c);
@@ -884,7 +884,7 @@ extern "C" bh_status bh_build_star_cubemap(bh_ctx *ctx, const bh_star *stars, lo
     occupancy_launch(ctx, c, N >= kRegion ? 3 : 0, s);
     e = cudaGetLastError();
   }
-  pool_put(ctx, mem, s);
+  pool_put(*ctx->pool, mem, s);
   if (e != cudaSuccess) {
     bh_cubemap_free(c);
     return cuda_fail(e, "bh_build_star_cubemap");
@@ -911,12 +911,13 @@ namespace bh {
 bh_status cubemap_alloc_public(bh_ctx *ctx, int N, bh_dtype storage, cudaStream_t s, bh_cubemap **out) {
   bh_cubemap *c = new bh_cubemap();
   c->ctx = ctx;
+  c->pool = ctx->pool;
   c->n = N;
   c->levels = cube_levels(N);
   c->storage = storage;
   c->records = bh_cubemap_records(N);
   const size_t rec_bytes = (sizeof(uint2) * c->records + 255) / 256 * 256;
-  const cudaError_t e = pool_get(ctx, rec_bytes + sizeof(uint2) * mask_level_offset(N, c->levels), s, &c->mem);
+  const cudaError_t e = pool_get(*ctx->pool, rec_bytes + sizeof(uint2) * mask_level_offset(N, c->levels), s, &c->mem);
   if (e != cudaSuccess) {
     delete c;
     return cuda_fail(e, "cube map allocation");
@@ -930,9 +931,9 @@ bh_status cubemap_alloc_public(bh_ctx *ctx, int N, bh_dtype storage, cudaStream_
 
 extern "C" void bh_cubemap_free(bh_cubemap *c) {
   if (!c) return;
-  cudaSetDevice(c->ctx->device);
+  cudaSetDevice(c->pool->device);
   cudaDeviceSynchronize();
-  pool_put_idle(c->ctx, c->mem);
+  pool_put_idle(*c->pool, c->mem);
   delete c;
 }
 

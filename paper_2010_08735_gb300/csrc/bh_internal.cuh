@@ -8,6 +8,7 @@
 #include <atomic>
 #include <cstdarg>
 #include <cstdint>
+#include <memory>
 #include <mutex>
 #include <vector>
 
@@ -107,6 +108,13 @@ struct PoolBlock {
   cudaEvent_t ready = nullptr;  // recorded behind its last use; nullptr: idle
 };
 constexpr size_t kPoolBytes = (size_t)512 << 20;
+struct Pool {  // shared with the handles: one freed after bh_destroy finds it closed
+  int device = 0;
+  std::mutex mu;  // guards what follows
+  std::vector<PoolBlock> kept;
+  size_t bytes = 0;
+  bool open = true;
+};
 
 }  // namespace bh
 
@@ -141,9 +149,7 @@ struct bh_ctx {
   unsigned *bloom_bar = nullptr;      // bh_bloom: grid-barrier counter
   bh::RenderTuning tuning;
   bh::ServeState *serve = nullptr;
-  std::vector<bh::PoolBlock> pool;    // free blocks, guarded by pool_mu
-  size_t pool_bytes = 0;
-  std::mutex pool_mu;
+  std::shared_ptr<bh::Pool> pool = std::make_shared<bh::Pool>();
   int inject_table_wait = 0;          // bh_inject_fault: next render's table wait never completes
   int inject_bloom_barrier = 0;       // bh_inject_fault: next bloom's first grid barrier is never complete
   std::mutex mu;
@@ -151,6 +157,7 @@ struct bh_ctx {
 
 struct bh_tables {
   bh_ctx *ctx = nullptr;
+  std::shared_ptr<bh::Pool> pool;
   bh::PoolBlock mem;  // all arrays below
   bh_table_desc desc{};
   double *D64 = nullptr, *U64 = nullptr;  // FP64 values
@@ -169,6 +176,7 @@ struct bh_particles {
 
 struct bh_cubemap {
   bh_ctx *ctx = nullptr;
+  std::shared_ptr<bh::Pool> pool;
   bh::PoolBlock mem;  // records and mask
   int n = 0;        // face size
   int levels = 0;
@@ -207,9 +215,9 @@ inline int cube_levels(int N) {
 // A block of at least `bytes`, usable by work on stream s from now on; give it
 // back behind the work on stream s (pool_put), or once the device is idle
 // (pool_put_idle).  From any thread.
-cudaError_t pool_get(bh_ctx *ctx, size_t bytes, cudaStream_t s, PoolBlock *out);
-void pool_put(bh_ctx *ctx, PoolBlock b, cudaStream_t s);
-void pool_put_idle(bh_ctx *ctx, PoolBlock b);
+cudaError_t pool_get(Pool &pool, size_t bytes, cudaStream_t s, PoolBlock *out, bool scratch = false);
+void pool_put(Pool &pool, PoolBlock b, cudaStream_t s);
+void pool_put_idle(Pool &pool, PoolBlock b);
 void count_launch(bh_ctx *ctx, int n = 1);
 bh_status check_status(bh_ctx *ctx, cudaStream_t s);
 bh_status colour_tables_launch(bh_ctx *ctx, bh_tables *t, cudaStream_t s);

@@ -243,6 +243,50 @@ def test_memory_kept_by_a_context_is_bounded_and_given_back():
                 assert torch.cuda.mem_get_info()[0] >= free0 - (64 << 20)
 
 
+def test_handles_freed_after_their_context_give_their_memory_back():
+    for _ in range(2):  # the second of two equal rounds: the driver's one-time allocations are behind it
+        free0 = torch.cuda.mem_get_info()[0]
+        c = bh.bh_create()
+        tables = bh.bh_precompute_tables(c, 66, 10, 6)
+        cube = bh.bh_build_star_cubemap(c, synth.stars(1000, 5), 1024, 1)  # 67 MB of records
+        bh.bh_destroy(c)
+        bh.bh_tables_free(tables)
+        bh.bh_cubemap_free(cube)
+        left = free0 - torch.cuda.mem_get_info()[0]
+    assert left < (64 << 20)
+
+
+def test_tables_and_map_built_under_a_relaxed_capture(ctx):
+    """The builds of a captured stream take nothing from the memory that the
+    context keeps: a graph replayed later fills the handles it was captured with,
+    and calls outside the capture go on as before."""
+    stars = torch.from_numpy(synth.stars(2000, 5)).cuda()
+
+    def build(stream=None):
+        return (bh.bh_precompute_tables(ctx, 66, 10, 6, bh.BH_F32, stream),
+                bh.bh_build_star_cubemap(ctx, stars, 64, 1, stream))
+
+    def read(handles):
+        torch.cuda.synchronize()
+        out = (*bh.bh_tables_copy_out(handles[0], 66, 10, 6), bh.bh_cubemap_copy_out(handles[1], 64))
+        bh.bh_tables_free(handles[0])
+        bh.bh_cubemap_free(handles[1])
+        return out
+
+    expect = read(build())  # its memory stays with the context
+    stream, graph = torch.cuda.Stream(), torch.cuda.CUDAGraph()
+    torch.cuda.synchronize()
+    with torch.cuda.stream(stream):
+        graph.capture_begin(capture_error_mode="relaxed")
+        captured = build(stream)
+        graph.capture_end()
+    between = read(build())
+    graph.replay()
+    for got in (between, read(captured)):
+        assert all(np.array_equal(a, b) for a, b in zip(got, expect))
+    del graph
+
+
 def test_cubemap_from_device_stars(ctx, orc):
     st = synth.stars(4000, seed=12)
     dst = torch.from_numpy(st).cuda()
