@@ -137,6 +137,21 @@ constexpr int kBloomRegionLevels = 7;
 // whose box texels, with a 3-texel halo at clamped coordinates, are in sD.
 __device__ void blur_staged(const BloomParams &P, int k, int x0, int y0, const float4 *sD, float4 *sH);
 
+// A block's share of units of work of one warp each: a run of neighbouring units
+// (they share rows in L1), the same number in every block, so that a frame of
+// fewer warps than the grid's uses every SM's load path, not that of a few full
+// blocks, and the last wave is even: 46.8 -> 43.2 us at 1080p, six levels.
+struct Share {
+  long long first, end;
+  int step;
+  __device__ explicit Share(long long units) {
+    const long long per = (units + gridDim.x - 1) / gridDim.x;
+    first = blockIdx.x * per + (threadIdx.x >> 5);
+    end = min((blockIdx.x + 1) * per, units);
+    step = blockDim.x >> 5;
+  }
+};
+
 // The blur of levels 2 and up (a twelfth of the frame's texels in all), straight
 // from L2: two outputs of a column per thread, eight rows of seven texels each,
 // in the order of blur_staged's sums.  Tiles staged in shared memory kept 58 of
@@ -146,8 +161,10 @@ __device__ void blur_upper(const BloomParams &P) {
   before[2] = 0;
 #pragma unroll
   for (int k = 2; k <= kBloomMaxLevels; ++k) before[k + 1] = before[k] + (k <= P.n ? (long long)P.w[k] * ((P.h[k] + 1) / 2) : 0);
-  for (long long it = (long long)blockIdx.x * blockDim.x + threadIdx.x; it < before[P.n + 1];
-       it += (long long)gridDim.x * blockDim.x) {
+  const Share share((before[P.n + 1] + 31) / 32);
+  for (long long unit = share.first; unit < share.end; unit += share.step) {
+    const long long it = unit * 32 + (threadIdx.x & 31);
+    if (it >= before[P.n + 1]) break;
     int k = 2;
 #pragma unroll
     for (int l = 3; l <= kBloomMaxLevels; ++l)
@@ -437,8 +454,8 @@ __device__ void bloom_body(const BloomParams &P) {
   // ---- composite: a warp takes 32 columns x 8 rows of the frame, neighbouring
   // warps neighbouring columns
   const int W = P.w[0], H = P.h[0], across = (W + 31) / 32, units = across * ((H + kCompRun - 1) / kCompRun);
-  const int warps = blockDim.x >> 5;
-  for (int unit = blockIdx.x * warps + (threadIdx.x >> 5); unit < units; unit += gridDim.x * warps) {
+  const Share share(units);
+  for (int unit = (int)share.first; unit < share.end; unit += share.step) {
     const int x = unit % across * 32 + (threadIdx.x & 31), y0 = unit / across * kCompRun;
     if (x < W) composite_run(P, x, y0);
   }
