@@ -8,9 +8,10 @@ division and square root, and is also compiled without contraction: every
 fused multiply-add in it is written out (fmaf), so that the single-camera and
 batched instantiations of the pixel code round identically.  It flushes
 denormals: every reciprocal, root and logarithm otherwise carries the scaling
-of an operand below 1.2e-38, which no quantity of a pixel reaches before it is
-invisible (80.2 -> 76.4 M warp instructions per 1080p frame, 90.5 -> 87.3 us,
-frames equal bit for bit).
+of an operand below 1.2e-38 (80.2 -> 76.4 M warp instructions per 1080p frame,
+90.5 -> 87.3 us, frames equal bit for bit).  No visible quantity of a pixel gets
+there: radiances are relative to the disc's peak and to the exposures (the
+disc's own luminance, 4e-50 at 256 K, is only ever handled as a logarithm).
 """
 from __future__ import annotations
 

@@ -252,8 +252,8 @@ __global__ void __launch_bounds__(256, BH_RENDER_MIN_BLOCKS) render_kernel(const
         "l"(P.U), "r"((unsigned)P.u_bytes), "r"(mb)
         : "memory");
   }
-  // peak-temperature luminance for the disc normalisation: its table entries are
-  // asked for here, behind the copy above
+  // ln Y at the peak temperature, by which the disc's light is divided: its table
+  // entries are asked for here, behind the copy above
   float peak_t, peak_a, peak_b;
   {
     float f = (log2f(P.t_peak) - 8.f) / 12.f * kDiscN - 0.5f;
@@ -309,7 +309,8 @@ __global__ void __launch_bounds__(256, BH_RENDER_MIN_BLOCKS) render_kernel(const
   const DT *D = reinterpret_cast<const DT *>(P.D);
   const int n_half = dn / 2;
 
-  const float y_peak = expf(fmaf(peak_t, peak_b - peak_a, peak_a));
+  // below the table (256 K) the light is not normalised
+  const float ln_peak = P.t_peak >= 256.f ? fmaf(peak_t, peak_b - peak_a, peak_a) : 0.f;
 
   // Dynamic schedule: a warp's first tiles follow from its place in the grid; then
   // it takes the next ones from a global counter until none are left: P.fetch at
@@ -537,7 +538,6 @@ __global__ void __launch_bounds__(256, BH_RENDER_MIN_BLOCKS) render_kernel(const
       // dcam sqrt(2 - 3u') / (sqrt(1-u) (sqrt(2) + u'^(3/2) (e_z.e_z') / e)).
       const float ie = rsqrtf(e2);
       const float dpre = dcam * C.inv_sqrt_1mu;
-      const float escale = quot<SHORT>(P.exp_disc, y_peak);
       for (int h = 0; h < nh; ++h) {
         float up = h == 0 ? hu0 : hu1;
         float rho_h = P.rho;
@@ -548,7 +548,7 @@ __global__ void __launch_bounds__(256, BH_RENDER_MIN_BLOCKS) render_kernel(const
                                    atan2f(sg * tsy, sg * tsx));
         }
         if (h == 0) dens0 = rho_h; else dens1 = rho_h;
-        const float sc = rho_h * escale;
+        const float sc = rho_h * P.exp_disc;
         float su = sqrtf(up);
         float Dk = quot<SHORT>(dpre * sqrtf(fmaf(-3.f, up, 2.f)), fmaf(up * su * z2, ie, 1.41421356f));
         if (h == 0) dop0 = Dk; else dop1 = Dk;
@@ -565,7 +565,11 @@ __global__ void __launch_bounds__(256, BH_RENDER_MIN_BLOCKS) render_kernel(const
             float tt = f - k0;
             if (!check(k0 >= 0 && k1 < kDiscN)) k0 = k1 = 0;
             float4 a = s_disc[k0], b = s_disc[k1];
-            float wy = trans * sc * __expf(fmaf(tt, b.x - a.x, a.x));  // (ln Y, X/Y, Z/Y) table
+            // (ln Y, X/Y, Z/Y) table.  Y over the peak's by the difference of the
+            // logarithms: Y itself leaves the float range below 383 K (at 256 K it is
+            // e^-113), the ratio does not, and the exponential of a small number is
+            // the more accurate one.
+            float wy = trans * sc * __expf(fmaf(tt, b.x - a.x, a.x) - ln_peak);
             LX = fmaf(wy, fmaf(tt, b.y - a.y, a.y), LX);
             LY += wy;
             LZ = fmaf(wy, fmaf(tt, b.z - a.z, a.z), LZ);

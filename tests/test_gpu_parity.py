@@ -445,6 +445,36 @@ def test_render_animated_disc(ctx, orc, orc_tables_t, orc_colour, gpu_tables, st
     check_rgb(og, oo, od, mask, cam, "animated")
 
 
+@pytest.mark.parametrize("animated", [False, True])
+@pytest.mark.parametrize("t_peak", [200.0, 260.0, 300.0, 350.0, 380.0, 450.0])
+def test_render_cold_disc(ctx, orc, orc_tables_t, orc_colour, gpu_tables, t_peak, animated):
+    """Discs so cold that their luminance (e^-113 at 256 K) is below the float
+    range: their light relative to their peak is not.  The tolerances are those
+    at 10,000 K times the ratio of the slopes of ln Y in ln T, by which the same
+    error of a hit's temperature weighs more here."""
+    D, U, DT, UT = (a.astype(np.float32) for a in orc_tables_t)
+    scene = orc.SceneTables(D, U, orc_colour[0].astype(np.float32), orc_colour[1].astype(np.float32), DT=DT, UT=UT)
+    ln_T = np.log(2.0) * (8 + 12 * (np.arange(1024) + 0.5) / 1024)
+    slope = np.gradient(orc_colour[1][:, 0], ln_T)
+    worse = slope.max() / np.interp(np.log(1e4), ln_T, slope)
+    cam = synth.camera(6.0, 85.0, v=(0.0, 0.0, 0.5), width=96, height=54)
+    disc = synth.disc(3.0, 12.0, t_peak=t_peak)
+    ph = None
+    try:
+        if animated:
+            parts = synth.disc_particles(16, 5)
+            ph = bh.bh_disc_particles_create(ctx, parts)
+            disc.update(particles=parts, particles_handle=ph, time=250.0)
+        og, gd, oo, od, mask = compare_render(orc, ctx, gpu_tables, None, scene, cam, disc)
+        timed, _ = gpu_render(ctx, gpu_tables, None, cam, disc, debug=False)
+    finally:
+        if ph:
+            bh.bh_disc_particles_free(ph)
+    assert np.isfinite(og).all() and np.array_equal(timed, og)
+    mean, mx, _ = image_error(og, oo, mask)
+    assert mean <= RGB_MEAN_REL * worse and mx <= RGB_MAX_REL * worse, (mean, mx, worse)
+
+
 def test_disc_particles_invalid(ctx):
     good = synth.disc_particles(4, 5)
     for bad in (good[:0], np.vstack([good] * 65), np.array([[0.2, 0.1, 0.0]]), np.array([[0.1, 0.4, 0.0]]),
