@@ -52,16 +52,26 @@ bh_status cuda_fail(cudaError_t e, const char *what) {
 
 void count_launch(bh_ctx *ctx, int n) { ctx->launches.fetch_add(n, std::memory_order_relaxed); }
 
-static void pool_release(Pool &pool) {  // pool.mu held
+static void pool_release(Pool &pool, bool closing) {  // pool.mu held
   for (PoolBlock &b : pool.kept) {
     if (b.ready) {
       cudaEventSynchronize(b.ready);
       cudaEventDestroy(b.ready);
     }
     cudaFree(b.p);
+    pool.bytes -= b.bytes;
   }
   pool.kept.clear();
-  pool.bytes = 0;
+  if (pool.held.empty()) return;
+  if (cudaDeviceSynchronize() != cudaSuccess) {
+    cudaGetLastError();
+    if (!closing) return;
+  }
+  for (HeldBlock &h : pool.held) {  // without a synchronisation, cudaFree waits for the device
+    cudaFree(h.b.p);
+    pool.bytes -= h.b.bytes;
+  }
+  pool.held.clear();
 }
 
 cudaError_t pool_get(Pool &pool, size_t bytes, cudaStream_t s, PoolBlock *out, bool scratch) {
@@ -102,7 +112,7 @@ cudaError_t pool_get(Pool &pool, size_t bytes, cudaStream_t s, PoolBlock *out, b
   cudaError_t e = cudaMalloc(&b.p, bytes);
   if (e == cudaErrorMemoryAllocation && !pool.kept.empty()) {
     cudaGetLastError();
-    pool_release(pool);
+    pool_release(pool, false);
     e = cudaMalloc(&b.p, bytes);
   }
   if (e == cudaSuccess) *out = b;
@@ -141,10 +151,42 @@ void pool_put(Pool &pool, PoolBlock b, cudaStream_t s) {
   pool_keep(pool, b);
 }
 
-void pool_put_idle(Pool &pool, PoolBlock b) {
+void pool_put_synced(Pool &pool, PoolBlock b) {
+  unsigned long long before;
+  {
+    std::lock_guard<std::mutex> lk(pool.mu);
+    before = pool.holds;
+  }
+  const bool idle = cudaDeviceSynchronize() == cudaSuccess;
+  if (!idle) cudaGetLastError();
   if (!b.p) return;
   b.ready = nullptr;
-  pool_keep(pool, b);
+  if (idle) {
+    // what was held when the synchronisation began is idle too
+    {
+      std::lock_guard<std::mutex> lk(pool.mu);
+      size_t left = 0;
+      for (const HeldBlock &h : pool.held) {
+        if (h.seq < before) pool.kept.push_back(h.b);
+        else pool.held[left++] = h;
+      }
+      pool.held.resize(left);
+    }
+    pool_keep(pool, b);
+    return;
+  }
+  // The device cannot be synchronised while one of its streams is captured: a
+  // launch of another stream may still use the block, which therefore goes to
+  // nobody until a synchronisation succeeds.
+  {
+    std::lock_guard<std::mutex> lk(pool.mu);
+    if (pool.open && pool.bytes + b.bytes <= kPoolBytes) {
+      pool.held.push_back({b, pool.holds++});
+      pool.bytes += b.bytes;
+      return;
+    }
+  }
+  if (cudaFree(b.p) != cudaSuccess) cudaGetLastError();  // waits for the device
 }
 
 bh_status check_status(bh_ctx *ctx, cudaStream_t s) {
@@ -775,7 +817,7 @@ extern "C" void bh_destroy(bh_ctx *c) {
   {
     std::lock_guard<std::mutex> lk(c->pool->mu);
     c->pool->open = false;
-    bh::pool_release(*c->pool);
+    bh::pool_release(*c->pool, true);
   }
   if (c->status_dev) cudaFree(c->status_dev);
   if (c->sched_dev) cudaFree(c->sched_dev);
@@ -1001,7 +1043,6 @@ extern "C" bh_status bh_tables_copy_colour(const bh_tables *t, float *Ch, float 
 extern "C" void bh_tables_free(bh_tables *t) {
   if (!t) return;
   cudaSetDevice(t->pool->device);
-  cudaDeviceSynchronize();
-  pool_put_idle(*t->pool, t->mem);
+  pool_put_synced(*t->pool, t->mem);
   delete t;
 }

@@ -932,8 +932,7 @@ bh_status cubemap_alloc_public(bh_ctx *ctx, int N, bh_dtype storage, cudaStream_
 extern "C" void bh_cubemap_free(bh_cubemap *c) {
   if (!c) return;
   cudaSetDevice(c->pool->device);
-  cudaDeviceSynchronize();
-  pool_put_idle(*c->pool, c->mem);
+  pool_put_synced(*c->pool, c->mem);
   delete c;
 }
 

@@ -108,11 +108,17 @@ struct PoolBlock {
   cudaEvent_t ready = nullptr;  // recorded behind its last use; nullptr: idle
 };
 constexpr size_t kPoolBytes = (size_t)512 << 20;
+struct HeldBlock {
+  PoolBlock b;
+  unsigned long long seq;  // its number among all that were ever held
+};
 struct Pool {  // shared with the handles: one freed after bh_destroy finds it closed
   int device = 0;
   std::mutex mu;  // guards what follows
   std::vector<PoolBlock> kept;
-  size_t bytes = 0;
+  std::vector<HeldBlock> held;  // freed, but not known to be idle
+  unsigned long long holds = 0;
+  size_t bytes = 0;             // of kept and held
   bool open = true;
 };
 
@@ -213,11 +219,11 @@ inline int cube_levels(int N) {
   return L + 1;
 }
 // A block of at least `bytes`, usable by work on stream s from now on; give it
-// back behind the work on stream s (pool_put), or once the device is idle
-// (pool_put_idle).  From any thread.
+// back behind the work on stream s (pool_put), or behind all work of the device
+// (pool_put_synced, which synchronises it).  From any thread.
 cudaError_t pool_get(Pool &pool, size_t bytes, cudaStream_t s, PoolBlock *out, bool scratch = false);
 void pool_put(Pool &pool, PoolBlock b, cudaStream_t s);
-void pool_put_idle(Pool &pool, PoolBlock b);
+void pool_put_synced(Pool &pool, PoolBlock b);
 void count_launch(bh_ctx *ctx, int n = 1);
 bh_status check_status(bh_ctx *ctx, cudaStream_t s);
 bh_status colour_tables_launch(bh_ctx *ctx, bh_tables *t, cudaStream_t s);

@@ -1,0 +1,108 @@
+"""The device memory that a context keeps, on the CPU: the library runs with a
+stand-in for the CUDA runtime (fake_cudart.cpp) that counts its calls and holds
+a budget of device memory.  Each scenario runs in a process of its own, which
+the stand-in is preloaded into."""
+import ctypes
+import os
+import shutil
+import subprocess
+import sys
+import threading
+from pathlib import Path
+
+import numpy as np
+import pytest
+
+HERE = Path(__file__).resolve().parent
+ROOT = HERE.parent
+MiB = 1 << 20
+
+
+def _fake():
+    f = ctypes.CDLL(None)
+    f.fake_used.restype = ctypes.c_size_t
+    f.fake_total.argtypes = [ctypes.c_size_t]
+    f.fake_calls.argtypes = [ctypes.c_char_p]
+    return f
+
+
+def _calls(f, name):
+    return f.fake_calls(name.encode())
+
+
+def _elsewhere(fn, *args):
+    """A call on another thread (whose CUDA errors are its own)."""
+    t = threading.Thread(target=fn, args=args)
+    t.start()
+    t.join()
+
+
+def free_during_a_capture(bh, f):
+    """While any stream of the device is captured, the device cannot be
+    synchronised, so nothing shows that a freed handle's memory is idle: no later
+    call may get it before a synchronisation succeeds."""
+    ctx = bh.bh_create(0, 0)
+    make = {"tables": lambda: bh.bh_precompute_tables(ctx, 66, 10, 6),
+            "cube": lambda: bh.bh_build_star_cubemap(ctx, np.zeros((0, 5), np.float32), 64, 1)}
+    free = {"tables": bh.bh_tables_free, "cube": bh.bh_cubemap_free}
+    for kind in make:
+        free[kind](make[kind]())  # kept, and idle
+        f.fake_clear()
+        first = make[kind]()
+        assert _calls(f, "cudaMalloc") == 0  # the kept memory
+        f.fake_capture(1)
+        _elsewhere(free[kind], first)
+        second = make[kind]()
+        assert _calls(f, "cudaMalloc") == 1, kind  # not the memory of `first`
+        third = make[kind]()
+        assert _calls(f, "cudaMalloc") == 2, kind
+        assert _calls(f, "cudaFree") == 0
+        free[kind](third)  # the error of its synchronisation stays with it
+        fourth = make[kind]()
+        assert _calls(f, "cudaMalloc") == 3, kind
+        f.fake_capture(0)
+        f.fake_clear()
+        free[kind](second)  # synchronises: first, second and third are idle
+        handles = [fourth] + [make[kind]() for _ in range(3)]
+        assert _calls(f, "cudaMalloc") == 0, kind
+        for h in handles:
+            free[kind](h)
+    # what waits for a synchronisation is bounded with the rest
+    maps = [bh.bh_build_star_cubemap(ctx, np.zeros((0, 5), np.float32), 1024, 1) for _ in range(12)]  # 69 MB each
+    f.fake_capture(1)
+    for m in maps:
+        bh.bh_cubemap_free(m)
+    assert f.fake_used() <= 512 * MiB + 16 * MiB
+    f.fake_capture(0)
+    bh.bh_destroy(ctx)
+    assert f.fake_used() == 0
+
+
+SCENARIOS = [free_during_a_capture]
+
+
+@pytest.fixture(scope="module")
+def fake_runtime(tmp_path_factory):
+    from paper_2010_08735_gb300 import build
+    build.build()
+    cxx = shutil.which("g++")
+    if cxx is None:
+        pytest.skip("no C++ compiler")
+    so = tmp_path_factory.mktemp("fake") / "libfake_cudart.so"
+    include = Path(build.nvcc()).resolve().parent.parent / "include"
+    subprocess.run([cxx, "-std=c++17", "-O1", "-shared", "-fPIC", "-I", str(include), str(HERE / "fake_cudart.cpp"),
+                    "-o", str(so)], check=True)
+    return so
+
+
+@pytest.mark.parametrize("scenario", [s.__name__ for s in SCENARIOS])
+def test_kept_memory(fake_runtime, scenario):
+    r = subprocess.run([sys.executable, __file__, scenario], cwd=ROOT, capture_output=True, text=True, timeout=300,
+                       env=dict(os.environ, LD_PRELOAD=str(fake_runtime)))
+    assert r.returncode == 0, r.stdout + r.stderr
+
+
+if __name__ == "__main__":
+    sys.path.insert(0, str(ROOT))
+    from paper_2010_08735_gb300 import bh
+    {s.__name__: s for s in SCENARIOS}[sys.argv[1]](bh, _fake())

@@ -549,6 +549,37 @@ def test_render_configs_small(ctx, orc, gpu_tables, static_scene, cam):
     check_rgb(og, oo, od, mask, cam, "small")
 
 
+def test_tables_freed_under_a_render_during_a_capture(ctx):
+    """While another stream is captured, freeing a handle cannot wait for the
+    device: frames in flight still read its tables, and no later build gets
+    their memory."""
+    import ctypes
+    rt = ctypes.CDLL("libcudart.so.13")
+    cam, disc, sh = synth.camera(6.0, 85.0, width=3840, height=2160), synth.disc(), bh.make_shading(1.0, 0.0)
+    frames = [torch.zeros((2160, 3840, 4), device="cuda") for _ in range(2)]
+    render, build, capture = (torch.cuda.Stream() for _ in range(3))
+    bh.bh_tables_free(bh.bh_precompute_tables(ctx, 512, 64, 32))  # kept
+    t = bh.bh_precompute_tables(ctx, 512, 64, 32)
+    bh.bh_render(ctx, t, None, cam, disc, sh, frames[0])
+    torch.cuda.synchronize()
+    graph = ctypes.c_void_p()
+    assert rt.cudaStreamBeginCapture(ctypes.c_void_p(capture.cuda_stream), 2) == 0  # relaxed
+    try:
+        for _ in range(30):
+            bh.bh_render(ctx, t, None, cam, disc, sh, frames[1], render)
+        bh.bh_tables_free(t)
+        other = [bh.bh_tables_upload(ctx, np.zeros((512, 512)), np.zeros((32, 64)), bh.BH_F32, build) for _ in range(2)]
+    finally:
+        rt.cudaStreamEndCapture(ctypes.c_void_p(capture.cuda_stream), ctypes.byref(graph))
+        rt.cudaGetLastError()
+        if graph:
+            rt.cudaGraphDestroy(graph)
+    torch.cuda.synchronize()
+    for o in other:
+        bh.bh_tables_free(o)
+    assert torch.equal(*frames)
+
+
 @pytest.mark.parametrize("face,n,dtype", [(1, 50, 1), (2, 50, 2), (4, 200, 1), (8, 300, 2), (16, 40, 1),
                                           (32, 60_000, 1), (64, 3_000, 2), (256, 400_000, 1), (512, 20_000, 2)])
 def test_render_star_windows(ctx, orc, orc_tables, orc_colour, gpu_tables, face, n, dtype):
