@@ -84,6 +84,7 @@ cudaError_t pool_get(Pool &pool, size_t bytes, cudaStream_t s, PoolBlock *out, b
   if (cap != cudaStreamCaptureStatusNone) {
     PoolBlock b;
     b.bytes = scratch ? 0 : bytes;  // 0: freed on its stream
+    b.ordered = scratch;
     const cudaError_t e = scratch ? cudaMallocAsync(&b.p, bytes, s) : cudaMalloc(&b.p, bytes);
     if (e == cudaSuccess) *out = b;
     return e;
@@ -92,7 +93,7 @@ cudaError_t pool_get(Pool &pool, size_t bytes, cudaStream_t s, PoolBlock *out, b
   int best = -1;  // the smallest that fits and wastes less than its half
   for (int k = 0; k < (int)pool.kept.size(); ++k) {
     const size_t have = pool.kept[k].bytes;
-    if (have >= bytes && have / 2 <= bytes && (best < 0 || have < pool.kept[best].bytes)) best = k;
+    if (pool.kept[k].ordered == scratch && have >= bytes && have / 2 <= bytes && (best < 0 || have < pool.kept[best].bytes)) best = k;
   }
   if (best >= 0) {
     PoolBlock b = pool.kept[best];
@@ -109,46 +110,61 @@ cudaError_t pool_get(Pool &pool, size_t bytes, cudaStream_t s, PoolBlock *out, b
   }
   PoolBlock b;
   b.bytes = bytes;
-  cudaError_t e = cudaMalloc(&b.p, bytes);
+  b.ordered = scratch;
+  auto allocate = [&] { return scratch ? cudaMallocAsync(&b.p, bytes, s) : cudaMalloc(&b.p, bytes); };
+  cudaError_t e = allocate();
   if (e == cudaErrorMemoryAllocation && !pool.kept.empty()) {
     cudaGetLastError();
     pool_release(pool, false);
-    e = cudaMalloc(&b.p, bytes);
+    e = allocate();
   }
   if (e == cudaSuccess) *out = b;
   return e;
 }
 
-static void pool_keep(Pool &pool, PoolBlock b) {  // b.ready behind its last use, or idle
-  {
-    std::lock_guard<std::mutex> lk(pool.mu);
-    if (pool.open && pool.bytes + b.bytes <= kPoolBytes) {
-      pool.kept.push_back(b);
-      pool.bytes += b.bytes;
-      return;
+// Keeps b, whose `ready` lies behind its last use or which is idle, in the place
+// of the oldest blocks (with any_kind: of handles too) where there is no room
+// for it.  What is not kept is left in `out` for the caller to free.
+static void pool_keep(Pool &pool, const PoolBlock &b, bool any_kind, std::vector<PoolBlock> &out) {
+  std::lock_guard<std::mutex> lk(pool.mu);
+  size_t may_go = 0;
+  for (const PoolBlock &k : pool.kept)
+    if (any_kind || k.ordered) may_go += k.bytes;
+  if (!pool.open || pool.bytes - may_go + b.bytes > kPoolBytes) {
+    out.push_back(b);
+    return;
+  }
+  size_t left = 0;
+  for (const PoolBlock &k : pool.kept) {
+    if (pool.bytes + b.bytes > kPoolBytes && (any_kind || k.ordered)) {
+      out.push_back(k);
+      pool.bytes -= k.bytes;
+    } else {
+      pool.kept[left++] = k;
     }
   }
-  if (b.ready) {
-    cudaEventSynchronize(b.ready);
-    cudaEventDestroy(b.ready);
-  }
-  cudaFree(b.p);
+  pool.kept.resize(left);
+  pool.kept.push_back(b);
+  pool.bytes += b.bytes;
 }
 
 void pool_put(Pool &pool, PoolBlock b, cudaStream_t s) {
   if (!b.p) return;
-  if (b.bytes == 0) {
-    cudaFreeAsync(b.p, s);
-    return;
-  }
   b.ready = nullptr;
-  if (cudaEventCreateWithFlags(&b.ready, cudaEventDisableTiming) != cudaSuccess || cudaEventRecord(b.ready, s) != cudaSuccess) {
-    if (b.ready) cudaEventDestroy(b.ready);
-    b.ready = nullptr;
-    cudaFree(b.p);  // waits for the device
-    return;
+  std::vector<PoolBlock> out;
+  if (b.bytes != 0 && cudaEventCreateWithFlags(&b.ready, cudaEventDisableTiming) == cudaSuccess &&
+      cudaEventRecord(b.ready, s) == cudaSuccess)
+    pool_keep(pool, b, false, out);
+  else
+    out.push_back(b);
+  // freed in the order of s, without a wait of the host
+  for (PoolBlock &o : out) {
+    if (o.ready) {
+      if (o.p != b.p && cudaStreamWaitEvent(s, o.ready, 0) != cudaSuccess) cudaEventSynchronize(o.ready);
+      cudaEventDestroy(o.ready);
+    }
+    cudaFreeAsync(o.p, s);
   }
-  pool_keep(pool, b);
 }
 
 void pool_put_synced(Pool &pool, PoolBlock b) {
@@ -172,7 +188,15 @@ void pool_put_synced(Pool &pool, PoolBlock b) {
       }
       pool.held.resize(left);
     }
-    pool_keep(pool, b);
+    std::vector<PoolBlock> out;
+    pool_keep(pool, b, true, out);
+    for (PoolBlock &o : out) {
+      if (o.ready) {
+        cudaEventSynchronize(o.ready);
+        cudaEventDestroy(o.ready);
+      }
+      cudaFree(o.p);
+    }
     return;
   }
   // The device cannot be synchronised while one of its streams is captured: a

@@ -99,13 +99,16 @@ constexpr int kSchedRing = 1024;
 
 // Device memory of the context's tables, cube maps and builds, kept when it is
 // given back: a cudaMalloc of a 1M-star map's 277 MB and its cudaFree take 0.5
-// ms, as long as building it.  At most kPoolBytes are kept (larger blocks and
-// what would exceed it go back to the device at once); bh_destroy and an
-// allocation that fails give all of it back.
+// ms, as long as building it.  At most kPoolBytes are kept, the newest; what
+// would exceed them goes back to the device at once.  bh_destroy and an
+// allocation that fails give all of it back.  Scratch comes from the stream-ordered
+// allocator and is only kept for scratch: a call that gives it back to a full
+// pool frees it behind its stream's work, where cudaFree would wait for it.
 struct PoolBlock {
   void *p = nullptr;
   size_t bytes = 0;
   cudaEvent_t ready = nullptr;  // recorded behind its last use; nullptr: idle
+  bool ordered = false;         // scratch, from cudaMallocAsync
 };
 constexpr size_t kPoolBytes = (size_t)512 << 20;
 struct HeldBlock {
@@ -218,9 +221,10 @@ inline int cube_levels(int N) {
   while ((1 << L) < N) ++L;
   return L + 1;
 }
-// A block of at least `bytes`, usable by work on stream s from now on; give it
-// back behind the work on stream s (pool_put), or behind all work of the device
-// (pool_put_synced, which synchronises it).  From any thread.
+// A block of at least `bytes`, usable by work on stream s from now on.  Scratch is
+// given back behind the work on stream s (pool_put, which waits for nothing), a
+// handle's memory behind all work of the device (pool_put_synced, which
+// synchronises it).  From any thread.
 cudaError_t pool_get(Pool &pool, size_t bytes, cudaStream_t s, PoolBlock *out, bool scratch = false);
 void pool_put(Pool &pool, PoolBlock b, cudaStream_t s);
 void pool_put_synced(Pool &pool, PoolBlock b);

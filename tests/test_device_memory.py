@@ -78,7 +78,62 @@ def free_during_a_capture(bh, f):
     assert f.fake_used() == 0
 
 
-SCENARIOS = [free_during_a_capture]
+class _DeviceStars:
+    """n stars in device memory, as the binding sees them."""
+    is_cuda, dtype = True, np.dtype(np.float32)
+
+    def __init__(self, n):
+        self.shape = (n, 5)
+
+    def is_contiguous(self):
+        return True
+
+    def data_ptr(self):
+        return 1 << 30
+
+
+WAITS = ("cudaDeviceSynchronize", "cudaStreamSynchronize", "cudaEventSynchronize", "cudaFree")
+
+
+def builds_only_enqueue(bh, f):
+    """Scratch that cannot be kept goes back in the order of its stream: no call
+    that waits for the device, whatever the scratch's size and however full the
+    kept memory is."""
+    ctx = bh.bh_create(0, 0)
+    fill = [bh.bh_build_star_cubemap(ctx, _DeviceStars(0), 1024, 1) for _ in range(7)]  # 69 MB each
+    for full in (False, True):
+        if full:
+            for m in fill:
+                bh.bh_cubemap_free(m)
+        for n in (1000, 1_000_000, 12_000_000):  # 48 bytes of scratch each
+            f.fake_clear()
+            cube = bh.bh_build_star_cubemap(ctx, _DeviceStars(n), 64, 1, 1)
+            tables = bh.bh_precompute_tables(ctx, 66, 10, 6, bh.BH_F32, 1)
+            assert [w for w in WAITS if _calls(f, w)] == [], (full, n)
+            bh.bh_cubemap_free(cube)
+            bh.bh_tables_free(tables)
+            assert f.fake_used() <= 512 * MiB + 16 * MiB + (0 if full else 7 * 71 * MiB)
+    bh.bh_destroy(ctx)
+    assert f.fake_used() == 0
+
+
+def kept_memory_follows_the_work(bh, f):
+    """Memory kept for sizes that are no longer asked for makes room for what is."""
+    ctx = bh.bh_create(0, 0)
+    for m in [bh.bh_build_star_cubemap(ctx, _DeviceStars(0), 1024, 1) for _ in range(8)]:
+        bh.bh_cubemap_free(m)
+    for face, n in ((2048, 100), (512, 2_000_000), (512, 3_000_000), (512, 1_000_000), (2048, 7_000_000)):
+        for again in (False, True):
+            f.fake_clear()
+            m = bh.bh_build_star_cubemap(ctx, _DeviceStars(n), face, 1)
+            bh.bh_cubemap_free(m)
+            assert f.fake_used() <= 512 * MiB + MiB
+        assert _calls(f, "cudaMalloc") == 0, (face, n)
+    bh.bh_destroy(ctx)
+    assert f.fake_used() == 0
+
+
+SCENARIOS = [free_during_a_capture, builds_only_enqueue, kept_memory_follows_the_work]
 
 
 @pytest.fixture(scope="module")
