@@ -512,12 +512,12 @@ extern "C" bh_status bh_bloom(bh_ctx *ctx, const float *in_device, float *out_de
       ctx->bloom_dev = nullptr;
       ctx->bloom_cap = 0;
     }
-    BH_CUDA(cudaMalloc((void **)&ctx->bloom_dev, need));
+    BH_CUDA(pool_malloc(*ctx->pool, (void **)&ctx->bloom_dev, need));
     ctx->bloom_cap = need;
   }
   if (!ctx->bloom_bar) {
     // arrivals and blocks done: zero now; every launch leaves them zero again
-    BH_CUDA(cudaMalloc((void **)&ctx->bloom_bar, 2 * sizeof(unsigned)));
+    BH_CUDA(pool_malloc(*ctx->pool, (void **)&ctx->bloom_bar, 2 * sizeof(unsigned)));
     BH_CUDA(cudaMemsetAsync(ctx->bloom_bar, 0, 2 * sizeof(unsigned), s));
   }
   static bool taps_ready[64] = {false};

@@ -52,7 +52,7 @@ bh_status cuda_fail(cudaError_t e, const char *what) {
 
 void count_launch(bh_ctx *ctx, int n) { ctx->launches.fetch_add(n, std::memory_order_relaxed); }
 
-static void pool_release(Pool &pool, bool closing) {  // pool.mu held
+static void pool_release(Pool &pool) {  // pool.mu held
   for (PoolBlock &b : pool.kept) {
     if (b.ready) {
       cudaEventSynchronize(b.ready);
@@ -62,16 +62,32 @@ static void pool_release(Pool &pool, bool closing) {  // pool.mu held
     pool.bytes -= b.bytes;
   }
   pool.kept.clear();
-  if (pool.held.empty()) return;
-  if (cudaDeviceSynchronize() != cudaSuccess) {
-    cudaGetLastError();
-    if (!closing) return;
-  }
-  for (HeldBlock &h : pool.held) {  // without a synchronisation, cudaFree waits for the device
-    cudaFree(h.b.p);
+  for (HeldBlock &h : pool.held) {
+    if (cudaFree(h.b.p) != cudaSuccess) cudaGetLastError();  // waits for the device
     pool.bytes -= h.b.bytes;
   }
   pool.held.clear();
+  // the stream-ordered allocator gives its free memory back at the next
+  // synchronisation only
+  cudaMemPool_t ordered;
+  if (cudaDeviceGetDefaultMemPool(&ordered, pool.device) == cudaSuccess) cudaMemPoolTrimTo(ordered, 0);
+}
+
+// An allocation, made again without the kept memory where it fails.  pool.mu held.
+template <typename Allocate>
+static cudaError_t pool_allocate(Pool &pool, const Allocate &allocate) {
+  cudaError_t e = allocate();
+  if (e == cudaErrorMemoryAllocation && !(pool.kept.empty() && pool.held.empty())) {
+    cudaGetLastError();
+    pool_release(pool);
+    e = allocate();
+  }
+  return e;
+}
+
+cudaError_t pool_malloc(Pool &pool, void **p, size_t bytes) {
+  std::lock_guard<std::mutex> lk(pool.mu);
+  return pool_allocate(pool, [&] { return cudaMalloc(p, bytes); });
 }
 
 cudaError_t pool_get(Pool &pool, size_t bytes, cudaStream_t s, PoolBlock *out, bool scratch) {
@@ -111,13 +127,8 @@ cudaError_t pool_get(Pool &pool, size_t bytes, cudaStream_t s, PoolBlock *out, b
   PoolBlock b;
   b.bytes = bytes;
   b.ordered = scratch;
-  auto allocate = [&] { return scratch ? cudaMallocAsync(&b.p, bytes, s) : cudaMalloc(&b.p, bytes); };
-  cudaError_t e = allocate();
-  if (e == cudaErrorMemoryAllocation && !pool.kept.empty()) {
-    cudaGetLastError();
-    pool_release(pool, false);
-    e = allocate();
-  }
+  const cudaError_t e =
+      pool_allocate(pool, [&] { return scratch ? cudaMallocAsync(&b.p, bytes, s) : cudaMalloc(&b.p, bytes); });
   if (e == cudaSuccess) *out = b;
   return e;
 }
@@ -841,7 +852,7 @@ extern "C" void bh_destroy(bh_ctx *c) {
   {
     std::lock_guard<std::mutex> lk(c->pool->mu);
     c->pool->open = false;
-    bh::pool_release(*c->pool, true);
+    bh::pool_release(*c->pool);
   }
   if (c->status_dev) cudaFree(c->status_dev);
   if (c->sched_dev) cudaFree(c->sched_dev);

@@ -228,6 +228,9 @@ inline int cube_levels(int N) {
 cudaError_t pool_get(Pool &pool, size_t bytes, cudaStream_t s, PoolBlock *out, bool scratch = false);
 void pool_put(Pool &pool, PoolBlock b, cudaStream_t s);
 void pool_put_synced(Pool &pool, PoolBlock b);
+// cudaMalloc for a context's other buffers, which takes the kept memory where
+// the device has no more.
+cudaError_t pool_malloc(Pool &pool, void **p, size_t bytes);
 void count_launch(bh_ctx *ctx, int n = 1);
 bh_status check_status(bh_ctx *ctx, cudaStream_t s);
 bh_status colour_tables_launch(bh_ctx *ctx, bh_tables *t, cudaStream_t s);

@@ -1000,7 +1000,7 @@ extern "C" bh_status bh_disc_particles_create(bh_ctx *ctx, const double *ph, int
   bh_particles *p = new bh_particles();
   p->ctx = ctx;
   p->n = n;
-  cudaError_t e = cudaMalloc((void **)&p->dev, sorted.size() * sizeof(double));
+  cudaError_t e = pool_malloc(*ctx->pool, (void **)&p->dev, sorted.size() * sizeof(double));
   if (e == cudaSuccess) e = cudaMemcpy(p->dev, sorted.data(), sorted.size() * sizeof(double), cudaMemcpyHostToDevice);
   if (e != cudaSuccess) {
     cudaFree(p->dev);
@@ -1234,7 +1234,7 @@ static bh_status ensure_cam_staging(bh_ctx *ctx, int n) {
   ctx->cam_cap = 0;
   int cap = std::max(n, 64);
   BH_CUDA(cudaMallocHost(&ctx->cam_host, sizeof(CamConst) * cap));
-  BH_CUDA(cudaMalloc(&ctx->cam_dev, sizeof(CamConst) * cap));
+  BH_CUDA(pool_malloc(*ctx->pool, &ctx->cam_dev, sizeof(CamConst) * cap));
   ctx->cam_cap = cap;
   return BH_OK;
 }
@@ -1558,7 +1558,7 @@ static bh_status render_to_host(bh_ctx *ctx, const bh_tables *t, const bh_cubema
     if (ctx->frame_dev) cudaFree(ctx->frame_dev);
     ctx->frame_dev = nullptr;
     ctx->frame_cap = 0;
-    BH_CUDA(cudaMalloc((void **)&ctx->frame_dev, bytes));
+    BH_CUDA(pool_malloc(*ctx->pool, (void **)&ctx->frame_dev, bytes));
     ctx->frame_cap = bytes;
   }
   bh_status st = render_one(ctx, t, cube, cam, disc, sh, ctx->frame_dev, nullptr, s, rgb);
@@ -1608,7 +1608,7 @@ static bh_status render_to_host_async(bh_ctx *ctx, const bh_tables *t, const bh_
       ctx->ring_dev[k] = nullptr;
     }
     ctx->ring_cap = 0;
-    for (int k = 0; k < 2; ++k) BH_CUDA(cudaMalloc((void **)&ctx->ring_dev[k], bytes));
+    for (int k = 0; k < 2; ++k) BH_CUDA(pool_malloc(*ctx->pool, (void **)&ctx->ring_dev[k], bytes));
     ctx->ring_cap = bytes;
   }
   const int k = (int)(ctx->ring_seq & 1u);
@@ -1716,7 +1716,7 @@ extern "C" bh_status bh_autotune_batch(bh_ctx *ctx, const bh_tables *t, const bh
   cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, ctx->device);
   const size_t flush_bytes = 2 * (size_t)std::max(l2, 0);
   void *flush = nullptr;
-  if (flush_bytes && cudaMalloc(&flush, flush_bytes) != cudaSuccess) {
+  if (flush_bytes && pool_malloc(*ctx->pool, &flush, flush_bytes) != cudaSuccess) {
     flush = nullptr;
     cudaGetLastError();
   }
@@ -1824,7 +1824,7 @@ extern "C" bh_status bh_render_orbits(bh_ctx *ctx, const bh_tables *t, const bh_
   }
   std::lock_guard<std::mutex> lk(ctx->mu);
   if (!ctx->orb_done) BH_CUDA(cudaEventCreateWithFlags(&ctx->orb_done, cudaEventDisableTiming));
-  if (!ctx->orb_cams_dev) BH_CUDA(cudaMalloc(&ctx->orb_cams_dev, sizeof(CamConst) * kMaxOrbits + 16));
+  if (!ctx->orb_cams_dev) BH_CUDA(pool_malloc(*ctx->pool, &ctx->orb_cams_dev, sizeof(CamConst) * kMaxOrbits + 16));
   // the last call's launch may still read the constants, on another stream
   BH_CUDA(cudaStreamWaitEvent(s, ctx->orb_done, 0));
   RenderParams P;

@@ -88,9 +88,9 @@ static bh_status serve_init(bh_ctx *ctx) {
     cudaError_t e = cudaStreamCreateWithFlags(&sl.stream, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&sl.done, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaMallocHost(&sl.cam_host, cam_const_size() * kMaxBatch);
-    if (e == cudaSuccess) e = cudaMalloc(&sl.cam_dev, cam_const_size() * kMaxBatch);
+    if (e == cudaSuccess) e = pool_malloc(*ctx->pool, &sl.cam_dev, cam_const_size() * kMaxBatch);
     if (e == cudaSuccess) e = cudaMallocHost((void **)&sl.job_host, sizeof(OrbitJob) * kMaxBatch);
-    if (e == cudaSuccess) e = cudaMalloc((void **)&sl.job_dev, sizeof(OrbitJob) * kMaxBatch + 16);
+    if (e == cudaSuccess) e = pool_malloc(*ctx->pool, (void **)&sl.job_dev, sizeof(OrbitJob) * kMaxBatch + 16);
     if (e == cudaSuccess) sl.total_dev = reinterpret_cast<int *>(sl.job_dev + kMaxBatch);
     if (e != cudaSuccess) {
       ctx->serve = S;

@@ -22,6 +22,7 @@ std::map<std::string, int> calls;
 std::map<void *, Block> device;
 std::set<void *> pinned;
 size_t total = (size_t)280 << 30, used = 0;
+size_t reserved = 0;  // of `used`: freed in stream order, until a synchronisation or a trim
 unsigned long long next_address = 1ull << 40;
 bool capture_open = false;  // some stream of the device is being captured
 thread_local cudaError_t last = cudaSuccess;
@@ -35,8 +36,10 @@ cudaError_t done(const char *name, cudaError_t e = cudaSuccess) {
 
 cudaError_t take(const char *name, void **p, size_t bytes, bool ordered) {
   std::lock_guard<std::recursive_mutex> lk(mu);
-  if (bytes > total - used) return done(name, cudaErrorMemoryAllocation);
-  used += bytes;
+  const size_t again = ordered && bytes < reserved ? bytes : ordered ? reserved : 0;
+  if (bytes - again > total - used) return done(name, cudaErrorMemoryAllocation);
+  reserved -= again;
+  used += bytes - again;
   *p = reinterpret_cast<void *>(next_address);
   next_address += (bytes + 4095) / 4096 * 4096;
   device[*p] = {bytes, ordered};
@@ -48,13 +51,21 @@ cudaError_t give(const char *name, void *p, bool stream_ordered) {
   if (!p) return done(name);
   const auto it = device.find(p);
   if (it == device.end() || (stream_ordered && !it->second.ordered)) return done(name, cudaErrorInvalidValue);
-  used -= it->second.bytes;
+  if (it->second.ordered) reserved += it->second.bytes;
+  else used -= it->second.bytes;
   device.erase(it);
   return done(name);
 }
 
+void trim() {
+  std::lock_guard<std::recursive_mutex> lk(mu);
+  used -= reserved;
+  reserved = 0;
+}
+
 // While a stream is captured, the device and the legacy stream cannot be synchronised.
 cudaError_t sync(const char *name, bool refused) {
+  if (!refused) trim();
   return done(name, refused ? cudaErrorStreamCaptureUnsupported : cudaSuccess);
 }
 
@@ -108,6 +119,14 @@ cudaError_t cudaMalloc(void **p, size_t bytes) { return take(__func__, p, bytes,
 cudaError_t cudaMallocAsync(void **p, size_t bytes, cudaStream_t) { return take(__func__, p, bytes, true); }
 cudaError_t cudaFree(void *p) { return give(__func__, p, false); }
 cudaError_t cudaFreeAsync(void *p, cudaStream_t) { return give(__func__, p, true); }
+cudaError_t cudaDeviceGetDefaultMemPool(cudaMemPool_t *pool, int) {
+  *pool = nullptr;
+  return done(__func__);
+}
+cudaError_t cudaMemPoolTrimTo(cudaMemPool_t, size_t) {
+  trim();
+  return done(__func__);
+}
 cudaError_t cudaMallocHost(void **p, size_t bytes) {
   *p = std::calloc(1, bytes);
   pinned.insert(*p);

@@ -23,6 +23,7 @@ def _fake():
     f.fake_used.restype = ctypes.c_size_t
     f.fake_total.argtypes = [ctypes.c_size_t]
     f.fake_calls.argtypes = [ctypes.c_char_p]
+    f.cudaMallocHost.argtypes = [ctypes.POINTER(ctypes.c_void_p), ctypes.c_size_t]
     return f
 
 
@@ -127,13 +128,80 @@ def kept_memory_follows_the_work(bh, f):
             f.fake_clear()
             m = bh.bh_build_star_cubemap(ctx, _DeviceStars(n), face, 1)
             bh.bh_cubemap_free(m)
+            f.cudaDeviceSynchronize()  # the stream-ordered allocator keeps nothing past it
             assert f.fake_used() <= 512 * MiB + MiB
         assert _calls(f, "cudaMalloc") == 0, (face, n)
     bh.bh_destroy(ctx)
     assert f.fake_used() == 0
 
 
-SCENARIOS = [free_during_a_capture, builds_only_enqueue, kept_memory_follows_the_work]
+def allocations_take_the_kept_memory(bh, f):
+    """Every allocation of a context that finds the device full gets the memory
+    that the context keeps, whatever it is for."""
+    from paper_2010_08735_gb300 import synth
+    frame = 1 << 32  # an output in device memory
+    cam, small = synth.camera(6.0, 85.0, width=1920, height=1080), synth.camera(6.0, 85.0, width=8, height=4)
+    disc, sh = synth.disc(), bh.make_shading(1.0, 0.05)
+
+    class Pinned:
+        dtype = np.dtype(np.float32)
+
+        def __init__(self):
+            self.p = ctypes.c_void_p()
+            f.cudaMallocHost(ctypes.byref(self.p), 1920 * 1080 * 16)
+
+        def is_contiguous(self):
+            return True
+
+        def numel(self):
+            return 1920 * 1080 * 4
+
+        def data_ptr(self):
+            return self.p.value
+
+    def orbits(ctx, t):
+        bh.bh_render_orbits(ctx, t, None, 1, frame, disc, sh, [frame])
+
+    def autotune(ctx, t):
+        f.fake_clear()
+        bh.bh_autotune_batch(ctx, t, None, [small] * 1000, disc, sh, [frame] * 1000)
+        assert _calls(f, "cudaMalloc") == 3  # the flush buffer, refused once, and the cameras
+
+    calls = {
+        "bloom": lambda ctx, t: bh.bh_bloom(ctx, frame, frame, 1920, 1080, np.ones(7) / 7),
+        "to host": lambda ctx, t: bh.bh_render_to_host(ctx, t, None, cam, disc, sh,
+                                                       np.zeros((1080, 1920, 4), np.float32)),
+        "to host, in flight": lambda ctx, t: bh.bh_render_to_host_async(ctx, t, None, cam, disc, sh, Pinned(), False),
+        "batch": lambda ctx, t: bh.bh_render_batch(ctx, t, None, [small] * 100, disc, sh, [frame] * 100),
+        "autotune": autotune,
+        "orbits": orbits,
+        "particles": lambda ctx, t: bh.bh_disc_particles_free(
+            bh.bh_disc_particles_create(ctx, synth.disc_particles(256, 5))),
+        "served": lambda ctx, t: bh.bh_serve_submit(ctx, t, None, 0, small, disc, sh, frame),
+        "tables": lambda ctx, t: bh.bh_tables_free(bh.bh_precompute_tables(ctx, 512, 64, 32)),
+        "map": lambda ctx, t: bh.bh_cubemap_free(bh.bh_build_star_cubemap(ctx, _DeviceStars(10_000_000), 64, 1)),
+    }
+    for name, call in calls.items():
+        for held in (False, True):  # kept as idle, or freed while nothing could be waited for
+            ctx = bh.bh_create(0, 0)
+            t = bh.bh_precompute_tables(ctx, 66, 10, 6)
+            maps = [bh.bh_build_star_cubemap(ctx, _DeviceStars(0), 1024, 1) for _ in range(7)]
+            f.fake_capture(int(held))
+            for m in maps:
+                bh.bh_cubemap_free(m)
+            f.fake_capture(0)
+            f.fake_total(f.fake_used() + 64)
+            try:
+                call(ctx, t)
+            except bh.BhError as e:
+                raise AssertionError((name, held)) from e
+            bh.bh_tables_free(t)
+            bh.bh_destroy(ctx)
+            assert f.fake_used() == 0, name
+            f.fake_total(280 << 30)
+
+
+SCENARIOS = [allocations_take_the_kept_memory, free_during_a_capture, builds_only_enqueue, kept_memory_follows_the_work]
 
 
 @pytest.fixture(scope="module")
