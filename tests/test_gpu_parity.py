@@ -193,6 +193,50 @@ def test_cubemap_uneven_stars_bit_exact(ctx, orc, N, dtype):
         assert np.array_equal(own.cpu().numpy().view(np.uint16), rec)
 
 
+@pytest.mark.parametrize("N,dtype", [(1, 2), (32, 1), (64, 2), (2048, 1)])
+@pytest.mark.parametrize("count", [128, 129, 1279, 1280, 1281, 20000])
+def test_cubemap_crowded_region_bit_exact(ctx, orc, N, dtype, count):
+    """One region of 32 x 32 texels with counts about those at which its stars are
+    listed, walked by bands or summed in place, beside sparse ones."""
+    st = synth.stars(count + 200, 13)
+    rng = np.random.default_rng(count)
+    st[:count, :3] = np.concatenate([np.ones((count, 1)), rng.uniform(1e-3, 0.03, (count, 2))], 1)
+    st[count:, 0] = -np.abs(st[count:, 0]) - np.float32(2.0)  # the -x face
+    st[:100, 3] *= np.float32(3e5)
+    st[:50, 4] = 500.0
+    st = st[rng.permutation(len(st))]
+    c = bh.bh_build_star_cubemap(ctx, st, N, dtype)
+    try:
+        rec = bh.bh_cubemap_copy_out(c, N)
+    finally:
+        bh.bh_cubemap_free(c)
+    assert np.array_equal(rec, orc.build_cubemap(st, N, dtype))
+
+
+@pytest.mark.parametrize("N", [32, 2048])
+def test_cubemap_crowded_stars_take_no_longer_than_a_few_times_uniform_ones(ctx, N):
+    """400,000 stars in one region against as many over the whole sky on faces of
+    2048^2, medians of five: walked by one block, the region takes 40 times as
+    long; ten times is the limit."""
+    st = synth.stars(400_000, 17)
+    one = st.copy()
+    one[:, :3] = np.concatenate([np.ones((len(st), 1)), np.random.default_rng(1).uniform(1e-3, 0.03, (len(st), 2))], 1)
+
+    def median(stars, face):
+        dev, ms = torch.from_numpy(stars).cuda(), []
+        for _ in range(6):
+            a, b = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+            a.record()
+            c = bh.bh_build_star_cubemap(ctx, dev, face, 1, torch.cuda.current_stream())
+            b.record()
+            torch.cuda.synchronize()
+            ms.append(a.elapsed_time(b))
+            bh.bh_cubemap_free(c)
+        return sorted(ms[1:])[2]
+
+    assert median(one, N) <= 10 * median(st, 2048)
+
+
 def test_memory_kept_by_a_context_is_bounded_and_given_back():
     """Maps and tables built and freed over and over, from two threads on streams
     of their own: every result is that of a fresh context, at most 512 MiB stay
