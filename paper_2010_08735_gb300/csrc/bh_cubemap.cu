@@ -846,20 +846,28 @@ extern "C" bh_status bh_build_star_cubemap(bh_ctx *ctx, const bh_star *stars, lo
   if (st) return st;
   // Scratch, one allocation: counters (cleared), offsets, colour fit, stage
   // nodes, then the sorted stars -- or, where those would take more than the
-  // dense sums of the level-0 texels and 1 GiB, the sums (cleared).
+  // dense sums of the level-0 texels and 1 GiB, or more than the device has, the
+  // sums (cleared).
   const long long per = std::max(N / kRegion, 1), regions = 6 * per * per, texels = 6LL * N * N;
   long long n_nodes, n_counters;
   stage_sizes(N, &n_nodes, &n_counters);
   const size_t sorted = (sizeof(StarBin) + sizeof(StarItem)) * (size_t)n, dense = sizeof(unsigned long long) * 5 * texels;
-  const bool sort = sorted <= std::max<size_t>(dense, (size_t)1 << 30);
   auto up16 = [](size_t b) { return (b + 15) / 16 * 16; };
   const size_t b_arrived = up16(sizeof(unsigned) * (kChromaCells + n_counters)), b_count = up16(sizeof(unsigned long long) * (regions + 1));
-  const size_t b_acc = sort ? 0 : dense, b_span = sizeof(RegionSpan) * regions;
+  const size_t b_span = sizeof(RegionSpan) * regions;
   const size_t b_fit = up16(sizeof(double) * (3 * kNLambda + kChromaCoefs + kChromaVals)), b_nodes = sizeof(Node) * n_nodes;
-  const size_t b_stars = sort ? sorted : 0, b_copy = n > 0 && !on_device ? up16(sizeof(bh_star) * (size_t)n) : 0;
-  const size_t cleared = b_arrived + b_count + b_acc;
+  const size_t b_copy = n > 0 && !on_device ? up16(sizeof(bh_star) * (size_t)n) : 0;
+  bool sort = sorted <= std::max<size_t>(dense, (size_t)1 << 30);
+  size_t b_stars, cleared;
   PoolBlock mem;
-  cudaError_t e = pool_get(*ctx->pool, cleared + b_span + b_fit + b_nodes + b_stars + b_copy, s, &mem, true);
+  cudaError_t e;
+  for (;; sort = false) {
+    b_stars = sort ? sorted : 0;
+    cleared = b_arrived + b_count + (sort ? 0 : dense);
+    e = pool_get(*ctx->pool, cleared + b_span + b_fit + b_nodes + b_stars + b_copy, s, &mem, true);
+    if (e != cudaErrorMemoryAllocation || !sort || dense >= sorted) break;
+    cudaGetLastError();
+  }
   unsigned char *scratch = static_cast<unsigned char *>(mem.p);
   if (e != cudaSuccess) {
     bh_cubemap_free(c);

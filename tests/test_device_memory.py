@@ -201,7 +201,21 @@ def allocations_take_the_kept_memory(bh, f):
             f.fake_total(280 << 30)
 
 
-SCENARIOS = [allocations_take_the_kept_memory, free_during_a_capture, builds_only_enqueue, kept_memory_follows_the_work]
+def many_stars_in_little_memory(bh, f):
+    """Where the device has no room for a sorted copy of the stars, the build makes
+    do with the sums of the texels (240 bytes a level-0 texel)."""
+    for face, n, room in ((128, 20_000_000, 32 * MiB), (64, 1_000_000, 16 * MiB), (8192, 1_000_000, 100 * MiB)):
+        ctx = bh.bh_create(0, 0)
+        records = 8 * bh.bh_cubemap_records(face)
+        f.fake_total(f.fake_used() + records + records // 8 + room)
+        cube = bh.bh_build_star_cubemap(ctx, _DeviceStars(n), face, 1)
+        bh.bh_cubemap_free(cube)
+        bh.bh_destroy(ctx)
+        assert f.fake_used() == 0
+        f.fake_total(280 << 30)
+
+
+SCENARIOS = [many_stars_in_little_memory, allocations_take_the_kept_memory, free_during_a_capture, builds_only_enqueue, kept_memory_follows_the_work]
 
 
 @pytest.fixture(scope="module")

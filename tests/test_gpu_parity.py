@@ -237,6 +237,33 @@ def test_cubemap_crowded_stars_take_no_longer_than_a_few_times_uniform_ones(ctx,
     assert median(one, N) <= 10 * median(st, 2048)
 
 
+def test_cubemap_of_more_stars_than_are_sorted(ctx, gpu_tables, tmp_path):
+    """More than 1 GiB of sorted stars: summed by texels instead.  Records as the
+    allocation-free build's, and the occupancy of the frame as that of the map
+    loaded from its records."""
+    N, n = 128, 23_000_000
+    g = torch.Generator("cuda").manual_seed(3)
+    dev = torch.randn((n, 5), generator=g, device="cuda")
+    dev[:, 2] *= 0.05
+    dev[:, 3] = 1e-3 * dev[:, 3].abs()
+    dev[:, 4] = 3000.0 + 500.0 * dev[:, 4].abs()
+    own = torch.empty((bh.bh_cubemap_records(N), 4), dtype=torch.int16, device="cuda")
+    bh.bh_build_star_cubemap_noalloc(dev, N, bh.BH_F16, own)
+    cube = bh.bh_build_star_cubemap(ctx, dev, N, bh.BH_F16)
+    loaded = None
+    try:
+        assert np.array_equal(bh.bh_cubemap_copy_out(cube, N), own.cpu().numpy().view(np.uint16))
+        bh.bh_cubemap_save(cube, tmp_path / "cube.bhc")
+        loaded = bh.bh_cubemap_load(ctx, tmp_path / "cube.bhc")
+        cam = synth.camera(9.0, 75.0, phi_deg=70.0, width=160, height=90)
+        frames = [gpu_render(ctx, gpu_tables, c, cam, synth.disc(), debug=False)[0] for c in (cube, loaded)]
+        assert np.array_equal(*frames) and frames[0][..., :3].max() > 0
+    finally:
+        bh.bh_cubemap_free(cube)
+        if loaded:
+            bh.bh_cubemap_free(loaded)
+
+
 def test_memory_kept_by_a_context_is_bounded_and_given_back():
     """Maps and tables built and freed over and over, from two threads on streams
     of their own: every result is that of a fresh context, at most 512 MiB stay
