@@ -777,6 +777,30 @@ def test_batch_of_small_cameras_equals_single(ctx, gpu_tables, static_scene, n):
         assert torch.equal(o, one)
 
 
+@pytest.mark.parametrize("animated", [False, True])
+def test_batch_of_thousands_of_cameras_equals_single(ctx, gpu_tables, static_scene, animated):
+    """More cameras than warps: a warp's next tile lies thousands of cameras on."""
+    cube, _ = static_scene
+    cams = synth.batch_cameras(7000, seed=3, resolutions=((8, 4), (1, 1), (33, 17)))
+    disc, sh, ph = synth.disc(), bh.make_shading(1.0, EXPOSURE_STARS), None
+    if animated:
+        ph = bh.bh_disc_particles_create(ctx, synth.disc_particles(4, 5))
+        disc.update(particles_handle=ph, time=37.5)
+    try:
+        at = np.cumsum([0] + [c["width"] * c["height"] for c in cams])
+        all_outs = torch.zeros((int(at[-1]), 4), device="cuda")
+        outs = [all_outs[a:b] for a, b in zip(at, at[1:])]
+        bh.bh_render_batch(ctx, gpu_tables, cube, cams, disc, sh, outs)
+        for k in [*range(0, 7000, 97), *range(6990, 7000)]:
+            one = torch.zeros_like(outs[k])
+            bh.bh_render(ctx, gpu_tables, cube, cams[k], disc, sh, one)
+            assert torch.equal(outs[k], one), k
+    finally:
+        if ph:
+            torch.cuda.synchronize()
+            bh.bh_disc_particles_free(ph)
+
+
 def test_autotune_every_candidate_same_image(gpu_tables, static_scene):
     """The autotuner launches every candidate launch shape; the image does not
     depend on the shape, and batched renders stay equal to single ones."""
