@@ -1713,10 +1713,12 @@ extern "C" bh_status bh_autotune_batch(bh_ctx *ctx, const bh_tables *t, const bh
   bh_status st = validate_batch(n, cams, disc, outs);
   if (st) return st;
   BH_CUDA(cudaSetDevice(ctx->device));
-  // candidates: warps per block, warp tiles per fetch, resident blocks per SM
+  // Candidates: warps per block, warp tiles per fetch, resident blocks per SM.  All
+  // have the 32 warps per SM that fit at 64 registers: of a larger grid the last
+  // blocks, whose first tiles are theirs by their place in it, would start when
+  // the others leave.
   static const RenderTuning cand[] = {{8, 1, 4}, {8, 2, 4}, {8, 4, 4}, {8, 8, 4},
-                                      {4, 1, 8}, {4, 2, 8}, {4, 4, 8}, {8, 16, 4},
-                                      {4, 1, 9}, {4, 2, 9}};
+                                      {4, 1, 8}, {4, 2, 8}, {4, 4, 8}, {8, 16, 4}};
   const int nc = sizeof(cand) / sizeof(cand[0]);
   cudaStream_t s;
   BH_CUDA(cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking));

@@ -24,6 +24,7 @@ std::set<void *> pinned;
 size_t total = (size_t)280 << 30, used = 0;
 size_t reserved = 0;  // of `used`: freed in stream order, until a synchronisation or a trim
 unsigned long long next_address = 1ull << 40;
+unsigned node_threads = 0;  // most threads of a graph's kernel so far
 bool capture_open = false;  // some stream of the device is being captured
 thread_local cudaError_t last = cudaSuccess;
 
@@ -69,6 +70,12 @@ cudaError_t sync(const char *name, bool refused) {
   return done(name, refused ? cudaErrorStreamCaptureUnsupported : cudaSuccess);
 }
 
+cudaError_t kernel_node(const char *name, const cudaKernelNodeParams *p) {
+  const unsigned threads = p->gridDim.x * p->blockDim.x;
+  if (threads > node_threads) node_threads = threads;
+  return done(name);
+}
+
 template <typename T>
 cudaError_t handle(const char *name, T *out) {
   *out = reinterpret_cast<T>(std::malloc(1));
@@ -97,6 +104,7 @@ int fake_calls(const char *name) {
 void fake_capture(int open) { capture_open = open != 0; }
 void fake_total(size_t bytes) { total = bytes; }
 size_t fake_used() { return used; }
+unsigned fake_node_threads() { return node_threads; }
 
 // ---- device
 cudaError_t cudaGetDeviceCount(int *n) { *n = 1; return cudaSuccess; }
@@ -180,14 +188,14 @@ cudaError_t cudaGraphAddMemcpyNode1D(cudaGraphNode_t *n, cudaGraph_t, const cuda
   return done(__func__);
 }
 cudaError_t cudaGraphAddKernelNode(cudaGraphNode_t *n, cudaGraph_t, const cudaGraphNode_t *, size_t,
-                                   const cudaKernelNodeParams *) {
+                                   const cudaKernelNodeParams *p) {
   *n = nullptr;
-  return done(__func__);
+  return kernel_node(__func__, p);
 }
 cudaError_t cudaGraphInstantiate(cudaGraphExec_t *e, cudaGraph_t, unsigned long long) { return handle(__func__, e); }
 cudaError_t cudaGraphExecDestroy(cudaGraphExec_t e) { return drop(__func__, e); }
-cudaError_t cudaGraphExecKernelNodeSetParams(cudaGraphExec_t, cudaGraphNode_t, const cudaKernelNodeParams *) {
-  return done(__func__);
+cudaError_t cudaGraphExecKernelNodeSetParams(cudaGraphExec_t, cudaGraphNode_t, const cudaKernelNodeParams *p) {
+  return kernel_node(__func__, p);
 }
 cudaError_t cudaGraphLaunch(cudaGraphExec_t, cudaStream_t) { return done(__func__); }
 

@@ -1,6 +1,6 @@
-"""The device memory that a context keeps, on the CPU: the library runs with a
-stand-in for the CUDA runtime (fake_cudart.cpp) that counts its calls and holds
-a budget of device memory.  Each scenario runs in a process of its own, which
+"""The device memory that a context keeps, and what it launches, on the CPU: the
+library runs with a stand-in for the CUDA runtime (fake_cudart.cpp) that counts
+its calls and holds a budget of device memory.  Each scenario runs in a process of its own, which
 the stand-in is preloaded into."""
 import ctypes
 import os
@@ -215,7 +215,21 @@ def many_stars_in_little_memory(bh, f):
         f.fake_total(280 << 30)
 
 
-SCENARIOS = [many_stars_in_little_memory, allocations_take_the_kept_memory, free_during_a_capture, builds_only_enqueue, kept_memory_follows_the_work]
+def tuned_launches_are_resident(bh, f):
+    """The render's warps take their first tiles by their place in the grid, which
+    is only even while every block of the launch is resident: 1,024 threads of 64
+    registers an SM, in every shape that the autotuner tries."""
+    from paper_2010_08735_gb300 import synth
+    ctx = bh.bh_create(0, 0)
+    t = bh.bh_precompute_tables(ctx, 66, 10, 6)
+    cam = synth.camera(6.0, 85.0, width=1920, height=1080)
+    bh.bh_autotune_batch(ctx, t, None, [cam] * 8, synth.disc(), bh.make_shading(1.0, 0.05), [1 << 32] * 8)
+    assert f.fake_node_threads() == 152 * 1024
+    bh.bh_tables_free(t)
+    bh.bh_destroy(ctx)
+
+
+SCENARIOS = [tuned_launches_are_resident, many_stars_in_little_memory, allocations_take_the_kept_memory, free_during_a_capture, builds_only_enqueue, kept_memory_follows_the_work]
 
 
 @pytest.fixture(scope="module")
@@ -233,7 +247,7 @@ def fake_runtime(tmp_path_factory):
 
 
 @pytest.mark.parametrize("scenario", [s.__name__ for s in SCENARIOS])
-def test_kept_memory(fake_runtime, scenario):
+def test_host_calls(fake_runtime, scenario):
     r = subprocess.run([sys.executable, __file__, scenario], cwd=ROOT, capture_output=True, text=True, timeout=300,
                        env=dict(os.environ, LD_PRELOAD=str(fake_runtime)))
     assert r.returncode == 0, r.stdout + r.stderr
