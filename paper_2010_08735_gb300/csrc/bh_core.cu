@@ -24,6 +24,7 @@
 //    with 128 nodes: 1.7e-13 on Delta (before: 2.0e-12), 6e-13 on R (4.4e-12),
 //    1.0e-15 on u (1.1e-15), 1.1e-12 on U's R (1.6e-12).
 //  * The colour tables (Sec. 3.4.2): C(xy, D) and the disc black-body table.
+#include <algorithm>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -67,10 +68,6 @@ static void pool_release(Pool &pool) {  // pool.mu held
     pool.bytes -= h.b.bytes;
   }
   pool.held.clear();
-  // the stream-ordered allocator gives its free memory back at the next
-  // synchronisation only
-  cudaMemPool_t ordered;
-  if (cudaDeviceGetDefaultMemPool(&ordered, pool.device) == cudaSuccess) cudaMemPoolTrimTo(ordered, 0);
 }
 
 // An allocation, made again without the kept memory where it fails.  pool.mu held.
@@ -80,6 +77,10 @@ static cudaError_t pool_allocate(Pool &pool, const Allocate &allocate) {
   if (e == cudaErrorMemoryAllocation && !(pool.kept.empty() && pool.held.empty())) {
     cudaGetLastError();
     pool_release(pool);
+    // the stream-ordered allocator gives its free memory back at the next
+    // synchronisation only
+    cudaMemPool_t ordered;
+    if (cudaDeviceGetDefaultMemPool(&ordered, pool.device) == cudaSuccess) cudaMemPoolTrimTo(ordered, 0);
     e = allocate();
   }
   return e;
@@ -100,7 +101,6 @@ cudaError_t pool_get(Pool &pool, size_t bytes, cudaStream_t s, PoolBlock *out, b
   if (cap != cudaStreamCaptureStatusNone) {
     PoolBlock b;
     b.bytes = scratch ? 0 : bytes;  // 0: freed on its stream
-    b.ordered = scratch;
     const cudaError_t e = scratch ? cudaMallocAsync(&b.p, bytes, s) : cudaMalloc(&b.p, bytes);
     if (e == cudaSuccess) *out = b;
     return e;
@@ -109,7 +109,7 @@ cudaError_t pool_get(Pool &pool, size_t bytes, cudaStream_t s, PoolBlock *out, b
   int best = -1;  // the smallest that fits and wastes less than its half
   for (int k = 0; k < (int)pool.kept.size(); ++k) {
     const size_t have = pool.kept[k].bytes;
-    if (pool.kept[k].ordered == scratch && have >= bytes && have / 2 <= bytes && (best < 0 || have < pool.kept[best].bytes)) best = k;
+    if (have >= bytes && have / 2 <= bytes && (best < 0 || have < pool.kept[best].bytes)) best = k;
   }
   if (best >= 0) {
     PoolBlock b = pool.kept[best];
@@ -121,61 +121,42 @@ cudaError_t pool_get(Pool &pool, size_t bytes, cudaStream_t s, PoolBlock *out, b
     }
     pool.kept.erase(pool.kept.begin() + best);
     pool.bytes -= b.bytes;
+    if (scratch) pool.lent += b.bytes;
     *out = b;
     return cudaSuccess;
   }
+  // Scratch that there will be room to keep; other scratch is freed behind its
+  // stream's work, where a cudaFree would make the caller wait for it.
+  const bool keep = scratch && pool.bytes + pool.lent + bytes <= kPoolBytes;
   PoolBlock b;
-  b.bytes = bytes;
-  b.ordered = scratch;
-  const cudaError_t e =
-      pool_allocate(pool, [&] { return scratch ? cudaMallocAsync(&b.p, bytes, s) : cudaMalloc(&b.p, bytes); });
-  if (e == cudaSuccess) *out = b;
-  return e;
-}
-
-// Keeps b, whose `ready` lies behind its last use or which is idle, in the place
-// of the oldest blocks (with any_kind: of handles too) where there is no room
-// for it.  What is not kept is left in `out` for the caller to free.
-static void pool_keep(Pool &pool, const PoolBlock &b, bool any_kind, std::vector<PoolBlock> &out) {
-  std::lock_guard<std::mutex> lk(pool.mu);
-  size_t may_go = 0;
-  for (const PoolBlock &k : pool.kept)
-    if (any_kind || k.ordered) may_go += k.bytes;
-  if (!pool.open || pool.bytes - may_go + b.bytes > kPoolBytes) {
-    out.push_back(b);
-    return;
-  }
-  size_t left = 0;
-  for (const PoolBlock &k : pool.kept) {
-    if (pool.bytes + b.bytes > kPoolBytes && (any_kind || k.ordered)) {
-      out.push_back(k);
-      pool.bytes -= k.bytes;
-    } else {
-      pool.kept[left++] = k;
-    }
-  }
-  pool.kept.resize(left);
-  pool.kept.push_back(b);
-  pool.bytes += b.bytes;
+  b.bytes = scratch && !keep ? 0 : bytes;
+  const cudaError_t e = pool_allocate(
+      pool, [&] { return scratch && !keep ? cudaMallocAsync(&b.p, bytes, s) : cudaMalloc(&b.p, bytes); });
+  if (e != cudaSuccess) return e;
+  if (keep) pool.lent += bytes;
+  if (scratch && !keep) pool.missed = std::max(pool.missed, bytes);
+  *out = b;
+  return cudaSuccess;
 }
 
 void pool_put(Pool &pool, PoolBlock b, cudaStream_t s) {
   if (!b.p) return;
-  b.ready = nullptr;
-  std::vector<PoolBlock> out;
-  if (b.bytes != 0 && cudaEventCreateWithFlags(&b.ready, cudaEventDisableTiming) == cudaSuccess &&
-      cudaEventRecord(b.ready, s) == cudaSuccess)
-    pool_keep(pool, b, false, out);
-  else
-    out.push_back(b);
-  // freed in the order of s, without a wait of the host
-  for (PoolBlock &o : out) {
-    if (o.ready) {
-      if (o.p != b.p && cudaStreamWaitEvent(s, o.ready, 0) != cudaSuccess) cudaEventSynchronize(o.ready);
-      cudaEventDestroy(o.ready);
-    }
-    cudaFreeAsync(o.p, s);
+  if (b.bytes == 0) {
+    cudaFreeAsync(b.p, s);
+    return;
   }
+  b.ready = nullptr;
+  const bool ok = cudaEventCreateWithFlags(&b.ready, cudaEventDisableTiming) == cudaSuccess &&
+                  cudaEventRecord(b.ready, s) == cudaSuccess;
+  std::lock_guard<std::mutex> lk(pool.mu);
+  pool.lent -= b.bytes;
+  if (ok) {
+    pool.kept.push_back(b);
+    pool.bytes += b.bytes;
+    return;
+  }
+  if (b.ready) cudaEventDestroy(b.ready);
+  cudaFree(b.p);  // waits for the device
 }
 
 void pool_put_synced(Pool &pool, PoolBlock b) {
@@ -188,40 +169,52 @@ void pool_put_synced(Pool &pool, PoolBlock b) {
   if (!idle) cudaGetLastError();
   if (!b.p) return;
   b.ready = nullptr;
-  if (idle) {
-    // what was held when the synchronisation began is idle too
-    {
-      std::lock_guard<std::mutex> lk(pool.mu);
+  std::vector<PoolBlock> out;  // to be freed
+  {
+    std::lock_guard<std::mutex> lk(pool.mu);
+    if (!idle) {
+      // The device cannot be synchronised while one of its streams is captured: a
+      // launch of another stream may still use the block, which therefore goes to
+      // nobody until a synchronisation succeeds.
+      if (pool.open && pool.bytes + pool.lent + b.bytes <= kPoolBytes) {
+        pool.held.push_back({b, pool.holds++});
+        pool.bytes += b.bytes;
+      } else {
+        out.push_back(b);  // cudaFree waits for the device
+      }
+    } else {
+      // what was held when the synchronisation began is idle too
       size_t left = 0;
       for (const HeldBlock &h : pool.held) {
         if (h.seq < before) pool.kept.push_back(h.b);
         else pool.held[left++] = h;
       }
       pool.held.resize(left);
-    }
-    std::vector<PoolBlock> out;
-    pool_keep(pool, b, true, out);
-    for (PoolBlock &o : out) {
-      if (o.ready) {
-        cudaEventSynchronize(o.ready);
-        cudaEventDestroy(o.ready);
+      if (pool.open && b.bytes + pool.lent <= kPoolBytes) {
+        pool.kept.push_back(b);
+        pool.bytes += b.bytes;
+      } else {
+        out.push_back(b);
       }
-      cudaFree(o.p);
-    }
-    return;
-  }
-  // The device cannot be synchronised while one of its streams is captured: a
-  // launch of another stream may still use the block, which therefore goes to
-  // nobody until a synchronisation succeeds.
-  {
-    std::lock_guard<std::mutex> lk(pool.mu);
-    if (pool.open && pool.bytes + b.bytes <= kPoolBytes) {
-      pool.held.push_back({b, pool.holds++});
-      pool.bytes += b.bytes;
-      return;
+      // The oldest blocks go where there is no room, also for the scratch that had
+      // none lately.
+      const size_t room = pool.missed <= kPoolBytes / 2 ? pool.missed : 0;
+      pool.missed = 0;
+      size_t k = 0;
+      while (k < pool.kept.size() && pool.bytes + pool.lent + room > kPoolBytes) {
+        pool.bytes -= pool.kept[k].bytes;
+        out.push_back(pool.kept[k++]);
+      }
+      pool.kept.erase(pool.kept.begin(), pool.kept.begin() + k);
     }
   }
-  if (cudaFree(b.p) != cudaSuccess) cudaGetLastError();  // waits for the device
+  for (PoolBlock &o : out) {
+    if (o.ready) {
+      cudaEventSynchronize(o.ready);
+      cudaEventDestroy(o.ready);
+    }
+    if (cudaFree(o.p) != cudaSuccess) cudaGetLastError();
+  }
 }
 
 bh_status check_status(bh_ctx *ctx, cudaStream_t s) {

@@ -99,16 +99,13 @@ constexpr int kSchedRing = 1024;
 
 // Device memory of the context's tables, cube maps and builds, kept when it is
 // given back: a cudaMalloc of a 1M-star map's 277 MB and its cudaFree take 0.5
-// ms, as long as building it.  At most kPoolBytes are kept, the newest; what
-// would exceed them goes back to the device at once.  bh_destroy and an
-// allocation that fails give all of it back.  Scratch comes from the stream-ordered
-// allocator and is only kept for scratch: a call that gives it back to a full
-// pool frees it behind its stream's work, where cudaFree would wait for it.
+// ms, as long as building it.  At most kPoolBytes are kept, the newest; the rest
+// goes back to the device at once.  bh_destroy and an allocation that fails give
+// all of it back.
 struct PoolBlock {
   void *p = nullptr;
-  size_t bytes = 0;
+  size_t bytes = 0;             // 0: stream-ordered scratch, never kept
   cudaEvent_t ready = nullptr;  // recorded behind its last use; nullptr: idle
-  bool ordered = false;         // scratch, from cudaMallocAsync
 };
 constexpr size_t kPoolBytes = (size_t)512 << 20;
 struct HeldBlock {
@@ -118,10 +115,12 @@ struct HeldBlock {
 struct Pool {  // shared with the handles: one freed after bh_destroy finds it closed
   int device = 0;
   std::mutex mu;  // guards what follows
-  std::vector<PoolBlock> kept;
+  std::vector<PoolBlock> kept;  // oldest first
   std::vector<HeldBlock> held;  // freed, but not known to be idle
   unsigned long long holds = 0;
   size_t bytes = 0;             // of kept and held
+  size_t lent = 0;              // of scratch in use that will be kept: bytes + lent <= kPoolBytes
+  size_t missed = 0;            // the largest scratch that there was no room for
   bool open = true;
 };
 
