@@ -214,13 +214,10 @@ constexpr int kCullAbove = 6;
 constexpr unsigned kTailTiles = 6;
 
 // The camera of a tile past `cam`, by a whole warp: its lanes look at 32 parts of
-// the cameras that are left.  A warp's next tile is mostly in the same camera, so
-// this is a function of its own, whose registers the pixel work does not carry
-// (batch of 64 frames 1811 us before, 1814 after; a binary search for every tile
-// 2007).  Stepping through the cameras one by one took 6.1 ms for 20,000
-// thumbnails and 448 us for 1,000 cameras of 64 x 64; this 1.2 ms (the host's
-// part) and 347 us, 300 of them 154 -> 127 us.
-__device__ __noinline__ int search_camera(const CamConst *cams, int ncams, int cam, int tile) {
+// the cameras that are left.  Stepping through the cameras one by one took 6.1 ms
+// for 20,000 thumbnails and 448 us for 1,000 cameras of 64 x 64; this 1.2 ms (the
+// host's part) and 347 us, 300 of them 154 -> 127 us.
+__device__ __forceinline__ int camera_of_tile(const CamConst *cams, int ncams, int cam, int tile) {
   const int lane = threadIdx.x & 31;
   for (int left = ncams - 1 - cam; left > 0;) {
     const int part = (left + 31) >> 5, at = min((lane + 1) * part, left);
@@ -230,6 +227,13 @@ __device__ __noinline__ int search_camera(const CamConst *cams, int ncams, int c
     left = n == 32 ? 0 : min(part - 1, left - go);
   }
   return cam;
+}
+
+// A warp's next tile is mostly in the same camera, so the search is a function of
+// its own (4K 351 -> 346 us); in the animated variant, which lacks registers for
+// the call, it is not (64 frames of 640 x 360 with 64 particles 853 -> 831 us).
+__device__ __noinline__ int search_camera(const CamConst *cams, int ncams, int cam, int tile) {
+  return camera_of_tile(cams, ncams, cam, tile);
 }
 
 // Kernel variants: plain, animated disc (Appendix B), debug (any disc, plus
@@ -893,7 +897,8 @@ __global__ void __launch_bounds__(256, BH_RENDER_MIN_BLOCKS) render_kernel(const
     };
     if (P.cams) {
       if (cam + 1 < P.ncams && __ldg(&P.cams[cam + 1].tile0) <= (int)tile)
-        cam = search_camera(P.cams, P.ncams, cam, (int)tile);
+        cam = MODE == kAnimated ? camera_of_tile(P.cams, P.ncams, cam, (int)tile)
+                                : search_camera(P.cams, P.ncams, cam, (int)tile);
       const CamConst &Cb = P.cams[cam];
       const int t = (int)tile - Cb.tile0;
       ++tile;
