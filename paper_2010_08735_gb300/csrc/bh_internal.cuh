@@ -78,7 +78,8 @@ struct BatchGraph {
 
 struct RenderTuning {
   int warps_per_block = 8;   // block = warps * 32 threads
-  int fetch = 4;             // 8 x 4 pixel warp tiles a warp takes per fetch (before the launch's tail)
+  int fetch = 0;             // 8 x 4 pixel warp tiles a warp takes per fetch (before the launch's
+                             // tail); 0: by the launch's size
   int blocks_per_sm = 4;     // persistent grid = SMs * blocks_per_sm
 };
 

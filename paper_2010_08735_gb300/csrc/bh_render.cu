@@ -50,7 +50,8 @@ struct RenderParams {
   int ncams, total_tiles;   // tiles are 8 x 4 pixel warp tiles, row-major per camera
   const int *total_tiles_dev;  // if set, the tile count computed on the device
   unsigned *sched;          // {next fetch, retired warps}: zero before and after every launch
-  int fetch;                // warp tiles taken per fetch
+  unsigned fetch, tail;     // warp tiles taken per fetch, and handed out singly at the end
+  unsigned by_place;        // fetches up to which a launch has no counter
   const void *D;
   int d_n;
   const void *U;
@@ -208,11 +209,6 @@ __device__ __forceinline__ float particle_density(const float4 *sp, int n, float
 // a 4K one (4M on 4096^2); without it 106 us at 1080p.
 constexpr int kCullAbove = 6;
 
-// Warp tiles per warp that are handed out one at a time at the end of a
-// launch.  Measured at 2 / 4 / 6 / 8 / 16 (chunks of four before them): 1080p
-// frame 92.2 / 87.0 / 84.4 / 84.8 / 86.0 us, 4K 353 / 350 / 349 / 349 / 352 us.
-constexpr unsigned kTailTiles = 6;
-
 // The camera of a tile past `cam`, by a whole warp: its lanes look at 32 parts of
 // the cameras that are left.  Stepping through the cameras one by one took 6.1 ms
 // for 20,000 thumbnails and 448 us for 1,000 cameras of 64 x 64; this 1.2 ms (the
@@ -337,17 +333,16 @@ __global__ void __launch_bounds__(256, BH_RENDER_MIN_BLOCKS) render_kernel(const
 
   // Dynamic schedule: a warp's first tiles follow from its place in the grid; then
   // it takes the next ones from a global counter until none are left: P.fetch at
-  // a time while plenty are left, one at a time for the last kTailTiles per warp,
-  // so that no warp sits on a second tile while others have run out.  A launch
-  // with no more to hand out than it has warps (a frame of 2,048 tiles) never
-  // touches the counter, whose round trips were a fifth of such a frame's time
-  // (256 x 256: 13.8 -> 10.5 us; 1080p 82.6 -> 81.5, 4K 341 -> 346).
+  // a time while plenty are left, one at a time for the last P.tail, so that no
+  // warp sits on a second tile while others have run out.  A launch with no more
+  // to hand out than P.by_place never touches the counter, whose round trips were
+  // a fifth of such a frame's time (256 x 256: 13.8 -> 10.5 us).
   // Asking for the next fetch before the current one is rendered measured slower
   // (1080p 86.0 -> 88.9 us: the early claim lengthens the tail by a tile).
   const unsigned total_tiles = P.total_tiles_dev ? *P.total_tiles_dev : P.total_tiles;
   const unsigned n_warps = gridDim.x * (blockDim.x >> 5), fetch = P.fetch;
-  const unsigned chunked = total_tiles > kTailTiles * n_warps ? (total_tiles - kTailTiles * n_warps) / fetch * fetch : 0u;
-  const bool counted = chunked / fetch + (total_tiles - chunked) > n_warps;
+  const unsigned chunked = total_tiles > P.tail ? (total_tiles - P.tail) / fetch * fetch : 0u;
+  const bool counted = chunked / fetch + (total_tiles - chunked) > P.by_place;
   int cam = 0;  // the camera of the warp's last tile: its tiles only ever increase
   for (unsigned g = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); table_ok;) {
     // whole chunks first, then single tiles (g stays below total_tiles + 2 n_warps)
@@ -909,7 +904,11 @@ __global__ void __launch_bounds__(256, BH_RENDER_MIN_BLOCKS) render_kernel(const
       shade(P.cam0, t);
     }
     } while (tile != tile_end);
-    if (!counted) return;
+    if (!counted) {
+      if (MODE == kAnimated) return;
+      g += n_warps;
+      continue;
+    }
     if (lane == 0) g = n_warps + atomicAdd(P.sched, 1u);
     g = __shfl_sync(0xffffffffu, g, 0);
   }
@@ -1181,7 +1180,6 @@ static bh_status fill_params(bh_ctx *ctx, const bh_tables *t, const bh_cubemap *
     P.inject_wait = 1;
     ctx->inject_table_wait = 0;
   }
-  P.fetch = ctx->tuning.fetch;
   P.sched = ctx->sched_dev + 2 * (ctx->sched_next.fetch_add(1, std::memory_order_relaxed) % kSchedRing);
   return BH_OK;
 }
@@ -1194,6 +1192,31 @@ __host__ __device__ static inline int warp_tiles(int w, int h) { return tiles_ac
 static int render_grid(const bh_ctx *ctx, long long tiles) {
   const long long need = (tiles + ctx->tuning.warps_per_block - 1) / ctx->tuning.warps_per_block;
   return (int)std::min<long long>(need, (long long)ctx->sm_count * ctx->tuning.blocks_per_sm);
+}
+
+// Tiles of a launch by chunks of two where it has up to kFewTiles per warp, the
+// last kFewTail per warp singly; above it by chunks of four, the last kTail singly.
+// A chunk in a disc of 256 particles takes four to five times the mean tile's
+// time, of which a 1080p frame has 13 per warp: by fours such a chunk was the
+// whole frame's time (1080p infall 307 against 229 us, a wide view 276 against 213,
+// 4K, with 53 tiles per warp, 323 against 280).  With many tiles per warp the
+// counter's round trips are what counts: 64 frames of 1080p (852 per warp) 4072 us
+// by fours, 4124 by twos.  kTail measured at 2 / 4 / 6 / 8 / 16 with chunks of four:
+// 1080p frame 92.2 / 87.0 / 84.4 / 84.8 / 86.0 us, 4K 353 / 350 / 349 / 349 / 352;
+// kFewTail at 3 / 4 / 6 / 8 with chunks of two: 80.0 / 79.8 / 80.0 / 80.1 us, without
+// stars 47.5 / 47.5 / 49.5 / 49.5, the infall with 256 particles 231 / 230 / 232 / 190.
+// Up to two tiles per warp are taken by place: 640 x 360 23.2 -> 18.7 us, without
+// stars 14.6 -> 9.6, all of it in the shadow 14.6 -> 8.6 (counted two at a time 12.6);
+// in an animated disc, where two slow tiles of a warp are the frame's time, one (two:
+// 64 particles 39 -> 47 us).
+constexpr long long kFewTiles = 64, kFewTail = 4, kTail = 6;
+
+static void set_schedule(const bh_ctx *ctx, RenderParams &P, int grid, long long tiles) {
+  const long long warps = (long long)grid * ctx->tuning.warps_per_block;
+  const bool few = tiles <= kFewTiles * warps;
+  P.fetch = ctx->tuning.fetch ? ctx->tuning.fetch : few ? 2 : 4;
+  P.by_place = (unsigned)((P.n_parts ? 1 : 2) * warps);
+  P.tail = (unsigned)((few ? kFewTail : kTail) * warps);
 }
 
 static const void *kernel_ptr(bool half, int mode) {
@@ -1212,6 +1235,7 @@ static bh_status launch(bh_ctx *ctx, const bh_tables *t, RenderParams &P, bool d
                 (P.cams == nullptr && P.cam0.rgb ? sizeof(float) * 96 * ctx->tuning.warps_per_block : 0);
   int grid = render_grid(ctx, P.total_tiles);
   if (grid < 1) return BH_OK;
+  set_schedule(ctx, P, grid, P.total_tiles);
   bool half = t->desc.storage == BH_F16;
   const void *f = kernel_ptr(half, debug ? kDebug : (P.n_parts > 0 ? kAnimated : kPlain));
   void *args[] = {&P};
@@ -1286,6 +1310,7 @@ bh_status render_batch_impl(bh_ctx *ctx, const bh_tables *t, const bh_cubemap *c
   size_t smem = P.u_bytes + 2 * sizeof(float4) * P.n_parts;
   int grid = render_grid(ctx, P.total_tiles);
   if (grid < 1) return BH_OK;
+  set_schedule(ctx, P, grid, P.total_tiles);
   const void *func = kernel_ptr(t->desc.storage == BH_F16, P.n_parts > 0 ? kAnimated : kPlain);
   void *args[] = {&P};
   cudaKernelNodeParams kp = {};
@@ -1509,6 +1534,9 @@ bh_status render_orbit_jobs(bh_ctx *ctx, const bh_tables *t, const bh_cubemap *c
   int threads = 32 * ctx->tuning.warps_per_block;
   size_t smem = P.u_bytes + 2 * sizeof(float4) * P.n_parts;
   int grid = ctx->sm_count * ctx->tuning.blocks_per_sm;
+  long long tiles = 0;
+  for (int k = 0; k < n; ++k) tiles += warp_tiles(jobs_host[k].width, jobs_host[k].height);
+  set_schedule(ctx, P, grid, tiles);
   void *args[] = {&P};
   const void *f = kernel_ptr(t->desc.storage == BH_F16, P.n_parts > 0 ? kAnimated : kPlain);
   BH_CUDA(cudaLaunchKernel(f, dim3(grid), dim3(threads), args, smem, s));
@@ -1873,6 +1901,10 @@ extern "C" bh_status bh_render_orbits(bh_ctx *ctx, const bh_tables *t, const bh_
   int threads = 32 * ctx->tuning.warps_per_block;
   size_t smem = P.u_bytes + 2 * sizeof(float4) * P.n_parts;
   int grid = ctx->sm_count * ctx->tuning.blocks_per_sm;
+  // Only the device knows the sizes: taken as 640 x 360.  Chunks of two cost 16 frames
+  // of 1080p 1.2 %, chunks of four as many of 640 x 360 2 % and, in an animated
+  // disc, one of 1080p a third.
+  set_schedule(ctx, P, grid, (long long)n * warp_tiles(640, 360));
   void *args[] = {&P};
   const void *f = kernel_ptr(t->desc.storage == BH_F16, P.n_parts > 0 ? kAnimated : kPlain);
   BH_CUDA(cudaLaunchKernel(f, dim3(grid), dim3(threads), args, smem, s));

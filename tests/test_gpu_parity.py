@@ -801,6 +801,28 @@ def test_batch_of_thousands_of_cameras_equals_single(ctx, gpu_tables, static_sce
             bh.bh_disc_particles_free(ph)
 
 
+@pytest.mark.parametrize("animated", [False, True])
+@pytest.mark.parametrize("W,H", [(512, 304), (1112, 140), (1024, 304), (1656, 188), (1920, 1080)])
+def test_frame_does_not_depend_on_the_schedule(ctx, gpu_tables, static_scene, W, H, animated):
+    """Frames of 4,864 warp tiles (one per warp of the GPU), one more, twice as
+    many, one more, and many: equal to their part of a batch of over 64 tiles per
+    warp, bit for bit."""
+    cube, _ = static_scene
+    disc, sh, ph = synth.disc(), bh.make_shading(1.0, EXPOSURE_STARS), None
+    if animated:
+        ph = bh.bh_disc_particles_create(ctx, synth.disc_particles(16, 5))
+        disc.update(particles_handle=ph, time=37.5)
+    cams = [synth.camera(6.0, 85.0, v=(0.0, 0.0, 0.5), width=w, height=h) for w, h in ((W, H), (3840, 2160), (1920, 1080))]
+    outs = [torch.zeros((c["height"], c["width"], 4), device="cuda") for c in cams]
+    one = torch.zeros_like(outs[0])
+    bh.bh_render(ctx, gpu_tables, cube, cams[0], disc, sh, one)
+    bh.bh_render_batch(ctx, gpu_tables, cube, cams, disc, sh, outs)
+    torch.cuda.synchronize()
+    if ph:
+        bh.bh_disc_particles_free(ph)
+    assert torch.equal(one, outs[0]) and one[..., 3].min() == 1.0
+
+
 def test_autotune_every_candidate_same_image(gpu_tables, static_scene):
     """The autotuner launches every candidate launch shape; the image does not
     depend on the shape, and batched renders stay equal to single ones."""
