@@ -448,8 +448,10 @@ __device__ void bloom_body(const BloomParams &P) {
       }
     }
     if (!grid_barrier(P, ++phase)) return;
-    blur_upper(P);  // level 1 was blurred by regions
-    if (!grid_barrier(P, ++phase)) return;
+    if (P.n > 1) {  // level 1 was blurred by regions
+      blur_upper(P);
+      if (!grid_barrier(P, ++phase)) return;
+    }
   }
   // ---- composite: a warp takes 32 columns x 8 rows of the frame, neighbouring
   // warps neighbouring columns

@@ -131,3 +131,17 @@ def test_bloom_barrier_timeout_is_reported_and_context_recovers(ctx):
     torch.cuda.synchronize()
     assert bh.bh_check_status(ctx) == bh.BH_OK
     assert compare(out.cpu().numpy(), ob.bloom(img, w)) <= BLOOM_REL
+
+
+@pytest.mark.parametrize("H,W", [(720, 1280), (61, 97), (1, 1)])
+def test_bloom_of_one_level_matches_oracle(ctx, H, W):
+    """One level has no upper blur, and one grid barrier fewer."""
+    img = hdr_frame(H, W, seed=H * 7 + W)
+    w = bh.bh_bloom_weights(math.radians(60), max(H, 2), 1)
+    buf = torch.from_numpy(img).cuda()
+    for _ in range(2):  # in place, the second on the first one's counters
+        bh.bh_bloom(ctx, buf, buf, W, H, w)
+    torch.cuda.synchronize()
+    assert bh.bh_check_status(ctx) == bh.BH_OK
+    once = ob.bloom(img, w)
+    assert compare(buf.cpu().numpy(), ob.bloom(once.astype(np.float32), w)) <= 2 * BLOOM_REL
