@@ -16,7 +16,9 @@
  *    the caller.
  *  - A context keeps up to 512 MiB of the device memory of freed tables, cube
  *    maps and build scratch for the next ones; bh_destroy gives it back, and so
- *    does an allocation of the context that would fail otherwise.
+ *    does an allocation of the context that would fail otherwise.  Freeing a
+ *    handle synchronises the device; while a stream of it is being captured,
+ *    which forbids that, the handle's memory is held until a later free can.
  *  - "device" pointers are CUDA device pointers of the context's device;
  *    "host" pointers are ordinary (preferably pinned) host memory.
  *  - Streams are passed as void* holding a cudaStream_t (NULL = the legacy
@@ -128,8 +130,8 @@ typedef struct {
 } bh_table_desc;
 
 /* Compute D and U on the GPU by FP64 quadrature of the ray equation
- * (Eq. rayequation: (du/dphi)^2 = e^2 - u^2 (1-u)), one thread per texel, and
- * the colour tables: C(xy, D) (64 x 32 x 64, Sec. 3.4.2) and the black-body
+ * (Eq. rayequation: (du/dphi)^2 = e^2 - u^2 (1-u)), one block per e, and the
+ * colour tables: C(xy, D) (64 x 32 x 64, Sec. 3.4.2) and the black-body
  * table used for the disc.  Enqueued on `stream`; *out is usable by later
  * work on the same stream at once.  Allocates device memory (~10 MiB). */
 bh_status bh_precompute_tables(bh_ctx *ctx, const bh_table_desc *desc, void *stream,
@@ -200,9 +202,11 @@ typedef struct {
  * the texel (two unorm8); mips sum colours and average positions weighted by
  * Y.  face_size: power of two, 1..8192.  storage: BH_F16 or BH_BF16.
  * stars: host array (stars_on_device = 0) or device array (1).  Enqueued on
- * `stream` (a host star list is staged synchronously first).  Uses
- * 48 bytes of scratch per star -- where that is more than 1 GiB, at most
- * 240 * face_size^2 bytes --, given back before return. */
+ * `stream` (a host star list is staged synchronously first).  Scratch, given
+ * back before return: 48 bytes per star -- or 240 * face_size^2 bytes, where the
+ * stars take more than that and more than 1 GiB, or more than the device has
+ * left --, 20 more per star of a host list, 58 bytes per region of 32 x 32 texels
+ * (23 MB for faces of 8192) and 32 KB. */
 bh_status bh_build_star_cubemap(bh_ctx *ctx, const bh_star *stars, long long n, int face_size,
                                 bh_dtype storage, int stars_on_device, void *stream,
                                 bh_cubemap **out);

@@ -695,7 +695,8 @@ __global__ void __launch_bounds__(256, BH_RENDER_MIN_BLOCKS) render_kernel(const
           // the lanes moved from row to row together (of 123 occupied texels in a
           // tile's 32 bounding boxes only 15 hold a star with a weight: the rest lie
           // beside thin, slanted footprints; the cull leaves 61).  Every star's weight is rounded in the
-          // same steps as in a walk row by row, and stars are taken in row order.
+          // same steps as in a walk row by row; stars are taken window by window
+          // (in row order up to eight columns) and by rows inside one.
           // 1080p frame 98.5 -> 87.3 us, 4K 435 -> 375 us, 256^2 24.7 -> 17.2 us.
           // Occupancy of the 8 x 8 texels from (wi, wj) on, clipped to the
           // footprint: bit 31 - (8 r + c) of x (rows 0-3) or y (rows 4-7) is
